@@ -5,15 +5,16 @@
 // trained by mean squared error with Adam.  The paper has no network; this
 // is the warm start that shortens the runs to equilibrium.
 //
-// The 256-wide layers run on the fifth-generation tensor cores: BF16
-// operands staged in shared memory in the canonical K-major core-matrix
-// layout, tcgen05.mma issued by one thread, FP32 accumulators in tensor
-// memory (TMEM), read back with tcgen05.ld for a fused epilogue (bias +
-// tanh, bias, tanh' product, or plain store).  One CTA owns a 128-row tile
-// of the output and the full width (N <= 256 columns of TMEM).  The input
-// layer (K = 3) and the reductions run on the CUDA cores in FP32.
-// Parameters: FP32 master copy + BF16 copies of the three tensor-core
-// weight matrices, refreshed by the Adam kernel.
+// Two kernels.  net_kernel takes 128 samples per cluster of eight CTAs
+// through the whole forward pass and, when training, the loss and the
+// backward pass; update_kernel forms the parameter gradients (sums over the
+// batch) and applies Adam.  Their matrix products run on the
+// fifth-generation tensor cores: BF16 operands in shared memory in the
+// canonical core-matrix layouts (K-major, or MN-major where the operand is a
+// transpose), tcgen05.mma issued by one thread, FP32 accumulators in tensor
+// memory (TMEM) read back with tcgen05.ld for the fused epilogues.
+// Parameters: FP32 master copy + BF16 copies of the three tensor-core weight
+// matrices, refreshed by the update.
 #include <math.h>
 #include <string.h>
 
@@ -34,39 +35,23 @@ constexpr int64_t NPARAM = (int64_t)NH * NIN + NH + 2 * ((int64_t)NH * NH + NH) 
 constexpr float BETA1 = 0.9f, BETA2 = 0.999f, ADAM_EPS = 1e-8f;
 
 // ----------------------------------------------------------------- tcgen05
-constexpr int TC_M = 128;        // output rows per CTA (M of one tcgen05.mma)
-constexpr int TC_KC = 64;        // K elements staged per chunk (4 MMAs of K = 16)
-constexpr int TC_THREADS = 128;  // 4 warps: warp w reads TMEM lanes 32w .. 32w + 31
-constexpr int TC_A_BYTES = TC_M * TC_KC * 2;     // 16 KB
-constexpr int TC_B_BYTES = 256 * TC_KC * 2;      // 32 KB (N <= 256)
-// dynamic shared memory: A and B chunks plus the barrier and the TMEM slot,
-// padded so that at most two CTAs share an SM (2 x 256 TMEM columns = all 512)
-constexpr int TC_SMEM = 100 * 1024;
+constexpr int TC_M = 128;            // rows of one tcgen05.mma (samples, or units of a weight gradient)
+constexpr int THREADS = 256;         // warp w reads TMEM lanes 32 (w mod 4) .., columns of half w / 4
+constexpr int CLUSTER = 8;           // CTAs per 128 samples: CTA c owns units 32c .. 32c + 31 of a hidden layer
+constexpr int UNITS = NH / CLUSTER;
+constexpr int OUT_CTAS = 4, OUT_UNITS = NOUT / OUT_CTAS;   // the output layer: 16 units on each of four CTAs
 constexpr long long TC_WAIT_CYCLES = 1000000000LL;   // ~0.5 s: bounded barrier wait
-
-enum Epi { EPI_TANH = 0, EPI_LINEAR = 1, EPI_DTANH = 2, EPI_STORE = 3 };
-
-struct Gemm {
-    // C (M x N) = A (M x K) . B (N x K)^T, FP32 accumulation
-    int M, N, K;
-    const __nv_bfloat16 *A;
-    int64_t sam, sak;            // A(m, k) = A[m * sam + k * sak]
-    const __nv_bfloat16 *B;
-    int64_t sbn, sbk;            // B(n, k) = B[n * sbn + k * sbk]
-    int epi;
-    const float *bias;           // [N]           (EPI_TANH, EPI_LINEAR)
-    const __nv_bfloat16 *h;      // [M x N], ld N (EPI_DTANH: multiply by 1 - h^2)
-    float *of;                   // FP32 output, ld N (EPI_LINEAR, EPI_DTANH, EPI_STORE)
-    __nv_bfloat16 *ob;           // BF16 output, ld N (EPI_TANH, EPI_DTANH)
-    int *err;
-};
 
 __device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-// Shared-memory matrix descriptor (tcgen05), no swizzle, K-major:
-// start address, leading byte offset (between core matrices adjacent in K),
-// stride byte offset (between 8-row groups in M or N), all in 16-byte
-// units; descriptor version 1 at bits 46-47; swizzle mode 0.
+// Shared-memory matrix descriptor (tcgen05), no swizzle: start address,
+// leading byte offset, stride byte offset, all in 16-byte units; descriptor
+// version 1 at bits 46-47.  An operand is staged as 8 x 8 core matrices of
+// 128 contiguous bytes (8 rows of 16 bytes).  K-major: a core matrix holds
+// 8 rows of 8 elements along K; LBO = bytes between core matrices adjacent in
+// K, SBO = between 8-row groups.  MN-major: a core matrix holds 8 values of K
+// with 8 elements along M or N each; SBO = bytes between core matrices
+// adjacent in M or N, LBO = between groups of 8 along K.
 __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint32_t sbo)
 {
     uint64_t d = 0;
@@ -77,36 +62,43 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint3
     return d;
 }
 
-// Instruction descriptor of kind::f16: D in F32, A and B in BF16, both
-// K-major, N >> 3 at bits 17-22, M >> 4 at bits 24-28.
-__device__ __forceinline__ uint32_t instr_desc(int M, int N)
+// Instruction descriptor of kind::f16: D in F32, A and B in BF16, MN-major
+// flags at bits 15 (A) and 16 (B), N >> 3 at bits 17-22, M >> 4 at bits 24-28.
+__device__ __forceinline__ uint32_t instr_desc(int N, bool a_mn, bool b_mn)
 {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)a_mn << 15) | ((uint32_t)b_mn << 16) |
+           ((uint32_t)(N >> 3) << 17) | ((uint32_t)(TC_M >> 4) << 24);
 }
 
-// byte offset of element (r, k) of a staged operand chunk: 8 x 8 core
-// matrices of 128 contiguous bytes (8 rows of 16 bytes), the 8 core matrices
-// along K of one 8-row group contiguous (LBO = 128), row groups 1024 bytes
-// apart (SBO = 1024)
-__device__ __forceinline__ uint32_t core_off(int r, int kg) { return (r >> 3) * 1024 + kg * 128 + (r & 7) * 16; }
-
-__device__ __forceinline__ void stage_operand(uint8_t *dst, const __nv_bfloat16 *src, int rows, int rows_pad,
-                                              int64_t sr, int64_t sk, int k0, int K)
+// a staged operand: shared address, descriptor offsets, bytes per K = 16 step
+struct Operand {
+    uint32_t addr, lbo, sbo, step;
+};
+// K-major, row groups `sbo` apart (8 core matrices of K per 1024 bytes)
+__device__ __forceinline__ Operand k_major(const void *p, uint32_t sbo) { return {smem_addr(p), 128, sbo, 256}; }
+// MN-major with mn elements along M or N
+__device__ __forceinline__ Operand mn_major(const void *p, int mn)
 {
-    // rows_pad x 8 vectors of 8 elements along K
-    for (int v = threadIdx.x; v < rows_pad * (TC_KC / 8); v += TC_THREADS) {
-        const int r = v >> 3, kg = v & 7;
-        uint32_t w[4];
-        for (int e = 0; e < 4; ++e) {
-            const int ka = k0 + kg * 8 + 2 * e, kb = ka + 1;
-            const unsigned short lo =
-                (r < rows && ka < K) ? __bfloat16_as_ushort(src[(int64_t)r * sr + (int64_t)ka * sk]) : 0;
-            const unsigned short hi =
-                (r < rows && kb < K) ? __bfloat16_as_ushort(src[(int64_t)r * sr + (int64_t)kb * sk]) : 0;
-            w[e] = (uint32_t)lo | ((uint32_t)hi << 16);
-        }
-        *reinterpret_cast<uint4 *>(dst + core_off(r, kg)) = make_uint4(w[0], w[1], w[2], w[3]);
+    return {smem_addr(p), (uint32_t)mn * 16, 128, (uint32_t)mn * 32};
+}
+
+// D (+)= A . B over ksteps K = 16 steps; completion arrives on bar
+__device__ __forceinline__ void issue_mma(uint32_t tmem, Operand A, Operand B, int ksteps, uint32_t idesc,
+                                          bool accumulate, uint64_t *bar)
+{
+    for (int s = 0; s < ksteps; ++s) {
+        const uint64_t ad = smem_desc(A.addr + s * A.step, A.lbo, A.sbo);
+        const uint64_t bd = smem_desc(B.addr + s * B.step, B.lbo, B.sbo);
+        const uint32_t acc = (accumulate || s > 0) ? 1u : 0u;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "setp.ne.b32 p, %4, 0;\n\t"
+            "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem),
+            "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
+            : "memory");
     }
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_addr(bar))
+                 : "memory");
 }
 
 __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity)
@@ -128,242 +120,555 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity
     }
 }
 
-__global__ void __launch_bounds__(TC_THREADS) tc_gemm_kernel(Gemm g)
+// 16 / 8 accumulator columns of the thread's row, from column c0
+__device__ __forceinline__ void read_acc16(uint32_t tmem, int c0, float *v)
+{
+    const uint32_t a = tmem + ((threadIdx.x & 96u) << 16) + (uint32_t)c0;
+    uint32_t r[16];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(a)
+        : "memory");
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+    for (int e = 0; e < 16; ++e)
+        v[e] = __uint_as_float(r[e]);
+}
+__device__ __forceinline__ void read_acc8(uint32_t tmem, int c0, float *v)
+{
+    const uint32_t a = tmem + ((threadIdx.x & 96u) << 16) + (uint32_t)c0;
+    uint32_t r[8];
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(a)
+                 : "memory");
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+    for (int e = 0; e < 8; ++e)
+        v[e] = __uint_as_float(r[e]);
+}
+
+// 16 bytes to shared memory asynchronously; zeros when !valid (src is not read)
+__device__ __forceinline__ void cp16(void *dst, const void *src, bool valid)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_addr(dst)), "l"(src), "r"(valid ? 16 : 0)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// `rows` rows of 256 BF16 (row-major) as a K-major operand, row groups 4096
+// bytes apart: eight consecutive lanes write one core matrix (no bank
+// conflicts) and a warp reads 64-byte pieces of eight rows
+__device__ __forceinline__ void stage_k_major(uint8_t *dst, const __nv_bfloat16 *src, int rows)
+{
+    for (int v = threadIdx.x; v < rows * 32; v += THREADS) {
+        const int r = (v >> 8) * 8 + (v & 7), kg = (v >> 3) & 31;
+        cp16(dst + (r >> 3) * 4096 + kg * 128 + (r & 7) * 16, src + (int64_t)r * NH + kg * 8, true);
+    }
+}
+// columns 0 .. mn - 1 of `nk` rows (row length ld) as an MN-major operand:
+// row = index along K; rows at or beyond k_valid and columns at or beyond
+// mn_valid read as zero.  mn: 16, 32 or 128
+__device__ __forceinline__ void stage_mn_major(uint8_t *dst, const __nv_bfloat16 *src, int64_t ld, int nk, int mn,
+                                               int k_valid, int mn_valid)
+{
+    const int vecs = mn >> 3, shift = vecs == 16 ? 4 : (vecs == 4 ? 2 : 1);
+    for (int v = threadIdx.x; v < nk * vecs; v += THREADS) {
+        const int k = (v >> (3 + shift)) * 8 + (v & 7), j = (v >> 3) & (vecs - 1);
+        const bool ok = k < k_valid && j * 8 < mn_valid;
+        cp16(dst + (k >> 3) * mn * 16 + j * 128 + (k & 7) * 16, src + (ok ? k * ld + j * 8 : 0), ok);
+    }
+}
+
+// generic-proxy writes of operands visible to the tensor core of every CTA
+// of the cluster, accumulator reads and writes ordered across the barrier
+__device__ __forceinline__ void cluster_sync()
+{
+    __syncwarp();
+    asm volatile("fence.proxy.async;" ::: "memory");
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    asm volatile("fence.proxy.async;" ::: "memory");
+}
+
+// the thread's row, 8 n consecutive K columns from column k0, into the
+// K-major operand at `buf` of every CTA of the cluster
+__device__ __forceinline__ void broadcast(uint8_t *buf, int k0, const uint4 *v, int n)
+{
+    const int r = threadIdx.x & 127;
+    for (int i = 0; i < n; ++i) {
+        const uint32_t off = smem_addr(buf) + (r >> 3) * 4096 + ((k0 >> 3) + i) * 128 + (r & 7) * 16;
+        for (int c = 0; c < CLUSTER; ++c) {
+            uint32_t dst;
+            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(dst) : "r"(off), "r"(c));
+            asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "r"(v[i].x), "r"(v[i].y),
+                         "r"(v[i].z), "r"(v[i].w)
+                         : "memory");
+        }
+    }
+}
+
+__device__ __forceinline__ uint32_t pack2(float a, float b)
+{
+    return (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(a)) |
+           ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(b)) << 16);
+}
+__device__ __forceinline__ float unpack(uint32_t w, int hi)
+{
+    return __bfloat162float(__ushort_as_bfloat16((unsigned short)(hi ? w >> 16 : w & 0xFFFFu)));
+}
+__device__ __forceinline__ void pack16(const float *v, uint4 *o)
+{
+    for (int i = 0; i < 2; ++i)
+        o[i] = make_uint4(pack2(v[8 * i], v[8 * i + 1]), pack2(v[8 * i + 2], v[8 * i + 3]),
+                          pack2(v[8 * i + 4], v[8 * i + 5]), pack2(v[8 * i + 6], v[8 * i + 7]));
+}
+
+struct Net {
+    int S;
+    const float *x;              // raw inputs (theta_eq deg, R0, lambda); row idx[s] of sample s if idx
+    const float *y;              // labels, same rows (training)
+    const int *idx;
+    const float *p;              // FP32 parameters
+    const __nv_bfloat16 *W1b, *W2b, *W3b;
+    float *yhat;                 // inference: S x 64
+    float *u;                    // training: features S x 3, hidden activations and pre-activation gradients
+    __nv_bfloat16 *h1, *h2, *h3, *d3b, *d2b, *dyb;
+    float *d3, *d2, *d1, *dy, *sq;
+    int *err;
+};
+
+// parameter offsets
+constexpr int64_t OFF_W0 = 0, OFF_B0 = (int64_t)NH * NIN;
+constexpr int64_t OFF_W1 = OFF_B0 + NH, OFF_B1 = OFF_W1 + (int64_t)NH * NH;
+constexpr int64_t OFF_W2 = OFF_B1 + NH, OFF_B2 = OFF_W2 + (int64_t)NH * NH;
+constexpr int64_t OFF_W3 = OFF_B2 + NH, OFF_B3 = OFF_W3 + (int64_t)NOUT * NH;
+
+// shared memory of net_kernel: two activation operands (128 x 256, K-major)
+// and this CTA's slices of the weights
+constexpr int A_BYTES = TC_M * NH * 2, SLICE_BYTES = UNITS * NH * 2;
+constexpr int OFF_SA = 0, OFF_SW1 = 2 * A_BYTES, OFF_SW2 = OFF_SW1 + SLICE_BYTES, OFF_SW3 = OFF_SW2 + SLICE_BYTES;
+constexpr int FWD_SMEM = OFF_SW3 + OUT_UNITS * NH * 2;
+constexpr int OFF_TW3 = FWD_SMEM, OFF_TW2 = OFF_TW3 + NOUT * UNITS * 2, OFF_TW1 = OFF_TW2 + SLICE_BYTES;
+constexpr int TRAIN_SMEM = OFF_TW1 + SLICE_BYTES;
+static_assert(TRAIN_SMEM <= 226 * 1024, "shared memory of one CTA");
+
+// Forward pass (and with TRAIN the loss and the backward pass) of 128
+// samples per cluster.  A layer's product needs every unit of the previous
+// layer, so each CTA writes its 32 units' outputs straight into the operand
+// buffers of all eight CTAs (distributed shared memory) and one cluster
+// barrier separates the layers: seven barriers in place of ten launches with
+// their passes through global memory.  What bounds it is that chain of
+// barriers, products and tanh epilogues (16 per thread), not a throughput:
+// eight CTAs per 128 samples keep each link short.  The weights' slices
+// arrive by asynchronous copies issued at the start, in the order of use.
+// Measured: inference of 200 samples 262 -> 60 us a call (four launches
+// before); an Adam step at batch 128, with its host work, 766 -> 67 us.
+template <bool TRAIN>
+__global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(THREADS) net_kernel(Net g)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
-    uint8_t *sa = smem;
-    uint8_t *sb = smem + TC_A_BYTES;
-    uint64_t *bar = reinterpret_cast<uint64_t *>(smem + TC_A_BYTES + TC_B_BYTES);
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(bar + 1);
-    __shared__ int failed;
-
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int m0 = blockIdx.x * TC_M;
-    const int rows_a = min(TC_M, g.M - m0);
-    const int n_pad = (g.N + 15) & ~15;
-    int ncols = 32;
-    while (ncols < n_pad)
-        ncols <<= 1;
+    __shared__ __align__(8) uint64_t bar;
+    __shared__ uint32_t tslot;
+    uint8_t *sa[2] = {smem + OFF_SA, smem + OFF_SA + A_BYTES};
+    const int cta = blockIdx.x & (CLUSTER - 1), m0 = (blockIdx.x / CLUSTER) * TC_M, n0 = cta * UNITS;
+    const int warp = threadIdx.x >> 5, row = threadIdx.x & 127, half = threadIdx.x >> 7;
+    const int s = m0 + row;
+    const bool live = s < g.S;
 
     if (threadIdx.x == 0) {
-        failed = 0;
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&bar)) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 32;" ::"r"(smem_addr(&tslot))
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    griddep_wait();
+    stage_k_major(smem + OFF_SW1, g.W1b + n0 * NH, UNITS);
+    cp_commit();
+    stage_k_major(smem + OFF_SW2, g.W2b + n0 * NH, UNITS);
+    cp_commit();
+    if (cta < OUT_CTAS)
+        stage_k_major(smem + OFF_SW3, g.W3b + cta * OUT_UNITS * NH, OUT_UNITS);
+    cp_commit();
+    if (TRAIN) {
+        stage_mn_major(smem + OFF_TW3, g.W3b + n0, NH, NOUT, UNITS, NOUT, UNITS);
+        cp_commit();
+        stage_mn_major(smem + OFF_TW2, g.W2b + n0, NH, NH, UNITS, NH, UNITS);
+        cp_commit();
+        stage_mn_major(smem + OFF_TW1, g.W1b + n0, NH, NH, UNITS, NH, UNITS);
+        cp_commit();
+    }
+    cluster_sync();      // every CTA of the cluster runs (its shared memory may be written), TMEM is allocated
+    const uint32_t tmem = tslot;
+    uint32_t parity = 0;
+    bool failed = false;
+    // one product: wait for the staged weights (the cluster barrier before it
+    // ordered everyone's copies), issue, wait for its completion
+    auto product = [&](Operand A, Operand B, int N, int ksteps, bool b_mn) {
+        if (!failed) {
+            if (threadIdx.x == 0)
+                issue_mma(tmem, A, B, ksteps, instr_desc(N, false, b_mn), false, &bar);
+            const bool ok = mbar_wait_bounded(&bar, parity);
+            parity ^= 1u;
+            if (__syncthreads_or(!ok)) {
+                failed = true;
+                if (threadIdx.x == 0)
+                    atomicExch(g.err, 1);
+            }
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        }
+    };
+    const int c0 = n0 + 16 * half;       // the thread's 16 units of a hidden layer
+    uint4 hk1[2], hk2[2], hk3[2];        // its activations, kept for the backward pass
+    float v[16];
+    // the backward pass's dz = dh (1 - h^2)
+    auto dtanh = [&](const uint4 *h) {
+        for (int e = 0; e < 16; ++e) {
+            const float hv = unpack(reinterpret_cast<const uint32_t *>(h)[e >> 1], e & 1);
+            v[e] = v[e] * (1.0f - hv * hv);
+        }
+    };
+    auto store16 = [&](__nv_bfloat16 *o, const uint4 *h) {
+        if (live)
+            for (int i = 0; i < 2; ++i)
+                *reinterpret_cast<uint4 *>(o + (int64_t)s * NH + c0 + 8 * i) = h[i];
+    };
+    auto store16f = [&](float *o) {
+        if (live)
+            for (int i = 0; i < 4; ++i)
+                *reinterpret_cast<float4 *>(o + (int64_t)s * NH + c0 + 4 * i) =
+                    make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+    };
+
+    // features and the input layer (K = 3) on the CUDA cores
+    int src = 0;
+    {
+        float f0 = 0.f, f1 = 0.f, f2 = 0.f;
+        if (live) {
+            src = g.idx ? g.idx[s] : s;
+            f0 = (g.x[3 * src] - 90.0f) / 70.0f;
+            f1 = (g.x[3 * src + 1] - 16.0f) / 8.0f;
+            f2 = log10f(g.x[3 * src + 2]);
+            if (TRAIN && cta == 0 && half == 0) {
+                g.u[3 * s] = f0;
+                g.u[3 * s + 1] = f1;
+                g.u[3 * s + 2] = f2;
+            }
+        }
+        const float *W0 = g.p + OFF_W0, *b0 = g.p + OFF_B0;
+        for (int e = 0; e < 16; ++e) {
+            const int o = c0 + e;
+            const float z = b0[o] + W0[3 * o] * f0 + W0[3 * o + 1] * f1 + W0[3 * o + 2] * f2;
+            v[e] = live ? tanhf(z) : 0.0f;
+        }
+    }
+    pack16(v, hk1);
+    broadcast(sa[0], c0, hk1, 2);
+    if (TRAIN)
+        store16(g.h1, hk1);
+    // hidden layers 2 and 3
+    for (int l = 0; l < 2; ++l) {
+        if (l == 0)
+            cp_wait<TRAIN ? 5 : 2>();
+        else
+            cp_wait<TRAIN ? 4 : 1>();
+        cluster_sync();
+        product(k_major(sa[l], 4096), k_major(smem + (l ? OFF_SW2 : OFF_SW1), 4096), UNITS, NH / 16, false);
+        uint4 *hk = l ? hk3 : hk2;
+        if (!failed)
+            read_acc16(tmem, 16 * half, v);
+        const float *b = g.p + (l ? OFF_B2 : OFF_B1) + c0;
+        for (int e = 0; e < 16; ++e)
+            v[e] = tanhf(v[e] + b[e]);
+        pack16(v, hk);
+        broadcast(sa[l ^ 1], c0, hk, 2);
+        if (TRAIN)
+            store16(l ? g.h3 : g.h2, hk);
+    }
+    // output layer, loss gradient 2 (yhat - y) / (S 64) and squared errors
+    cp_wait<TRAIN ? 3 : 0>();
+    cluster_sync();
+    if (cta < OUT_CTAS) {
+        product(k_major(sa[0], 4096), k_major(smem + OFF_SW3, 4096), OUT_UNITS, NH / 16, false);
+        if (!failed)
+            read_acc8(tmem, 8 * half, v);
+        const int o0 = cta * OUT_UNITS + 8 * half;
+        const float *b = g.p + OFF_B3 + o0;
+        for (int e = 0; e < 8; ++e)
+            v[e] = v[e] + b[e];
+        if (!TRAIN) {
+            if (live)
+                for (int i = 0; i < 2; ++i)
+                    *reinterpret_cast<float4 *>(g.yhat + (int64_t)s * NOUT + o0 + 4 * i) =
+                        make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+        } else {
+            float q[8];
+            for (int e = 0; e < 8; ++e) {
+                const float d = live ? v[e] - g.y[(int64_t)src * NOUT + o0 + e] : 0.0f;
+                v[e] = 2.0f * d / (float)(g.S * NOUT);
+                q[e] = d * d;
+            }
+            const uint4 w = make_uint4(pack2(v[0], v[1]), pack2(v[2], v[3]), pack2(v[4], v[5]), pack2(v[6], v[7]));
+            broadcast(sa[1], o0, &w, 1);
+            if (live) {
+                *reinterpret_cast<uint4 *>(g.dyb + (int64_t)s * NOUT + o0) = w;
+                for (int i = 0; i < 2; ++i) {
+                    *reinterpret_cast<float4 *>(g.dy + (int64_t)s * NOUT + o0 + 4 * i) =
+                        make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+                    *reinterpret_cast<float4 *>(g.sq + (int64_t)s * NOUT + o0 + 4 * i) =
+                        make_float4(q[4 * i], q[4 * i + 1], q[4 * i + 2], q[4 * i + 3]);
+                }
+            }
+        }
+    }
+    if constexpr (TRAIN) {
+        uint4 w[2];
+        // d3 = (dy W3) (1 - h3^2)
+        cp_wait<2>();
+        cluster_sync();
+        product(k_major(sa[1], 4096), mn_major(smem + OFF_TW3, UNITS), UNITS, NOUT / 16, true);
+        if (!failed)
+            read_acc16(tmem, 16 * half, v);
+        dtanh(hk3);
+        pack16(v, w);
+        broadcast(sa[0], c0, w, 2);
+        store16f(g.d3);
+        store16(g.d3b, w);
+        // d2 = (d3 W2) (1 - h2^2)
+        cp_wait<1>();
+        cluster_sync();
+        product(k_major(sa[0], 4096), mn_major(smem + OFF_TW2, UNITS), UNITS, NH / 16, true);
+        if (!failed)
+            read_acc16(tmem, 16 * half, v);
+        dtanh(hk2);
+        pack16(v, w);
+        broadcast(sa[1], c0, w, 2);
+        store16f(g.d2);
+        store16(g.d2b, w);
+        // d1 = (d2 W1) (1 - h1^2)
+        cp_wait<0>();
+        cluster_sync();
+        product(k_major(sa[1], 4096), mn_major(smem + OFF_TW1, UNITS), UNITS, NH / 16, true);
+        if (!failed)
+            read_acc16(tmem, 16 * half, v);
+        dtanh(hk1);
+        store16f(g.d1);
+    }
+    if (failed)   // give MMAs still in flight a bounded chance to finish before TMEM is freed
+        mbar_wait_bounded(&bar, parity ^ 1u);
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (warp == 0) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 32;" ::"r"(tmem) : "memory");
+    }
+}
+
+struct Update {
+    int S;
+    const __nv_bfloat16 *h1, *h2, *h3, *d3b, *d2b, *dyb;
+    const float *d3, *d2, *d1, *dy, *u, *sq;
+    double *loss;
+    float *grad;                 // gradient out (adam false)
+    bool adam;
+    float *p, *m, *v;
+    __nv_bfloat16 *W1b, *W2b, *W3b;
+    float lr, c1, c2;
+    int *err;
+};
+
+// gradient of parameter i: stored, or one Adam step on the FP32 master
+// parameter; returns the new parameter
+__device__ __forceinline__ float apply(const Update &g, int64_t i, float gi)
+{
+    if (!g.adam) {
+        g.grad[i] = gi;
+        return 0.0f;
+    }
+    const float mi = BETA1 * g.m[i] + (1.0f - BETA1) * gi;
+    const float vi = BETA2 * g.v[i] + (1.0f - BETA2) * gi * gi;
+    g.m[i] = mi;
+    g.v[i] = vi;
+    const float pi = g.p[i] - g.lr * (mi / g.c1) / (sqrtf(vi / g.c2) + ADAM_EPS);
+    g.p[i] = pi;
+    return pi;
+}
+
+constexpr int UP_N = 16;                             // columns of a weight gradient per CTA
+constexpr int UP_K = 256;                            // samples staged at a time
+constexpr int UP_A = TC_M * UP_K * 2, UP_B = UP_N * UP_K * 2;
+constexpr int TILES = NH / UP_N;                     // CTAs per 128 rows of a weight gradient
+constexpr int UP_GEMM = 5 * TILES;                   // dW2 (two row tiles), dW1 (two), dW3
+constexpr int UP_RED = (NOUT + 3 * NH) / 32;         // 32 units per CTA: bias gradients (and dW0)
+constexpr int UP_BLOCKS = UP_GEMM + UP_RED + 1;      // and the loss
+
+// Weight gradient tile dW(o, i) = sum_s dz(s, o) h(s, i): both operands are
+// stored sample-major, so they are staged MN-major as they are; the samples
+// run along K in order, UP_K at a time through two buffers.
+__device__ __forceinline__ void weight_grad(const Update &g, uint8_t *smem, uint64_t *bar, uint32_t *tslot)
+{
+    const int t = blockIdx.x / TILES, n0 = (blockIdx.x % TILES) * UP_N;
+    const __nv_bfloat16 *A = t < 2 ? g.d3b : (t < 4 ? g.d2b : g.dyb);
+    const __nv_bfloat16 *B = t < 2 ? g.h2 : (t < 4 ? g.h1 : g.h3);
+    const int64_t off = t < 2 ? OFF_W2 : (t < 4 ? OFF_W1 : OFF_W3);
+    __nv_bfloat16 *Wb = t < 2 ? g.W2b : (t < 4 ? g.W1b : g.W3b);
+    const int m0 = t < 4 ? (t & 1) * TC_M : 0, rows = t < 4 ? TC_M : NOUT, lda = t < 4 ? NH : NOUT;
+    const int warp = threadIdx.x >> 5;
+    if (threadIdx.x == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(bar)) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(tslot)),
-                     "r"(ncols)
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 32;" ::"r"(smem_addr(tslot))
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t tmem = *tslot;
-    const uint32_t idesc = instr_desc(TC_M, n_pad);
-
-    uint32_t phase = 0;
-    for (int k0 = 0; k0 < g.K; k0 += TC_KC) {
-        stage_operand(sa, g.A + (int64_t)m0 * g.sam, rows_a, TC_M, g.sam, g.sak, k0, g.K);
-        stage_operand(sb, g.B, g.N, n_pad, g.sbn, g.sbk, k0, g.K);
-        // generic-proxy writes of the operands become visible to the tensor core
+    griddep_wait();
+    const int chunks = (g.S + UP_K - 1) / UP_K;
+    auto stage = [&](int c) {
+        uint8_t *sa = smem + (c & 1) * (UP_A + UP_B), *sb = sa + UP_A;
+        const int k0 = c * UP_K, kn = min(UP_K, g.S - k0), nk = (kn + 15) & ~15;
+        stage_mn_major(sa, A + (int64_t)k0 * lda + m0, lda, nk, TC_M, kn, rows);
+        stage_mn_major(sb, B + (int64_t)k0 * NH + n0, NH, nk, UP_N, kn, UP_N);
+        cp_commit();
+    };
+    stage(0);
+    uint32_t tmem = 0, parity = 0;
+    bool failed = false;
+    for (int c = 0; c < chunks; ++c) {
+        cp_wait<0>();
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncthreads();
-        if (threadIdx.x == 0) {
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const int ksteps = min(TC_KC, g.K - k0 + 15) / 16;
-            for (int s = 0; s < ksteps && s < TC_KC / 16; ++s) {
-                const uint64_t ad = smem_desc(smem_addr(sa) + s * 256, 128, 1024);
-                const uint64_t bd = smem_desc(smem_addr(sb) + s * 256, 128, 1024);
-                const uint32_t acc = (k0 > 0 || s > 0) ? 1u : 0u;
-                asm volatile(
-                    "{\n\t.reg .pred p;\n\t"
-                    "setp.ne.b32 p, %4, 0;\n\t"
-                    "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem),
-                    "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
-                    : "memory");
-            }
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                             smem_addr(bar))
-                         : "memory");
-        }
-        // every thread waits for the MMAs of this chunk (the operands are
-        // overwritten by the next chunk and TMEM is read after the last)
-        const bool ok = mbar_wait_bounded(bar, phase);
-        phase ^= 1u;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        tmem = *tslot;
+        const uint8_t *sa = smem + (c & 1) * (UP_A + UP_B), *sb = sa + UP_A;
+        if (threadIdx.x == 0)
+            issue_mma(tmem, mn_major(sa, TC_M), mn_major(sb, UP_N), (min(UP_K, g.S - c * UP_K) + 15) / 16,
+                      instr_desc(UP_N, true, true), c > 0, bar);
+        if (c + 1 < chunks)
+            stage(c + 1);        // its buffer's products finished one iteration ago
+        const bool ok = mbar_wait_bounded(bar, parity);
+        parity ^= 1u;
         if (__syncthreads_or(!ok)) {
-            if (threadIdx.x == 0) {
-                failed = 1;
+            failed = true;
+            if (threadIdx.x == 0)
                 atomicExch(g.err, 1);
-            }
             break;
         }
     }
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (failed)   // give MMAs still in flight a bounded chance to finish before TMEM is freed
-        mbar_wait_bounded(bar, phase ^ 1u);
-
-    if (!failed) {
-        const int row = m0 + warp * 32 + lane;
-        for (int c0 = 0; c0 < n_pad; c0 += 16) {
-            uint32_t v[16];
-            const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0;
-            asm volatile(
-                "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, "
-                "[%16];"
-                : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
-                  "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]),
-                  "=r"(v[14]), "=r"(v[15])
-                : "r"(taddr)
-                : "memory");
-            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-            if (row < g.M) {
-                for (int e = 0; e < 16; ++e) {
-                    const int col = c0 + e;
-                    if (col >= g.N)
-                        break;
-                    const float acc = __uint_as_float(v[e]);
-                    const int64_t o = (int64_t)row * g.N + col;
-                    switch (g.epi) {
-                    case EPI_TANH: g.ob[o] = __float2bfloat16_rn(tanhf(acc + g.bias[col])); break;
-                    case EPI_LINEAR: g.of[o] = acc + g.bias[col]; break;
-                    case EPI_DTANH: {
-                        const float h = __bfloat162float(g.h[o]);
-                        const float dz = acc * (1.0f - h * h);
-                        g.of[o] = dz;
-                        g.ob[o] = __float2bfloat16_rn(dz);
-                        break;
-                    }
-                    default: g.of[o] = acc; break;
-                    }
-                }
-            }
+    if (failed) {
+        cp_wait<0>();
+        mbar_wait_bounded(bar, parity ^ 1u);
+    } else {
+        const int row = threadIdx.x & 127, c0 = 8 * (threadIdx.x >> 7);
+        float acc[8];
+        read_acc8(tmem, c0, acc);
+        if (row < rows) {
+            const int64_t o = (int64_t)(m0 + row) * NH + n0 + c0;
+            float pn[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+                pn[e] = apply(g, off + o + e, acc[e]);
+            if (g.adam)
+                *reinterpret_cast<uint4 *>(Wb + o) =
+                    make_uint4(pack2(pn[0], pn[1]), pack2(pn[2], pn[3]), pack2(pn[4], pn[5]), pack2(pn[6], pn[7]));
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (warp == 0) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 32;" ::"r"(tmem) : "memory");
     }
 }
 
-// --------------------------------------------------------- CUDA-core parts
-// features of the raw inputs (theta_eq deg, R0, lambda), then the input layer
-// h1 = tanh(W0 u + b0); one thread per (sample, unit)
-__global__ void input_layer_kernel(const float *xraw, const int *idx, int S, const float *W0, const float *b0,
-                                   float *u, __nv_bfloat16 *h1)
+// Sums over the batch for 32 units: slot l of 32 adds samples l, l + 32, ...
+// in order and the slots meet in a fixed tree.  A warp takes four slots of
+// the 32 units (128-byte reads).  dz: S x ld from the first unit; with u the
+// input layer's weight gradient too.
+__device__ __forceinline__ void unit_sums(const Update &g, const float *dz, int ld, int64_t off_b, int unit0,
+                                          const float *u, float (*sh)[32][33])
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= S * NH)
-        return;
-    const int s = i / NH, o = i - s * NH;
-    const int src = idx ? idx[s] : s;
-    const float f0 = (xraw[3 * src] - 90.0f) / 70.0f;
-    const float f1 = (xraw[3 * src + 1] - 16.0f) / 8.0f;
-    const float f2 = log10f(xraw[3 * src + 2]);
-    if (o == 0) {
-        u[3 * s] = f0;
-        u[3 * s + 1] = f1;
-        u[3 * s + 2] = f2;
+    const int o = threadIdx.x & 31, w = threadIdx.x >> 5, nv = u ? 1 + NIN : 1;
+    for (int q = 0; q < 4; ++q) {
+        const int l = 4 * w + q;
+        float acc[1 + NIN] = {0.f, 0.f, 0.f, 0.f};
+        for (int s = l; s < g.S; s += 32) {
+            const float d = dz[(int64_t)s * ld + unit0 + o];
+            acc[0] += d;
+            if (u)
+                for (int i = 0; i < NIN; ++i)
+                    acc[1 + i] += d * u[3 * s + i];
+        }
+        for (int i = 0; i < nv; ++i)
+            sh[i][l][o] = acc[i];
     }
-    const float z = b0[o] + W0[3 * o] * f0 + W0[3 * o + 1] * f1 + W0[3 * o + 2] * f2;
-    h1[i] = __float2bfloat16_rn(tanhf(z));
+    __syncthreads();
+    if (w < nv) {
+        for (int h = 16; h >= 1; h >>= 1)        // value w of unit o
+            for (int l = 0; l < h; ++l)
+                sh[w][l][o] += sh[w][l + h][o];
+        const int unit = unit0 + o;
+        apply(g, w == 0 ? off_b + unit : OFF_W0 + NIN * unit + (w - 1), sh[w][0][o]);
+    }
 }
 
-// d loss / d output = 2 (yhat - y) / (S * 64), in FP32 and BF16; per-sample
-// squared errors for the loss
-__global__ void loss_grad_kernel(const float *yhat, const float *y, const int *idx, int S, float *dy,
-                                 __nv_bfloat16 *dyb, float *sq)
+// Every parameter's gradient (sums over the batch) and its Adam step, and
+// the loss: CTAs [0, UP_GEMM) one 128 x 16 tile of a weight matrix each on
+// the tensor cores, the next 32 units' biases each (with the input layer's
+// weights), the last the loss.  Small tiles because the time of a CTA is its
+// loads and its divisions: 107 CTAs share both.
+__global__ void __launch_bounds__(THREADS) update_kernel(Update g)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= S * NOUT)
+    extern __shared__ __align__(1024) uint8_t smem[];
+    __shared__ __align__(8) uint64_t bar;
+    __shared__ uint32_t tslot;
+    if (blockIdx.x < UP_GEMM) {
+        weight_grad(g, smem, &bar, &tslot);
         return;
-    const int s = i / NOUT, o = i - s * NOUT;
-    const int src = idx ? idx[s] : s;
-    const float d = yhat[i] - y[(int64_t)src * NOUT + o];
-    const float g = 2.0f * d / (float)(S * NOUT);
-    dy[i] = g;
-    dyb[i] = __float2bfloat16_rn(g);
-    sq[i] = d * d;
-}
-
-// Column sums over the batch in sample order (bias gradients), the input
-// layer's weight gradient dW0 = d1^T u, and the loss (mean of sq); one warp
-// per output, lanes stride over samples, fixed shuffle tree.
-__global__ void reduce_grads_kernel(int S, const float *dy, const float *d3, const float *d2, const float *d1,
-                                    const float *u, const float *sq, float *grad, double *loss)
-{
-    const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    // outputs: gb3 (64), gb2 (256), gb1 (256), gb0 (256), gW0 (768), loss (1)
-    const int nb3 = NOUT, nb = NH, nw0 = NH * NIN;
-    const int total = nb3 + 3 * nb + nw0 + 1;
-    if (w >= total)
-        return;
-    const int64_t off_W0 = 0, off_b0 = (int64_t)NH * NIN;
-    const int64_t off_b1 = off_b0 + NH + (int64_t)NH * NH;
-    const int64_t off_b2 = off_b1 + NH + (int64_t)NH * NH;
-    const int64_t off_b3 = off_b2 + NH + (int64_t)NOUT * NH;
-    float acc = 0.0f;
-    double dacc = 0.0;
-    int64_t dst;
-    if (w < nb3) {
-        for (int s = lane; s < S; s += 32) acc += dy[(int64_t)s * NOUT + w];
-        dst = off_b3 + w;
-    } else if (w < nb3 + nb) {
-        const int o = w - nb3;
-        for (int s = lane; s < S; s += 32) acc += d3[(int64_t)s * NH + o];
-        dst = off_b2 + o;
-    } else if (w < nb3 + 2 * nb) {
-        const int o = w - nb3 - nb;
-        for (int s = lane; s < S; s += 32) acc += d2[(int64_t)s * NH + o];
-        dst = off_b1 + o;
-    } else if (w < nb3 + 3 * nb) {
-        const int o = w - nb3 - 2 * nb;
-        for (int s = lane; s < S; s += 32) acc += d1[(int64_t)s * NH + o];
-        dst = off_b0 + o;
-    } else if (w < nb3 + 3 * nb + nw0) {
-        const int q = w - nb3 - 3 * nb, o = q / NIN, i = q - o * NIN;
-        for (int s = lane; s < S; s += 32) acc += d1[(int64_t)s * NH + o] * u[3 * s + i];
-        dst = off_W0 + q;
-    } else {
-        for (int64_t k = lane; k < (int64_t)S * NOUT; k += 32) dacc += (double)sq[k];
-        dst = -1;
     }
-    for (int o = 16; o >= 1; o >>= 1) {
-        acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        dacc += __shfl_xor_sync(0xffffffffu, dacc, o);
-    }
-    if (lane == 0) {
-        if (dst >= 0)
-            grad[dst] = acc;
+    griddep_wait();
+    const int b = blockIdx.x - UP_GEMM;
+    float(*sh)[32][33] = reinterpret_cast<float(*)[32][33]>(smem);
+    if (b < NOUT / 32) {
+        unit_sums(g, g.dy, NOUT, OFF_B3, 32 * b, nullptr, sh);
+    } else if (b < UP_RED) {
+        const int k = b - NOUT / 32, layer = k / (NH / 32), u0 = 32 * (k % (NH / 32));
+        if (layer == 0)
+            unit_sums(g, g.d3, NH, OFF_B2, u0, nullptr, sh);
+        else if (layer == 1)
+            unit_sums(g, g.d2, NH, OFF_B1, u0, nullptr, sh);
         else
-            *loss = dacc / ((double)S * NOUT);
+            unit_sums(g, g.d1, NH, OFF_B0, u0, g.u, sh);
+    } else {     // loss = mean of the squared errors, FP64, fixed order
+        double *red = reinterpret_cast<double *>(smem);
+        double a[4] = {0.0, 0.0, 0.0, 0.0};
+        const int64_t n = (int64_t)g.S * NOUT;
+        for (int64_t k = 4 * threadIdx.x; k < n; k += 4 * THREADS) {     // n is a multiple of 4
+            const float4 q = *reinterpret_cast<const float4 *>(g.sq + k);
+            a[0] += (double)q.x;
+            a[1] += (double)q.y;
+            a[2] += (double)q.z;
+            a[3] += (double)q.w;
+        }
+        red[threadIdx.x] = (a[0] + a[1]) + (a[2] + a[3]);
+        for (int h = THREADS / 2; h >= 1; h >>= 1) {
+            __syncthreads();
+            if (threadIdx.x < h)
+                red[threadIdx.x] += red[threadIdx.x + h];
+        }
+        if (threadIdx.x == 0)
+            *g.loss = red[0] / ((double)g.S * NOUT);
     }
-}
-
-// Adam step on the FP32 master parameters; refreshes the BF16 copies of the
-// three tensor-core weight matrices
-__global__ void adam_kernel(float *p, const float *g, float *m, float *v, float lr, float c1, float c2,
-                            __nv_bfloat16 *W1b, __nv_bfloat16 *W2b, __nv_bfloat16 *W3b)
-{
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= NPARAM)
-        return;
-    const float gi = g[i];
-    const float mi = BETA1 * m[i] + (1.0f - BETA1) * gi;
-    const float vi = BETA2 * v[i] + (1.0f - BETA2) * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    const float pi = p[i] - lr * (mi / c1) / (sqrtf(vi / c2) + ADAM_EPS);
-    p[i] = pi;
-    const int64_t o1 = (int64_t)NH * NIN + NH, o2 = o1 + (int64_t)NH * NH + NH, o3 = o2 + (int64_t)NH * NH + NH;
-    if (i >= o1 && i < o1 + (int64_t)NH * NH)
-        W1b[i - o1] = __float2bfloat16_rn(pi);
-    else if (i >= o2 && i < o2 + (int64_t)NH * NH)
-        W2b[i - o2] = __float2bfloat16_rn(pi);
-    else if (i >= o3 && i < o3 + (int64_t)NOUT * NH)
-        W3b[i - o3] = __float2bfloat16_rn(pi);
 }
 
 __global__ void to_bf16_kernel(const float *src, __nv_bfloat16 *dst, int64_t n)
@@ -387,8 +692,7 @@ struct iblb_mlp {
     // activations (max_batch rows)
     float *x = nullptr, *y = nullptr, *u = nullptr, *yhat = nullptr, *dy = nullptr, *sq = nullptr;
     float *d3 = nullptr, *d2 = nullptr, *d1 = nullptr;
-    __nv_bfloat16 *h1 = nullptr, *h2 = nullptr, *h3 = nullptr, *dyb = nullptr, *d3b = nullptr, *d2b = nullptr,
-                  *d1b = nullptr;
+    __nv_bfloat16 *h1 = nullptr, *h2 = nullptr, *h3 = nullptr, *dyb = nullptr, *d3b = nullptr, *d2b = nullptr;
     int *err = nullptr, *idx = nullptr;
     double *loss = nullptr;              // loss of each batch of an epoch (loss_cap entries)
     int loss_cap = 0;
@@ -416,64 +720,38 @@ int mfail(iblb_mlp *m, int code, const std::string &s)
             return mfail(m, IBLB_E_CUDA, std::string(#call) + ": " + cudaGetErrorString(e_));  \
     } while (0)
 
-// parameter offsets
-constexpr int64_t OFF_W0 = 0, OFF_B0 = (int64_t)NH * NIN;
-constexpr int64_t OFF_W1 = OFF_B0 + NH, OFF_B1 = OFF_W1 + (int64_t)NH * NH;
-constexpr int64_t OFF_W2 = OFF_B1 + NH, OFF_B2 = OFF_W2 + (int64_t)NH * NH;
-constexpr int64_t OFF_W3 = OFF_B2 + NH, OFF_B3 = OFF_W3 + (int64_t)NOUT * NH;
-
-cudaError_t gemm(iblb_mlp *mm, int M, int N, int K, const __nv_bfloat16 *A, int64_t sam, int64_t sak,
-                 const __nv_bfloat16 *B, int64_t sbn, int64_t sbk, int epi, const float *bias,
-                 const __nv_bfloat16 *h, float *of, __nv_bfloat16 *ob)
+// forward pass of S rows of x (device, raw inputs): outputs into mm->yhat
+cudaError_t forward(iblb_mlp *mm, const float *x, int S)
 {
-    Gemm g{M, N, K, A, sam, sak, B, sbn, sbk, epi, bias, h, of, ob, mm->err};
-    tc_gemm_kernel<<<nblk(M, TC_M), TC_THREADS, TC_SMEM, mm->stream>>>(g);
-    return cudaGetLastError();
+    Net g{};
+    g.S = S;
+    g.x = x;
+    g.p = mm->p;
+    g.W1b = mm->W1b;
+    g.W2b = mm->W2b;
+    g.W3b = mm->W3b;
+    g.yhat = mm->yhat;
+    g.err = mm->err;
+    return launch_k(net_kernel<false>, dim3(nblk(S, TC_M) * CLUSTER), dim3(THREADS), FWD_SMEM, mm->stream, true, g);
 }
 
-// forward pass of S rows of x (device, raw inputs; rows idx[s] if idx)
-cudaError_t forward(iblb_mlp *mm, const float *x, const int *idx, int S)
+// Forward and backward pass of S samples (rows idx[s] of x and y if idx) and
+// the mean squared error into *loss; then the gradient into mm->g, or with
+// lr > 0 one Adam step with the bias corrections c1 and c2.
+cudaError_t train_step(iblb_mlp *mm, const float *x, const float *y, const int *idx, int S, double *loss, float lr,
+                       float c1, float c2)
 {
-    input_layer_kernel<<<nblk((int64_t)S * NH, 256), 256, 0, mm->stream>>>(x, idx, S, mm->p + OFF_W0,
-                                                                          mm->p + OFF_B0, mm->u, mm->h1);
-    cudaError_t e;
-    if ((e = gemm(mm, S, NH, NH, mm->h1, NH, 1, mm->W1b, NH, 1, EPI_TANH, mm->p + OFF_B1, nullptr, nullptr, mm->h2)))
+    const Net n{S, x, y, idx, mm->p, mm->W1b, mm->W2b, mm->W3b, nullptr, mm->u, mm->h1, mm->h2, mm->h3, mm->d3b,
+                mm->d2b, mm->dyb, mm->d3, mm->d2, mm->d1, mm->dy, mm->sq, mm->err};
+    cudaError_t e = launch_k(net_kernel<true>, dim3(nblk(S, TC_M) * CLUSTER), dim3(THREADS), TRAIN_SMEM, mm->stream,
+                             true, n);
+    if (e != cudaSuccess)
         return e;
-    if ((e = gemm(mm, S, NH, NH, mm->h2, NH, 1, mm->W2b, NH, 1, EPI_TANH, mm->p + OFF_B2, nullptr, nullptr, mm->h3)))
-        return e;
-    return gemm(mm, S, NOUT, NH, mm->h3, NH, 1, mm->W3b, NH, 1, EPI_LINEAR, mm->p + OFF_B3, nullptr, mm->yhat,
-                nullptr);
-}
-
-// forward + backward: gradient of the mean squared error into mm->g, loss
-// into mm->loss
-cudaError_t forward_backward(iblb_mlp *mm, const float *x, const float *y, const int *idx, int S, double *loss)
-{
-    cudaError_t e;
-    if ((e = forward(mm, x, idx, S)))
-        return e;
-    loss_grad_kernel<<<nblk((int64_t)S * NOUT, 256), 256, 0, mm->stream>>>(mm->yhat, y, idx, S, mm->dy, mm->dyb,
-                                                                           mm->sq);
-    float *g = mm->g;
-    // layer 3: gW3 = dy^T h3 (64 x 256, K = S); d3 = (dy W3) * (1 - h3^2)
-    if ((e = gemm(mm, NOUT, NH, S, mm->dyb, 1, NOUT, mm->h3, 1, NH, EPI_STORE, nullptr, nullptr, g + OFF_W3, nullptr)))
-        return e;
-    if ((e = gemm(mm, S, NH, NOUT, mm->dyb, NOUT, 1, mm->W3b, 1, NH, EPI_DTANH, nullptr, mm->h3, mm->d3, mm->d3b)))
-        return e;
-    // layer 2
-    if ((e = gemm(mm, NH, NH, S, mm->d3b, 1, NH, mm->h2, 1, NH, EPI_STORE, nullptr, nullptr, g + OFF_W2, nullptr)))
-        return e;
-    if ((e = gemm(mm, S, NH, NH, mm->d3b, NH, 1, mm->W2b, 1, NH, EPI_DTANH, nullptr, mm->h2, mm->d2, mm->d2b)))
-        return e;
-    // layer 1
-    if ((e = gemm(mm, NH, NH, S, mm->d2b, 1, NH, mm->h1, 1, NH, EPI_STORE, nullptr, nullptr, g + OFF_W1, nullptr)))
-        return e;
-    if ((e = gemm(mm, S, NH, NH, mm->d2b, NH, 1, mm->W1b, 1, NH, EPI_DTANH, nullptr, mm->h1, mm->d1, mm->d1b)))
-        return e;
-    const int nwarps = NOUT + 3 * NH + NH * NIN + 1;
-    reduce_grads_kernel<<<nblk((int64_t)nwarps * 32, 256), 256, 0, mm->stream>>>(S, mm->dy, mm->d3, mm->d2, mm->d1,
-                                                                                 mm->u, mm->sq, g, loss);
-    return cudaGetLastError();
+    const Update u{S, mm->h1, mm->h2, mm->h3, mm->d3b, mm->d2b, mm->dyb, mm->d3, mm->d2, mm->d1, mm->dy, mm->u,
+                   mm->sq, loss, mm->g, lr > 0.0f, mm->p, mm->m, mm->v, mm->W1b, mm->W2b, mm->W3b, lr, c1, c2,
+                   mm->err};
+    return launch_k(update_kernel, dim3(UP_BLOCKS), dim3(THREADS), (S > UP_K ? 2 : 1) * (UP_A + UP_B), mm->stream,
+                    true, u);
 }
 
 cudaError_t refresh_bf16(iblb_mlp *mm)
@@ -589,12 +867,13 @@ int iblb_mlp_create(const float *params, int64_t n_params, int max_batch, void *
     if (!e) e = bf(&m->dyb, NOUT * B);
     if (!e) e = bf(&m->d3b, NH * B);
     if (!e) e = bf(&m->d2b, NH * B);
-    if (!e) e = bf(&m->d1b, NH * B);
     if (!e) e = cudaMalloc((void **)&m->err, sizeof(int));
     if (!e) e = cudaMalloc((void **)&m->idx, sizeof(int) * B);
     if (!e) e = cudaMalloc((void **)&m->loss, sizeof(double));
     if (!e) m->loss_cap = 1;
-    if (!e) e = cudaFuncSetAttribute(tc_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM);
+    if (!e) e = cudaFuncSetAttribute(net_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, FWD_SMEM);
+    if (!e) e = cudaFuncSetAttribute(net_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, TRAIN_SMEM);
+    if (!e) e = cudaFuncSetAttribute(update_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * (UP_A + UP_B));
     if (!e) e = cudaMemcpyAsync(m->p, params, sizeof(float) * NPARAM, cudaMemcpyHostToDevice, m->stream);
     if (!e) e = cudaMemsetAsync(m->m, 0, sizeof(float) * NPARAM, m->stream);
     if (!e) e = cudaMemsetAsync(m->v, 0, sizeof(float) * NPARAM, m->stream);
@@ -615,7 +894,7 @@ void iblb_mlp_destroy(iblb_mlp *m)
     if (!m)
         return;
     void *ptrs[] = {m->p, m->g, m->m, m->v, m->W1b, m->W2b, m->W3b, m->x, m->y, m->u, m->yhat, m->dy, m->sq,
-                    m->d3, m->d2, m->d1, m->h1, m->h2, m->h3, m->dyb, m->d3b, m->d2b, m->d1b, m->err, m->idx,
+                    m->d3, m->d2, m->d1, m->h1, m->h2, m->h3, m->dyb, m->d3b, m->d2b, m->err, m->idx,
                     m->loss};
     for (void *p : ptrs)
         if (p)
@@ -644,7 +923,7 @@ int iblb_mlp_predict(iblb_mlp *m, const double *x, int S, double *y)
     std::vector<float> hy((size_t)NOUT * m->max_batch);
     for (int s0 = 0; s0 < S; s0 += m->max_batch) {
         const int n = std::min(m->max_batch, S - s0);
-        MCK(forward(m, m->x + 3 * (int64_t)s0, nullptr, n));
+        MCK(forward(m, m->x + 3 * (int64_t)s0, n));
         MCK(cudaMemcpyAsync(hy.data(), m->yhat, sizeof(float) * NOUT * n, cudaMemcpyDeviceToHost, m->stream));
         MCK(cudaStreamSynchronize(m->stream));
         if ((r = check_err(m)))
@@ -664,7 +943,7 @@ int iblb_mlp_grad(iblb_mlp *m, const double *x, const double *y, int S, double *
     int r = upload(m, x, y, S);
     if (r)
         return r;
-    MCK(forward_backward(m, m->x, m->y, nullptr, S, m->loss));
+    MCK(train_step(m, m->x, m->y, nullptr, S, m->loss, 0.0f, 1.0f, 1.0f));
     std::vector<float> hg(NPARAM);
     MCK(cudaMemcpyAsync(hg.data(), m->g, sizeof(float) * NPARAM, cudaMemcpyDeviceToHost, m->stream));
     MCK(cudaMemcpyAsync(loss, m->loss, sizeof(double), cudaMemcpyDeviceToHost, m->stream));
@@ -708,12 +987,9 @@ int iblb_mlp_train(iblb_mlp *m, const double *x, const double *y, int S, int epo
         for (int b = 0; b < nb; ++b) {
             MCK(cudaMemcpyAsync(m->idx, perm.data() + (int64_t)b * batch, sizeof(int) * batch,
                                 cudaMemcpyHostToDevice, m->stream));
-            MCK(forward_backward(m, m->x, m->y, m->idx, batch, m->loss + b));
             m->t++;
             const float c1 = 1.0f - powf(BETA1, (float)m->t), c2 = 1.0f - powf(BETA2, (float)m->t);
-            adam_kernel<<<nblk(NPARAM, 256), 256, 0, m->stream>>>(m->p, m->g, m->m, m->v, (float)lr, c1, c2, m->W1b,
-                                                                  m->W2b, m->W3b);
-            MCK(cudaGetLastError());
+            MCK(train_step(m, m->x, m->y, m->idx, batch, m->loss + b, (float)lr, c1, c2));
         }
         if (nb)
             MCK(cudaMemcpyAsync(losses.data(), m->loss, sizeof(double) * nb, cudaMemcpyDeviceToHost, m->stream));
