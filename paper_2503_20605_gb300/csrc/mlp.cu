@@ -20,7 +20,9 @@
 
 #include <cmath>
 
+#include <algorithm>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/iblb.h"
@@ -36,7 +38,8 @@ constexpr float BETA1 = 0.9f, BETA2 = 0.999f, ADAM_EPS = 1e-8f;
 
 // ----------------------------------------------------------------- tcgen05
 constexpr int TC_M = 128;            // rows of one tcgen05.mma (samples, or units of a weight gradient)
-constexpr int THREADS = 256;         // warp w reads TMEM lanes 32 (w mod 4) .., columns of half w / 4
+constexpr int THREADS = 256;         // update kernel: warp w reads TMEM lanes 32 (w mod 4) .., columns of half w / 4
+constexpr int NET_THREADS = 512;     // forward / backward kernel: columns of quarter w / 4
 constexpr int CLUSTER = 8;           // CTAs per 128 samples: CTA c owns units 32c .. 32c + 31 of a hidden layer
 constexpr int UNITS = NH / CLUSTER;
 constexpr int OUT_CTAS = 4, OUT_UNITS = NOUT / OUT_CTAS;   // the output layer: 16 units on each of four CTAs
@@ -120,31 +123,33 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity
     }
 }
 
-// 16 / 8 accumulator columns of the thread's row, from column c0
-__device__ __forceinline__ void read_acc16(uint32_t tmem, int c0, float *v)
-{
-    const uint32_t a = tmem + ((threadIdx.x & 96u) << 16) + (uint32_t)c0;
-    uint32_t r[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(a)
-        : "memory");
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-    for (int e = 0; e < 16; ++e)
-        v[e] = __uint_as_float(r[e]);
-}
-__device__ __forceinline__ void read_acc8(uint32_t tmem, int c0, float *v)
+// 8 / 4 accumulator columns of the thread's row, from column c0
+__device__ __forceinline__ void read_acc(uint32_t tmem, int c0, float (&v)[8])
 {
     const uint32_t a = tmem + ((threadIdx.x & 96u) << 16) + (uint32_t)c0;
     uint32_t r[8];
+    __syncwarp();
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
                  : "r"(a)
                  : "memory");
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
     for (int e = 0; e < 8; ++e)
+        v[e] = __uint_as_float(r[e]);
+}
+__device__ __forceinline__ void read_acc(uint32_t tmem, int c0, float (&v)[4])
+{
+    const uint32_t a = tmem + ((threadIdx.x & 96u) << 16) + (uint32_t)c0;
+    uint32_t r[4];
+    __syncwarp();
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(a)
+                 : "memory");
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
         v[e] = __uint_as_float(r[e]);
 }
 
@@ -163,7 +168,7 @@ __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0
 // conflicts) and a warp reads 64-byte pieces of eight rows
 __device__ __forceinline__ void stage_k_major(uint8_t *dst, const __nv_bfloat16 *src, int rows)
 {
-    for (int v = threadIdx.x; v < rows * 32; v += THREADS) {
+    for (int v = threadIdx.x; v < rows * 32; v += NET_THREADS) {
         const int r = (v >> 8) * 8 + (v & 7), kg = (v >> 3) & 31;
         cp16(dst + (r >> 3) * 4096 + kg * 128 + (r & 7) * 16, src + (int64_t)r * NH + kg * 8, true);
     }
@@ -171,45 +176,66 @@ __device__ __forceinline__ void stage_k_major(uint8_t *dst, const __nv_bfloat16 
 // columns 0 .. mn - 1 of `nk` rows (row length ld) as an MN-major operand:
 // row = index along K; rows at or beyond k_valid and columns at or beyond
 // mn_valid read as zero.  mn: 16, 32 or 128
+template <int NT>
 __device__ __forceinline__ void stage_mn_major(uint8_t *dst, const __nv_bfloat16 *src, int64_t ld, int nk, int mn,
                                                int k_valid, int mn_valid)
 {
     const int vecs = mn >> 3, shift = vecs == 16 ? 4 : (vecs == 4 ? 2 : 1);
-    for (int v = threadIdx.x; v < nk * vecs; v += THREADS) {
+    for (int v = threadIdx.x; v < nk * vecs; v += NT) {
         const int k = (v >> (3 + shift)) * 8 + (v & 7), j = (v >> 3) & (vecs - 1);
         const bool ok = k < k_valid && j * 8 < mn_valid;
         cp16(dst + (k >> 3) * mn * 16 + j * 128 + (k & 7) * 16, src + (ok ? k * ld + j * 8 : 0), ok);
     }
 }
 
-// generic-proxy writes of operands visible to the tensor core of every CTA
-// of the cluster, accumulator reads and writes ordered across the barrier
-__device__ __forceinline__ void cluster_sync()
+// The cluster barrier between two layers: operand writes to shared memory
+// (any CTA's) are visible to the tensor cores after it, accumulator reads and
+// writes are ordered across it.  In two halves, so that a thread's global
+// stores go out between them: before the arrival its release would wait for
+// them.
+__device__ __forceinline__ void cluster_arrive()
 {
     __syncwarp();
-    asm volatile("fence.proxy.async;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cluster;" ::: "memory");
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait()
+{
+    __syncwarp();
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    asm volatile("fence.proxy.async;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cluster;" ::: "memory");
 }
 
-// the thread's row, 8 n consecutive K columns from column k0, into the
+// the thread's row, K columns from k0 (8 in a uint4, 4 in a uint2), into the
 // K-major operand at `buf` of every CTA of the cluster
-__device__ __forceinline__ void broadcast(uint8_t *buf, int k0, const uint4 *v, int n)
+__device__ __forceinline__ uint32_t operand_at(uint8_t *buf, int k0)
 {
     const int r = threadIdx.x & 127;
-    for (int i = 0; i < n; ++i) {
-        const uint32_t off = smem_addr(buf) + (r >> 3) * 4096 + ((k0 >> 3) + i) * 128 + (r & 7) * 16;
-        for (int c = 0; c < CLUSTER; ++c) {
-            uint32_t dst;
-            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(dst) : "r"(off), "r"(c));
-            asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "r"(v[i].x), "r"(v[i].y),
-                         "r"(v[i].z), "r"(v[i].w)
-                         : "memory");
-        }
-    }
+    return smem_addr(buf) + (r >> 3) * 4096 + (k0 >> 3) * 128 + (r & 7) * 16 + (k0 & 7) * 2;
+}
+__device__ __forceinline__ uint32_t in_cta(uint32_t addr, int c)
+{
+    uint32_t dst;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(dst) : "r"(addr), "r"(c));
+    return dst;
+}
+__device__ __forceinline__ void broadcast(uint8_t *buf, int k0, uint4 v)
+{
+    const uint32_t at = operand_at(buf, k0);
+#pragma unroll
+    for (int c = 0; c < CLUSTER; ++c)
+        asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(in_cta(at, c)), "r"(v.x), "r"(v.y),
+                     "r"(v.z), "r"(v.w)
+                     : "memory");
+}
+__device__ __forceinline__ void broadcast(uint8_t *buf, int k0, uint2 v)
+{
+    const uint32_t at = operand_at(buf, k0);
+#pragma unroll
+    for (int c = 0; c < CLUSTER; ++c)
+        asm volatile("st.shared::cluster.v2.b32 [%0], {%1, %2};" ::"r"(in_cta(at, c)), "r"(v.x), "r"(v.y) : "memory");
 }
 
 __device__ __forceinline__ uint32_t pack2(float a, float b)
@@ -221,11 +247,29 @@ __device__ __forceinline__ float unpack(uint32_t w, int hi)
 {
     return __bfloat162float(__ushort_as_bfloat16((unsigned short)(hi ? w >> 16 : w & 0xFFFFu)));
 }
-__device__ __forceinline__ void pack16(const float *v, uint4 *o)
+__device__ __forceinline__ uint4 pack8(const float (&v)[8])
 {
-    for (int i = 0; i < 2; ++i)
-        o[i] = make_uint4(pack2(v[8 * i], v[8 * i + 1]), pack2(v[8 * i + 2], v[8 * i + 3]),
-                          pack2(v[8 * i + 4], v[8 * i + 5]), pack2(v[8 * i + 6], v[8 * i + 7]));
+    return make_uint4(pack2(v[0], v[1]), pack2(v[2], v[3]), pack2(v[4], v[5]), pack2(v[6], v[7]));
+}
+// n (a multiple of 4) floats at p, 16-byte aligned
+template <int N>
+__device__ __forceinline__ void load_floats(const float *p, float (&v)[N])
+{
+#pragma unroll
+    for (int i = 0; i < N; i += 4) {
+        const float4 q = *reinterpret_cast<const float4 *>(p + i);
+        v[i] = q.x;
+        v[i + 1] = q.y;
+        v[i + 2] = q.z;
+        v[i + 3] = q.w;
+    }
+}
+template <int N>
+__device__ __forceinline__ void store_floats(float *p, const float (&v)[N])
+{
+#pragma unroll
+    for (int i = 0; i < N; i += 4)
+        *reinterpret_cast<float4 *>(p + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
 }
 
 struct Net {
@@ -263,22 +307,28 @@ static_assert(TRAIN_SMEM <= 226 * 1024, "shared memory of one CTA");
 // buffers of all eight CTAs (distributed shared memory) and one cluster
 // barrier separates the layers: seven barriers in place of ten launches with
 // their passes through global memory.  What bounds it is that chain of
-// barriers, products and tanh epilogues (16 per thread), not a throughput:
-// eight CTAs per 128 samples keep each link short.  The weights' slices
-// arrive by asynchronous copies issued at the start, in the order of use.
-// Measured: inference of 200 samples 262 -> 60 us a call (four launches
-// before); an Adam step at batch 128, with its host work, 766 -> 67 us.
+// barriers, products and tanh epilogues (8 per thread), not a throughput:
+// eight CTAs of 512 threads per 128 samples keep each link short, and
+// everything a thread reads from global memory (weights' slices by
+// asynchronous copies in the order of use, biases, labels) is requested
+// before the first barrier.
+// Measured: inference of 200 samples 262 -> 37 us a call (four launches and
+// three copies before); 27 us of a training step at batch 128, about 2.3 us a
+// layer of which 0.6 are the product, 0.7 the barrier and the rest the
+// epilogue and its 64 KB of stores into the other CTAs.
 template <bool TRAIN>
-__global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(THREADS) net_kernel(Net g)
+__global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(NET_THREADS, 1) net_kernel(Net g)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
     __shared__ __align__(8) uint64_t bar;
     __shared__ uint32_t tslot;
     uint8_t *sa[2] = {smem + OFF_SA, smem + OFF_SA + A_BYTES};
     const int cta = blockIdx.x & (CLUSTER - 1), m0 = (blockIdx.x / CLUSTER) * TC_M, n0 = cta * UNITS;
-    const int warp = threadIdx.x >> 5, row = threadIdx.x & 127, half = threadIdx.x >> 7;
+    const int warp = threadIdx.x >> 5, row = threadIdx.x & 127, quarter = threadIdx.x >> 7;
     const int s = m0 + row;
     const bool live = s < g.S;
+    const int c0 = n0 + 8 * quarter;                        // the thread's 8 units of a hidden layer
+    const int o0 = (cta & (OUT_CTAS - 1)) * OUT_UNITS + 4 * quarter;   // its 4 outputs (CTAs below OUT_CTAS)
 
     if (threadIdx.x == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&bar)) : "memory");
@@ -289,7 +339,17 @@ __global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(THREADS) net_k
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    cluster_arrive();    // waited for before the first write to another CTA
     griddep_wait();
+    float w0[24], b0[8], b1[8], b2[8], b3[4], f[3] = {0.f, 0.f, 0.f}, yl[4] = {0.f, 0.f, 0.f, 0.f};
+    int src = 0;
+    if (live)
+        src = g.idx ? g.idx[s] : s;
+    load_floats(g.p + OFF_W0 + NIN * c0, w0);
+    load_floats(g.p + OFF_B0 + c0, b0);
+    load_floats(g.p + OFF_B1 + c0, b1);
+    load_floats(g.p + OFF_B2 + c0, b2);
+    load_floats(g.p + OFF_B3 + o0, b3);
     stage_k_major(smem + OFF_SW1, g.W1b + n0 * NH, UNITS);
     cp_commit();
     stage_k_major(smem + OFF_SW2, g.W2b + n0 * NH, UNITS);
@@ -298,19 +358,25 @@ __global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(THREADS) net_k
         stage_k_major(smem + OFF_SW3, g.W3b + cta * OUT_UNITS * NH, OUT_UNITS);
     cp_commit();
     if (TRAIN) {
-        stage_mn_major(smem + OFF_TW3, g.W3b + n0, NH, NOUT, UNITS, NOUT, UNITS);
+        stage_mn_major<NET_THREADS>(smem + OFF_TW3, g.W3b + n0, NH, NOUT, UNITS, NOUT, UNITS);
         cp_commit();
-        stage_mn_major(smem + OFF_TW2, g.W2b + n0, NH, NH, UNITS, NH, UNITS);
+        stage_mn_major<NET_THREADS>(smem + OFF_TW2, g.W2b + n0, NH, NH, UNITS, NH, UNITS);
         cp_commit();
-        stage_mn_major(smem + OFF_TW1, g.W1b + n0, NH, NH, UNITS, NH, UNITS);
+        stage_mn_major<NET_THREADS>(smem + OFF_TW1, g.W1b + n0, NH, NH, UNITS, NH, UNITS);
         cp_commit();
     }
-    cluster_sync();      // every CTA of the cluster runs (its shared memory may be written), TMEM is allocated
-    const uint32_t tmem = tslot;
+    if (live) {
+        f[0] = g.x[3 * src];
+        f[1] = g.x[3 * src + 1];
+        f[2] = g.x[3 * src + 2];
+        if (TRAIN)
+            load_floats(g.y + (int64_t)src * NOUT + o0, yl);
+    }
     uint32_t parity = 0;
     bool failed = false;
-    // one product: wait for the staged weights (the cluster barrier before it
-    // ordered everyone's copies), issue, wait for its completion
+    uint32_t tmem = 0;
+    // one product (the cluster barrier before it ordered everyone's operand
+    // writes): issue, wait for its completion
     auto product = [&](Operand A, Operand B, int N, int ksteps, bool b_mn) {
         if (!failed) {
             if (threadIdx.x == 0)
@@ -325,141 +391,141 @@ __global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(THREADS) net_k
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         }
     };
-    const int c0 = n0 + 16 * half;       // the thread's 16 units of a hidden layer
-    uint4 hk1[2], hk2[2], hk3[2];        // its activations, kept for the backward pass
-    float v[16];
+    uint4 hk1, hk2, hk3, w;              // its activations, kept for the backward pass
+    float v[8] = {};
     // the backward pass's dz = dh (1 - h^2)
-    auto dtanh = [&](const uint4 *h) {
-        for (int e = 0; e < 16; ++e) {
-            const float hv = unpack(reinterpret_cast<const uint32_t *>(h)[e >> 1], e & 1);
+    auto dtanh = [&](uint4 h) {
+        const uint32_t q[4] = {h.x, h.y, h.z, h.w};
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const float hv = unpack(q[e >> 1], e & 1);
             v[e] = v[e] * (1.0f - hv * hv);
         }
     };
-    auto store16 = [&](__nv_bfloat16 *o, const uint4 *h) {
+    auto store = [&](__nv_bfloat16 *o, uint4 h) {
         if (live)
-            for (int i = 0; i < 2; ++i)
-                *reinterpret_cast<uint4 *>(o + (int64_t)s * NH + c0 + 8 * i) = h[i];
+            *reinterpret_cast<uint4 *>(o + (int64_t)s * NH + c0) = h;
     };
-    auto store16f = [&](float *o) {
+    auto store_f = [&](float *o) {
         if (live)
-            for (int i = 0; i < 4; ++i)
-                *reinterpret_cast<float4 *>(o + (int64_t)s * NH + c0 + 4 * i) =
-                    make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+            store_floats(o + (int64_t)s * NH + c0, v);
     };
 
     // features and the input layer (K = 3) on the CUDA cores
-    int src = 0;
-    {
-        float f0 = 0.f, f1 = 0.f, f2 = 0.f;
-        if (live) {
-            src = g.idx ? g.idx[s] : s;
-            f0 = (g.x[3 * src] - 90.0f) / 70.0f;
-            f1 = (g.x[3 * src + 1] - 16.0f) / 8.0f;
-            f2 = log10f(g.x[3 * src + 2]);
-            if (TRAIN && cta == 0 && half == 0) {
-                g.u[3 * s] = f0;
-                g.u[3 * s + 1] = f1;
-                g.u[3 * s + 2] = f2;
-            }
-        }
-        const float *W0 = g.p + OFF_W0, *b0 = g.p + OFF_B0;
-        for (int e = 0; e < 16; ++e) {
-            const int o = c0 + e;
-            const float z = b0[o] + W0[3 * o] * f0 + W0[3 * o + 1] * f1 + W0[3 * o + 2] * f2;
-            v[e] = live ? tanhf(z) : 0.0f;
+    if (live) {
+        f[0] = (f[0] - 90.0f) / 70.0f;
+        f[1] = (f[1] - 16.0f) / 8.0f;
+        f[2] = log10f(f[2]);
+        if (TRAIN && cta == 0 && quarter == 0) {
+            g.u[3 * s] = f[0];
+            g.u[3 * s + 1] = f[1];
+            g.u[3 * s + 2] = f[2];
         }
     }
-    pack16(v, hk1);
-    broadcast(sa[0], c0, hk1, 2);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+        const float z = b0[e] + w0[3 * e] * f[0] + w0[3 * e + 1] * f[1] + w0[3 * e + 2] * f[2];
+        v[e] = live ? tanhf(z) : 0.0f;
+    }
+    hk1 = pack8(v);
+    cluster_wait();      // every CTA of the cluster runs: its shared memory may be written; TMEM is allocated
+    tmem = tslot;
+    broadcast(sa[0], c0, hk1);
+    cp_wait<TRAIN ? 5 : 2>();
+    cluster_arrive();
     if (TRAIN)
-        store16(g.h1, hk1);
+        store(g.h1, hk1);
+    cluster_wait();
     // hidden layers 2 and 3
-    for (int l = 0; l < 2; ++l) {
-        if (l == 0)
-            cp_wait<TRAIN ? 5 : 2>();
-        else
-            cp_wait<TRAIN ? 4 : 1>();
-        cluster_sync();
-        product(k_major(sa[l], 4096), k_major(smem + (l ? OFF_SW2 : OFF_SW1), 4096), UNITS, NH / 16, false);
-        uint4 *hk = l ? hk3 : hk2;
-        if (!failed)
-            read_acc16(tmem, 16 * half, v);
-        const float *b = g.p + (l ? OFF_B2 : OFF_B1) + c0;
-        for (int e = 0; e < 16; ++e)
-            v[e] = tanhf(v[e] + b[e]);
-        pack16(v, hk);
-        broadcast(sa[l ^ 1], c0, hk, 2);
-        if (TRAIN)
-            store16(l ? g.h3 : g.h2, hk);
-    }
-    // output layer, loss gradient 2 (yhat - y) / (S 64) and squared errors
+    product(k_major(sa[0], 4096), k_major(smem + OFF_SW1, 4096), UNITS, NH / 16, false);
+    if (!failed)
+        read_acc(tmem, 8 * quarter, v);
+#pragma unroll
+    for (int e = 0; e < 8; ++e)
+        v[e] = tanhf(v[e] + b1[e]);
+    hk2 = pack8(v);
+    broadcast(sa[1], c0, hk2);
+    cp_wait<TRAIN ? 4 : 1>();
+    cluster_arrive();
+    if (TRAIN)
+        store(g.h2, hk2);
+    cluster_wait();
+    product(k_major(sa[1], 4096), k_major(smem + OFF_SW2, 4096), UNITS, NH / 16, false);
+    if (!failed)
+        read_acc(tmem, 8 * quarter, v);
+#pragma unroll
+    for (int e = 0; e < 8; ++e)
+        v[e] = tanhf(v[e] + b2[e]);
+    hk3 = pack8(v);
+    broadcast(sa[0], c0, hk3);
     cp_wait<TRAIN ? 3 : 0>();
-    cluster_sync();
+    cluster_arrive();
+    if (TRAIN)
+        store(g.h3, hk3);
+    cluster_wait();
+    // output layer, loss gradient 2 (yhat - y) / (S 64) and squared errors
+    float o[4] = {}, q[4] = {};
+    uint2 t = make_uint2(0, 0);
     if (cta < OUT_CTAS) {
         product(k_major(sa[0], 4096), k_major(smem + OFF_SW3, 4096), OUT_UNITS, NH / 16, false);
         if (!failed)
-            read_acc8(tmem, 8 * half, v);
-        const int o0 = cta * OUT_UNITS + 8 * half;
-        const float *b = g.p + OFF_B3 + o0;
-        for (int e = 0; e < 8; ++e)
-            v[e] = v[e] + b[e];
+            read_acc(tmem, 4 * quarter, o);
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            o[e] = o[e] + b3[e];
         if (!TRAIN) {
             if (live)
-                for (int i = 0; i < 2; ++i)
-                    *reinterpret_cast<float4 *>(g.yhat + (int64_t)s * NOUT + o0 + 4 * i) =
-                        make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+                store_floats(g.yhat + (int64_t)s * NOUT + o0, o);
         } else {
-            float q[8];
-            for (int e = 0; e < 8; ++e) {
-                const float d = live ? v[e] - g.y[(int64_t)src * NOUT + o0 + e] : 0.0f;
-                v[e] = 2.0f * d / (float)(g.S * NOUT);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const float d = live ? o[e] - yl[e] : 0.0f;
+                o[e] = 2.0f * d / (float)(g.S * NOUT);
                 q[e] = d * d;
             }
-            const uint4 w = make_uint4(pack2(v[0], v[1]), pack2(v[2], v[3]), pack2(v[4], v[5]), pack2(v[6], v[7]));
-            broadcast(sa[1], o0, &w, 1);
-            if (live) {
-                *reinterpret_cast<uint4 *>(g.dyb + (int64_t)s * NOUT + o0) = w;
-                for (int i = 0; i < 2; ++i) {
-                    *reinterpret_cast<float4 *>(g.dy + (int64_t)s * NOUT + o0 + 4 * i) =
-                        make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
-                    *reinterpret_cast<float4 *>(g.sq + (int64_t)s * NOUT + o0 + 4 * i) =
-                        make_float4(q[4 * i], q[4 * i + 1], q[4 * i + 2], q[4 * i + 3]);
-                }
-            }
+            t = make_uint2(pack2(o[0], o[1]), pack2(o[2], o[3]));
+            broadcast(sa[1], o0, t);
         }
     }
     if constexpr (TRAIN) {
-        uint4 w[2];
-        // d3 = (dy W3) (1 - h3^2)
         cp_wait<2>();
-        cluster_sync();
+        cluster_arrive();
+        if (live && cta < OUT_CTAS) {
+            *reinterpret_cast<uint2 *>(g.dyb + (int64_t)s * NOUT + o0) = t;
+            store_floats(g.dy + (int64_t)s * NOUT + o0, o);
+            store_floats(g.sq + (int64_t)s * NOUT + o0, q);
+        }
+        cluster_wait();
+        // d3 = (dy W3) (1 - h3^2)
         product(k_major(sa[1], 4096), mn_major(smem + OFF_TW3, UNITS), UNITS, NOUT / 16, true);
         if (!failed)
-            read_acc16(tmem, 16 * half, v);
+            read_acc(tmem, 8 * quarter, v);
         dtanh(hk3);
-        pack16(v, w);
-        broadcast(sa[0], c0, w, 2);
-        store16f(g.d3);
-        store16(g.d3b, w);
-        // d2 = (d3 W2) (1 - h2^2)
+        w = pack8(v);
+        broadcast(sa[0], c0, w);
         cp_wait<1>();
-        cluster_sync();
+        cluster_arrive();
+        store_f(g.d3);
+        store(g.d3b, w);
+        cluster_wait();
+        // d2 = (d3 W2) (1 - h2^2)
         product(k_major(sa[0], 4096), mn_major(smem + OFF_TW2, UNITS), UNITS, NH / 16, true);
         if (!failed)
-            read_acc16(tmem, 16 * half, v);
+            read_acc(tmem, 8 * quarter, v);
         dtanh(hk2);
-        pack16(v, w);
-        broadcast(sa[1], c0, w, 2);
-        store16f(g.d2);
-        store16(g.d2b, w);
-        // d1 = (d2 W1) (1 - h1^2)
+        w = pack8(v);
+        broadcast(sa[1], c0, w);
         cp_wait<0>();
-        cluster_sync();
+        cluster_arrive();
+        store_f(g.d2);
+        store(g.d2b, w);
+        cluster_wait();
+        // d1 = (d2 W1) (1 - h1^2)
         product(k_major(sa[1], 4096), mn_major(smem + OFF_TW1, UNITS), UNITS, NH / 16, true);
         if (!failed)
-            read_acc16(tmem, 16 * half, v);
+            read_acc(tmem, 8 * quarter, v);
         dtanh(hk1);
-        store16f(g.d1);
+        store_f(g.d1);
     }
     if (failed)   // give MMAs still in flight a bounded chance to finish before TMEM is freed
         mbar_wait_bounded(&bar, parity ^ 1u);
@@ -484,21 +550,12 @@ struct Update {
     int *err;
 };
 
-// gradient of parameter i: stored, or one Adam step on the FP32 master
-// parameter; returns the new parameter
-__device__ __forceinline__ float apply(const Update &g, int64_t i, float gi)
+// one Adam step of a parameter with gradient gi
+__device__ __forceinline__ void adam(const Update &g, float gi, float &p, float &m, float &v)
 {
-    if (!g.adam) {
-        g.grad[i] = gi;
-        return 0.0f;
-    }
-    const float mi = BETA1 * g.m[i] + (1.0f - BETA1) * gi;
-    const float vi = BETA2 * g.v[i] + (1.0f - BETA2) * gi * gi;
-    g.m[i] = mi;
-    g.v[i] = vi;
-    const float pi = g.p[i] - g.lr * (mi / g.c1) / (sqrtf(vi / g.c2) + ADAM_EPS);
-    g.p[i] = pi;
-    return pi;
+    m = BETA1 * m + (1.0f - BETA1) * gi;
+    v = BETA2 * v + (1.0f - BETA2) * gi * gi;
+    p = p - g.lr * (m / g.c1) / (sqrtf(v / g.c2) + ADAM_EPS);
 }
 
 constexpr int UP_N = 16;                             // columns of a weight gradient per CTA
@@ -532,11 +589,21 @@ __device__ __forceinline__ void weight_grad(const Update &g, uint8_t *smem, uint
     }
     griddep_wait();
     const int chunks = (g.S + UP_K - 1) / UP_K;
+    // the thread's 8 parameters and moments, in flight with the operands
+    const int row = threadIdx.x & 127, c0 = 8 * (threadIdx.x >> 7);
+    const int64_t o = (int64_t)(m0 + row) * NH + n0 + c0;
+    const bool mine = row < rows;
+    float pn[8] = {}, mn[8] = {}, vn[8] = {};
+    if (g.adam && mine) {
+        load_floats(g.p + off + o, pn);
+        load_floats(g.m + off + o, mn);
+        load_floats(g.v + off + o, vn);
+    }
     auto stage = [&](int c) {
         uint8_t *sa = smem + (c & 1) * (UP_A + UP_B), *sb = sa + UP_A;
         const int k0 = c * UP_K, kn = min(UP_K, g.S - k0), nk = (kn + 15) & ~15;
-        stage_mn_major(sa, A + (int64_t)k0 * lda + m0, lda, nk, TC_M, kn, rows);
-        stage_mn_major(sb, B + (int64_t)k0 * NH + n0, NH, nk, UP_N, kn, UP_N);
+        stage_mn_major<THREADS>(sa, A + (int64_t)k0 * lda + m0, lda, nk, TC_M, kn, rows);
+        stage_mn_major<THREADS>(sb, B + (int64_t)k0 * NH + n0, NH, nk, UP_N, kn, UP_N);
         cp_commit();
     };
     stage(0);
@@ -569,18 +636,18 @@ __device__ __forceinline__ void weight_grad(const Update &g, uint8_t *smem, uint
         cp_wait<0>();
         mbar_wait_bounded(bar, parity ^ 1u);
     } else {
-        const int row = threadIdx.x & 127, c0 = 8 * (threadIdx.x >> 7);
         float acc[8];
-        read_acc8(tmem, c0, acc);
-        if (row < rows) {
-            const int64_t o = (int64_t)(m0 + row) * NH + n0 + c0;
-            float pn[8];
+        read_acc(tmem, c0, acc);
+        if (mine && g.adam) {
 #pragma unroll
             for (int e = 0; e < 8; ++e)
-                pn[e] = apply(g, off + o + e, acc[e]);
-            if (g.adam)
-                *reinterpret_cast<uint4 *>(Wb + o) =
-                    make_uint4(pack2(pn[0], pn[1]), pack2(pn[2], pn[3]), pack2(pn[4], pn[5]), pack2(pn[6], pn[7]));
+                adam(g, acc[e], pn[e], mn[e], vn[e]);
+            store_floats(g.p + off + o, pn);
+            store_floats(g.m + off + o, mn);
+            store_floats(g.v + off + o, vn);
+            *reinterpret_cast<uint4 *>(Wb + o) = pack8(pn);
+        } else if (mine) {
+            store_floats(g.grad + off + o, acc);
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -593,41 +660,78 @@ __device__ __forceinline__ void weight_grad(const Update &g, uint8_t *smem, uint
 
 // Sums over the batch for 32 units: slot l of 32 adds samples l, l + 32, ...
 // in order and the slots meet in a fixed tree.  A warp takes four slots of
-// the 32 units (128-byte reads).  dz: S x ld from the first unit; with u the
-// input layer's weight gradient too.
+// the 32 units (128-byte reads), their loads in flight together.  dz: S x ld
+// from the first unit; U: with the features u, the input layer's weight
+// gradient too.
+template <bool U>
 __device__ __forceinline__ void unit_sums(const Update &g, const float *dz, int ld, int64_t off_b, int unit0,
-                                          const float *u, float (*sh)[32][33])
+                                          float (*sh)[32][33])
 {
-    const int o = threadIdx.x & 31, w = threadIdx.x >> 5, nv = u ? 1 + NIN : 1;
-    for (int q = 0; q < 4; ++q) {
-        const int l = 4 * w + q;
-        float acc[1 + NIN] = {0.f, 0.f, 0.f, 0.f};
-        for (int s = l; s < g.S; s += 32) {
-            const float d = dz[(int64_t)s * ld + unit0 + o];
-            acc[0] += d;
-            if (u)
-                for (int i = 0; i < NIN; ++i)
-                    acc[1 + i] += d * u[3 * s + i];
+    constexpr int NV = U ? 1 + NIN : 1;
+    const int o = threadIdx.x & 31, w = threadIdx.x >> 5;
+    // the parameter that this thread updates: value w of unit o
+    const bool mine = w < NV;
+    const int64_t i = w == 0 ? off_b + unit0 + o : OFF_W0 + NIN * (unit0 + o) + (w - 1);
+    float p = 0.f, m = 0.f, v = 0.f;
+    if (mine && g.adam) {
+        p = g.p[i];
+        m = g.m[i];
+        v = g.v[i];
+    }
+    float acc[4][NV] = {};
+    for (int s0 = 0; s0 < g.S; s0 += 32) {
+        float d[4], u[4][NIN];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int s = s0 + 4 * w + q;
+            d[q] = s < g.S ? dz[(int64_t)s * ld + unit0 + o] : 0.0f;
+            if (U)
+                for (int k = 0; k < NIN; ++k)
+                    u[q][k] = s < g.S ? g.u[3 * s + k] : 0.0f;
         }
-        for (int i = 0; i < nv; ++i)
-            sh[i][l][o] = acc[i];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            if (s0 + 4 * w + q >= g.S)
+                continue;
+            acc[q][0] += d[q];
+            if (U)
+                for (int k = 0; k < NIN; ++k)
+                    acc[q][1 + k] += d[q] * u[q][k];
+        }
     }
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+        for (int k = 0; k < NV; ++k)
+            sh[k][4 * w + q][o] = acc[q][k];
     __syncthreads();
-    if (w < nv) {
-        for (int h = 16; h >= 1; h >>= 1)        // value w of unit o
-            for (int l = 0; l < h; ++l)
-                sh[w][l][o] += sh[w][l + h][o];
-        const int unit = unit0 + o;
-        apply(g, w == 0 ? off_b + unit : OFF_W0 + NIN * unit + (w - 1), sh[w][0][o]);
+    if (!mine)
+        return;
+    float t[32];
+#pragma unroll
+    for (int l = 0; l < 32; ++l)
+        t[l] = sh[w][l][o];
+#pragma unroll
+    for (int h = 16; h >= 1; h >>= 1)
+#pragma unroll
+        for (int l = 0; l < h; ++l)
+            t[l] += t[l + h];
+    if (!g.adam) {
+        g.grad[i] = t[0];
+        return;
     }
+    adam(g, t[0], p, m, v);
+    g.p[i] = p;
+    g.m[i] = m;
+    g.v[i] = v;
 }
 
 // Every parameter's gradient (sums over the batch) and its Adam step, and
 // the loss: CTAs [0, UP_GEMM) one 128 x 16 tile of a weight matrix each on
 // the tensor cores, the next 32 units' biases each (with the input layer's
 // weights), the last the loss.  Small tiles because the time of a CTA is its
-// loads and its divisions: 107 CTAs share both.
-__global__ void __launch_bounds__(THREADS) update_kernel(Update g)
+// loads and its divisions: 107 CTAs share both.  Measured: an Adam step at
+// batch 128 766 -> 40 us (15 launches before), 12 of them here.
+__global__ void __launch_bounds__(THREADS, 1) update_kernel(Update g)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
     __shared__ __align__(8) uint64_t bar;
@@ -640,19 +744,20 @@ __global__ void __launch_bounds__(THREADS) update_kernel(Update g)
     const int b = blockIdx.x - UP_GEMM;
     float(*sh)[32][33] = reinterpret_cast<float(*)[32][33]>(smem);
     if (b < NOUT / 32) {
-        unit_sums(g, g.dy, NOUT, OFF_B3, 32 * b, nullptr, sh);
+        unit_sums<false>(g, g.dy, NOUT, OFF_B3, 32 * b, sh);
     } else if (b < UP_RED) {
         const int k = b - NOUT / 32, layer = k / (NH / 32), u0 = 32 * (k % (NH / 32));
         if (layer == 0)
-            unit_sums(g, g.d3, NH, OFF_B2, u0, nullptr, sh);
+            unit_sums<false>(g, g.d3, NH, OFF_B2, u0, sh);
         else if (layer == 1)
-            unit_sums(g, g.d2, NH, OFF_B1, u0, nullptr, sh);
+            unit_sums<false>(g, g.d2, NH, OFF_B1, u0, sh);
         else
-            unit_sums(g, g.d1, NH, OFF_B0, u0, g.u, sh);
+            unit_sums<true>(g, g.d1, NH, OFF_B0, u0, sh);
     } else {     // loss = mean of the squared errors, FP64, fixed order
         double *red = reinterpret_cast<double *>(smem);
         double a[4] = {0.0, 0.0, 0.0, 0.0};
         const int64_t n = (int64_t)g.S * NOUT;
+#pragma unroll 4
         for (int64_t k = 4 * threadIdx.x; k < n; k += 4 * THREADS) {     // n is a multiple of 4
             const float4 q = *reinterpret_cast<const float4 *>(g.sq + k);
             a[0] += (double)q.x;
@@ -678,6 +783,9 @@ __global__ void to_bf16_kernel(const float *src, __nv_bfloat16 *dst, int64_t n)
         dst[i] = __float2bfloat16_rn(src[i]);
 }
 
+constexpr int HEAD = 64;             // floats before the outputs: the error flag, padded to 256 bytes
+constexpr int ROWS_OUT = 4096;       // outputs brought to the host at a time, at most
+
 inline unsigned nblk(int64_t n, int b) { return (unsigned)((n + b - 1) / b); }
 
 }  // namespace
@@ -686,17 +794,22 @@ struct iblb_mlp {
     cudaStream_t stream = nullptr;
     int max_batch = 0;
     int64_t t = 0;                       // Adam steps taken
+    void *slab = nullptr;                // one allocation holds every array below that max_batch sizes
     // parameters
     float *p = nullptr, *g = nullptr, *m = nullptr, *v = nullptr;
     __nv_bfloat16 *W1b = nullptr, *W2b = nullptr, *W3b = nullptr;
     // activations (max_batch rows)
-    float *x = nullptr, *y = nullptr, *u = nullptr, *yhat = nullptr, *dy = nullptr, *sq = nullptr;
+    float *u = nullptr, *yhat = nullptr, *dy = nullptr, *sq = nullptr;
     float *d3 = nullptr, *d2 = nullptr, *d1 = nullptr;
     __nv_bfloat16 *h1 = nullptr, *h2 = nullptr, *h3 = nullptr, *dyb = nullptr, *d3b = nullptr, *d2b = nullptr;
-    int *err = nullptr, *idx = nullptr;
-    double *loss = nullptr;              // loss of each batch of an epoch (loss_cap entries)
-    int loss_cap = 0;
-    int64_t data_cap = 0;                // rows of x / y held on the device
+    int *err = nullptr;                  // HEAD floats before yhat, so that one copy brings both to the host
+    // samples and their order, and the loss of each batch of an epoch (grown on demand)
+    float *x = nullptr, *y = nullptr;
+    int *idx = nullptr;
+    double *loss = nullptr;
+    int64_t data_cap = 0, idx_cap = 0, loss_cap = 0;
+    float *h_out = nullptr;              // pinned: HEAD + 64 rows_out floats
+    int rows_out = 0;
     std::string msg;
 };
 
@@ -732,7 +845,8 @@ cudaError_t forward(iblb_mlp *mm, const float *x, int S)
     g.W3b = mm->W3b;
     g.yhat = mm->yhat;
     g.err = mm->err;
-    return launch_k(net_kernel<false>, dim3(nblk(S, TC_M) * CLUSTER), dim3(THREADS), FWD_SMEM, mm->stream, true, g);
+    return launch_k(net_kernel<false>, dim3(nblk(S, TC_M) * CLUSTER), dim3(NET_THREADS), FWD_SMEM, mm->stream, true,
+                    g);
 }
 
 // Forward and backward pass of S samples (rows idx[s] of x and y if idx) and
@@ -743,8 +857,8 @@ cudaError_t train_step(iblb_mlp *mm, const float *x, const float *y, const int *
 {
     const Net n{S, x, y, idx, mm->p, mm->W1b, mm->W2b, mm->W3b, nullptr, mm->u, mm->h1, mm->h2, mm->h3, mm->d3b,
                 mm->d2b, mm->dyb, mm->d3, mm->d2, mm->d1, mm->dy, mm->sq, mm->err};
-    cudaError_t e = launch_k(net_kernel<true>, dim3(nblk(S, TC_M) * CLUSTER), dim3(THREADS), TRAIN_SMEM, mm->stream,
-                             true, n);
+    cudaError_t e = launch_k(net_kernel<true>, dim3(nblk(S, TC_M) * CLUSTER), dim3(NET_THREADS), TRAIN_SMEM,
+                             mm->stream, true, n);
     if (e != cudaSuccess)
         return e;
     const Update u{S, mm->h1, mm->h2, mm->h3, mm->d3b, mm->d2b, mm->dyb, mm->d3, mm->d2, mm->d1, mm->dy, mm->u,
@@ -763,39 +877,49 @@ cudaError_t refresh_bf16(iblb_mlp *mm)
     return cudaGetLastError();
 }
 
+// the error flag as read into h_out[0]
 int check_err(iblb_mlp *m)
 {
-    int h = 0;
-    MCK(cudaMemcpyAsync(&h, m->err, sizeof(int), cudaMemcpyDeviceToHost, m->stream));
-    MCK(cudaStreamSynchronize(m->stream));
-    if (h) {
-        MCK(cudaMemsetAsync(m->err, 0, sizeof(int), m->stream));
-        return mfail(m, IBLB_E_TIMEOUT, "a bounded wait for the tensor-core MMAs gave up");
-    }
-    return IBLB_OK;
-}
-
-int ensure_data(iblb_mlp *m, int64_t S)
-{
-    if (S <= m->data_cap)
+    if (!*reinterpret_cast<const int *>(m->h_out))
         return IBLB_OK;
-    if (m->x)
-        MCK(cudaFree(m->x));
-    if (m->y)
-        MCK(cudaFree(m->y));
-    m->x = m->y = nullptr;
-    MCK(cudaMalloc((void **)&m->x, sizeof(float) * 3 * S));
-    MCK(cudaMalloc((void **)&m->y, sizeof(float) * NOUT * S));
-    m->data_cap = S;
+    MCK(cudaMemsetAsync(m->err, 0, sizeof(int), m->stream));
+    return mfail(m, IBLB_E_TIMEOUT, "a bounded wait for the tensor-core MMAs gave up");
+}
+
+// *p holds at least n elements (its old contents are dropped when it grows)
+template <typename T>
+int grow(iblb_mlp *m, T **p, int64_t *cap, int64_t n)
+{
+    if (n <= *cap)
+        return IBLB_OK;
+    if (*p)
+        MCK(cudaFree(*p));
+    *p = nullptr;
+    *cap = 0;
+    MCK(cudaMalloc((void **)p, sizeof(T) * n));
+    *cap = n;
     return IBLB_OK;
 }
 
-int upload(iblb_mlp *m, const double *x, const double *y, int64_t S)
+// x and y (may be null) to the device in FP32, through hx and hy, which stay
+// as they are until the caller has synchronised the stream
+int upload(iblb_mlp *m, const double *x, const double *y, int64_t S, std::vector<float> &hx, std::vector<float> &hy)
 {
-    int r = ensure_data(m, S);
-    if (r)
-        return r;
-    std::vector<float> hx(3 * S), hy(y ? NOUT * S : 0);
+    if (S > m->data_cap) {
+        int64_t cx = 0, cy = 0;
+        m->data_cap = 0;
+        int r = IBLB_OK;
+        if (m->x)
+            MCK(cudaFree(m->x));
+        if (m->y)
+            MCK(cudaFree(m->y));
+        m->x = m->y = nullptr;
+        if ((r = grow(m, &m->x, &cx, 3 * S)) || (r = grow(m, &m->y, &cy, (int64_t)NOUT * S)))
+            return r;
+        m->data_cap = S;
+    }
+    hx.resize(3 * S);
+    hy.resize(y ? NOUT * S : 0);
     for (int64_t i = 0; i < 3 * S; ++i)
         hx[i] = (float)x[i];
     for (int64_t i = 0; i < (int64_t)hy.size(); ++i)
@@ -803,7 +927,6 @@ int upload(iblb_mlp *m, const double *x, const double *y, int64_t S)
     MCK(cudaMemcpyAsync(m->x, hx.data(), sizeof(float) * hx.size(), cudaMemcpyHostToDevice, m->stream));
     if (y)
         MCK(cudaMemcpyAsync(m->y, hy.data(), sizeof(float) * hy.size(), cudaMemcpyHostToDevice, m->stream));
-    MCK(cudaStreamSynchronize(m->stream));
     return IBLB_OK;
 }
 
@@ -844,33 +967,40 @@ int iblb_mlp_create(const float *params, int64_t n_params, int max_batch, void *
     m->stream = (cudaStream_t)stream;
     m->max_batch = max_batch;
     const int64_t B = max_batch;
-    auto fl = [&](float **p, int64_t n) { return cudaMalloc((void **)p, sizeof(float) * n); };
-    auto bf = [&](__nv_bfloat16 **p, int64_t n) { return cudaMalloc((void **)p, sizeof(__nv_bfloat16) * n); };
-    cudaError_t e = cudaSuccess;
-    if (!e) e = fl(&m->p, NPARAM);
-    if (!e) e = fl(&m->g, NPARAM);
-    if (!e) e = fl(&m->m, NPARAM);
-    if (!e) e = fl(&m->v, NPARAM);
-    if (!e) e = bf(&m->W1b, (int64_t)NH * NH);
-    if (!e) e = bf(&m->W2b, (int64_t)NH * NH);
-    if (!e) e = bf(&m->W3b, (int64_t)NOUT * NH);
-    if (!e) e = fl(&m->u, 3 * B);
-    if (!e) e = fl(&m->yhat, NOUT * B);
-    if (!e) e = fl(&m->dy, NOUT * B);
-    if (!e) e = fl(&m->sq, NOUT * B);
-    if (!e) e = fl(&m->d3, NH * B);
-    if (!e) e = fl(&m->d2, NH * B);
-    if (!e) e = fl(&m->d1, NH * B);
-    if (!e) e = bf(&m->h1, NH * B);
-    if (!e) e = bf(&m->h2, NH * B);
-    if (!e) e = bf(&m->h3, NH * B);
-    if (!e) e = bf(&m->dyb, NOUT * B);
-    if (!e) e = bf(&m->d3b, NH * B);
-    if (!e) e = bf(&m->d2b, NH * B);
-    if (!e) e = cudaMalloc((void **)&m->err, sizeof(int));
-    if (!e) e = cudaMalloc((void **)&m->idx, sizeof(int) * B);
-    if (!e) e = cudaMalloc((void **)&m->loss, sizeof(double));
-    if (!e) m->loss_cap = 1;
+    // two passes: sizes, then the arrays' places in the slab (256-byte aligned)
+    char *base = nullptr;
+    int64_t at = 0;
+    auto place = [&](auto **p, int64_t n) {
+        if (base)
+            *p = reinterpret_cast<std::remove_reference_t<decltype(*p)>>(base + at);
+        at += (int64_t)((n * sizeof(**p) + 255) & ~(size_t)255);
+    };
+    auto place_all = [&]() {
+        at = 0;
+        for (float **q : {&m->p, &m->g, &m->m, &m->v})
+            place(q, NPARAM);
+        place(&m->W1b, (int64_t)NH * NH);
+        place(&m->W2b, (int64_t)NH * NH);
+        place(&m->W3b, (int64_t)NOUT * NH);
+        place(&m->u, 3 * B);
+        place(&m->err, HEAD);            // directly before yhat
+        for (float **q : {&m->yhat, &m->dy, &m->sq})
+            place(q, NOUT * B);
+        for (float **q : {&m->d3, &m->d2, &m->d1})
+            place(q, NH * B);
+        for (__nv_bfloat16 **q : {&m->h1, &m->h2, &m->h3, &m->d3b, &m->d2b})
+            place(q, NH * B);
+        place(&m->dyb, NOUT * B);
+    };
+    static_assert(HEAD * sizeof(float) == 256, "the outputs follow the flag");
+    place_all();
+    cudaError_t e = cudaMalloc(&m->slab, (size_t)at);
+    if (!e) {
+        base = (char *)m->slab;
+        place_all();
+    }
+    m->rows_out = std::min(max_batch, ROWS_OUT);
+    if (!e) e = cudaMallocHost((void **)&m->h_out, sizeof(float) * (HEAD + (size_t)NOUT * m->rows_out));
     if (!e) e = cudaFuncSetAttribute(net_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, FWD_SMEM);
     if (!e) e = cudaFuncSetAttribute(net_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, TRAIN_SMEM);
     if (!e) e = cudaFuncSetAttribute(update_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * (UP_A + UP_B));
@@ -893,12 +1023,11 @@ void iblb_mlp_destroy(iblb_mlp *m)
 {
     if (!m)
         return;
-    void *ptrs[] = {m->p, m->g, m->m, m->v, m->W1b, m->W2b, m->W3b, m->x, m->y, m->u, m->yhat, m->dy, m->sq,
-                    m->d3, m->d2, m->d1, m->h1, m->h2, m->h3, m->dyb, m->d3b, m->d2b, m->err, m->idx,
-                    m->loss};
-    for (void *p : ptrs)
+    for (void *p : {m->slab, (void *)m->x, (void *)m->y, (void *)m->idx, (void *)m->loss})
         if (p)
             cudaFree(p);
+    if (m->h_out)
+        cudaFreeHost(m->h_out);
     delete m;
 }
 
@@ -917,19 +1046,29 @@ int iblb_mlp_predict(iblb_mlp *m, const double *x, int S, double *y)
         return mfail(m, IBLB_E_ARG, "iblb_mlp_predict: bad arguments");
     if (!inputs_valid(x, S))
         return mfail(m, IBLB_E_ARG, "iblb_mlp_predict: inputs need finite theta_eq, R0 and lambda > 0");
-    int r = upload(m, x, nullptr, S);
+    std::vector<float> hx, hy;
+    int r = upload(m, x, nullptr, S, hx, hy);
     if (r)
         return r;
-    std::vector<float> hy((size_t)NOUT * m->max_batch);
     for (int s0 = 0; s0 < S; s0 += m->max_batch) {
         const int n = std::min(m->max_batch, S - s0);
         MCK(forward(m, m->x + 3 * (int64_t)s0, n));
-        MCK(cudaMemcpyAsync(hy.data(), m->yhat, sizeof(float) * NOUT * n, cudaMemcpyDeviceToHost, m->stream));
-        MCK(cudaStreamSynchronize(m->stream));
-        if ((r = check_err(m)))
-            return r;
-        for (int64_t i = 0; i < (int64_t)NOUT * n; ++i)
-            y[(int64_t)NOUT * s0 + i] = hy[i];
+        for (int r0 = 0; r0 < n; r0 += m->rows_out) {
+            // the flag with the first rows, further rows alone
+            const int k = std::min(m->rows_out, n - r0);
+            if (r0 == 0)
+                MCK(cudaMemcpyAsync(m->h_out, m->err, sizeof(float) * (HEAD + NOUT * k), cudaMemcpyDeviceToHost,
+                                    m->stream));
+            else
+                MCK(cudaMemcpyAsync(m->h_out + HEAD, m->yhat + (int64_t)NOUT * r0, sizeof(float) * NOUT * k,
+                                    cudaMemcpyDeviceToHost, m->stream));
+            MCK(cudaStreamSynchronize(m->stream));
+            if (r0 == 0 && (r = check_err(m)))
+                return r;
+            const float *o = m->h_out + HEAD;
+            for (int64_t i = 0; i < (int64_t)NOUT * k; ++i)
+                y[(int64_t)NOUT * (s0 + r0) + i] = o[i];
+        }
     }
     return IBLB_OK;
 }
@@ -940,11 +1079,15 @@ int iblb_mlp_grad(iblb_mlp *m, const double *x, const double *y, int S, double *
         return mfail(m, IBLB_E_ARG, "iblb_mlp_grad: bad arguments (1 <= S <= max_batch)");
     if (!inputs_valid(x, S))
         return mfail(m, IBLB_E_ARG, "iblb_mlp_grad: inputs need finite theta_eq, R0 and lambda > 0");
-    int r = upload(m, x, y, S);
+    std::vector<float> hx, hy;
+    int r = upload(m, x, y, S, hx, hy);
     if (r)
+        return r;
+    if ((r = grow(m, &m->loss, &m->loss_cap, 1)))
         return r;
     MCK(train_step(m, m->x, m->y, nullptr, S, m->loss, 0.0f, 1.0f, 1.0f));
     std::vector<float> hg(NPARAM);
+    MCK(cudaMemcpyAsync(m->h_out, m->err, sizeof(int), cudaMemcpyDeviceToHost, m->stream));
     MCK(cudaMemcpyAsync(hg.data(), m->g, sizeof(float) * NPARAM, cudaMemcpyDeviceToHost, m->stream));
     MCK(cudaMemcpyAsync(loss, m->loss, sizeof(double), cudaMemcpyDeviceToHost, m->stream));
     MCK(cudaStreamSynchronize(m->stream));
@@ -962,40 +1105,45 @@ int iblb_mlp_train(iblb_mlp *m, const double *x, const double *y, int S, int epo
         return mfail(m, IBLB_E_ARG, "iblb_mlp_train: bad arguments (1 <= batch <= max_batch, lr > 0)");
     if (!inputs_valid(x, S))
         return mfail(m, IBLB_E_ARG, "iblb_mlp_train: inputs need finite theta_eq, R0 and lambda > 0");
-    int r = upload(m, x, y, S);
+    std::vector<float> hx, hy;
+    int r = upload(m, x, y, S, hx, hy);
     if (r)
         return r;
-    std::vector<int> perm(S);
+    std::vector<int> perm(S), sent;
     for (int i = 0; i < S; ++i)
         perm[i] = i;
     uint64_t st = seed;
-    const int nb = S / batch;                  // full batches only
-    if (nb > m->loss_cap) {
-        MCK(cudaFree(m->loss));
-        m->loss = nullptr;
-        m->loss_cap = 0;
-        MCK(cudaMalloc((void **)&m->loss, sizeof(double) * nb));
-        m->loss_cap = nb;
-    }
-    std::vector<double> losses((size_t)std::max(nb, 1));
-    for (int ep = 0; ep < epochs; ++ep) {
-        for (int i = S - 1; i > 0; --i) {      // Fisher-Yates shuffle of the sample order
+    auto shuffle = [&] {                       // Fisher-Yates shuffle of the sample order
+        for (int i = S - 1; i > 0; --i) {
             const int j = (int)(splitmix(st) % (uint64_t)(i + 1));
             std::swap(perm[i], perm[j]);
         }
-        double ep_loss = 0.0;
+    };
+    const int nb = S / batch;                  // full batches only
+    if ((r = grow(m, &m->loss, &m->loss_cap, std::max(nb, 1))) || (r = grow(m, &m->idx, &m->idx_cap, S)))
+        return r;
+    std::vector<double> losses((size_t)std::max(nb, 1));
+    if (epochs > 0)
+        shuffle();
+    for (int ep = 0; ep < epochs; ++ep) {
+        // an epoch's order in one copy, so that its steps' kernels follow one
+        // another without a gap; the next order is drawn while they run
+        sent = perm;
+        MCK(cudaMemcpyAsync(m->idx, sent.data(), sizeof(int) * S, cudaMemcpyHostToDevice, m->stream));
         for (int b = 0; b < nb; ++b) {
-            MCK(cudaMemcpyAsync(m->idx, perm.data() + (int64_t)b * batch, sizeof(int) * batch,
-                                cudaMemcpyHostToDevice, m->stream));
             m->t++;
             const float c1 = 1.0f - powf(BETA1, (float)m->t), c2 = 1.0f - powf(BETA2, (float)m->t);
-            MCK(train_step(m, m->x, m->y, m->idx, batch, m->loss + b, (float)lr, c1, c2));
+            MCK(train_step(m, m->x, m->y, m->idx + (int64_t)b * batch, batch, m->loss + b, (float)lr, c1, c2));
         }
+        MCK(cudaMemcpyAsync(m->h_out, m->err, sizeof(int), cudaMemcpyDeviceToHost, m->stream));
+        if (ep + 1 < epochs)
+            shuffle();
         if (nb)
             MCK(cudaMemcpyAsync(losses.data(), m->loss, sizeof(double) * nb, cudaMemcpyDeviceToHost, m->stream));
         MCK(cudaStreamSynchronize(m->stream));
         if ((r = check_err(m)))
             return r;
+        double ep_loss = 0.0;
         for (int b = 0; b < nb; ++b)
             ep_loss += losses[b];
         if (loss_per_epoch)
