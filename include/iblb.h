@@ -157,8 +157,9 @@ typedef struct {
                                  max(1, 256 / nx) rows (1..4; 0 = 1); setting it sets
                                  IBLB_OPT_LB_GROUP_CELLS to 0                            */
 #define IBLB_OPT_LB_STAGES 4  /* shared-memory stages of the stream-collide pipeline:
-                                 the most groups in flight per block (2..8; default 3;
-                                 lowered to the most that fit in shared memory)          */
+                                 the most groups in flight per block (2..8; lowered to the
+                                 most that fit in shared memory; until set, 2 or 3, chosen
+                                 with the group size)                                    */
 #define IBLB_OPT_FUSED_IB 5   /* 1: the membrane work of a step runs as two cooperative
                                  kernels (forces + spread; advection + volume
                                  correction) with grid barriers between their phases,
@@ -184,7 +185,8 @@ typedef struct {
 #define IBLB_OPT_LB_GROUP_CELLS 10 /* about this many cells per stream-collide group
                                  (whole rows: max(1, round(cells / nx)) rows, at most ny),
                                  in place of IBLB_OPT_LB_ROW_MULT (1..16384; 0 = use the
-                                 multiplier; default 768)                                */
+                                 multiplier; until either is set, chosen from the boxes'
+                                 sizes and the storage)                                  */
 #define IBLB_OPT_GRAPH_CHUNK 11 /* steps per replayed CUDA graph (1..64; default 1): with
                                  K > 1, iblb_step runs whole chunks of K steps as one
                                  captured graph each and the rest one step per graph,

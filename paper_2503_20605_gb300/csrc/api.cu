@@ -60,6 +60,11 @@ struct iblb_ctx {
     bool any_vartau = false, any_volcorr = false;
     Arrays A{};
     Drop *d_drops = nullptr;
+    std::vector<int4> grp;         // stream-collide groups and constants of the current layout
+    std::vector<LbConst> lbc;
+    bool grp_dirty = true;         // not yet on the device
+    int4 *d_grp = nullptr;
+    LbConst *d_lbc = nullptr;
     void *fbuf[2] = {nullptr, nullptr};
     int cur = 0;
     int *d_tri = nullptr, *d_adj_start = nullptr, *d_adj = nullptr;
@@ -87,7 +92,8 @@ struct iblb_ctx {
     double step_ms = 0.0;
     int64_t prof_steps = 0;
     int64_t step_count = 0;
-    LaunchCfg cfg{0, 2, 148, 3, 1, 768};
+    LaunchCfg cfg{0, 2, 148, 3, 1, 0};
+    bool auto_cells = true, auto_stages = true;   // group size / pipeline depth by pick_shape
     int *h_status = nullptr;     // pinned, 4 per droplet
     double *obs_scr = nullptr;   // scratch of the mesh observation kernels
     int64_t obs_scr_n = 0;
@@ -355,12 +361,79 @@ void fit_stages(iblb_ctx *c)
         --c->cfg.lb_stages;
 }
 
+// rows per stream-collide group for about `cells` cells, of ny rows of pitch P
+int rows_for(int cells, const Drop &D) { return std::min(D.ny, std::max(1, (cells + D.nx / 2) / D.nx)); }
+
+// Group size and pipeline depth of the stream-collide kernel, unless they were
+// set: the pair with the least estimated time over the persistent blocks.
+// A group costs its cells plus a fixed part worth kGroupCells cells (its
+// hand-over and the latency of one pass; 128^3 in FP16, one block's time per
+// group at 256 .. 1024 cells), and half of an uneven last round is idle (the
+// blocks that still run get the others' bandwidth).  Two blocks an SM, as
+// registers allow, need their stages to fit half its shared memory; two
+// stages instead of three make larger groups fit, which pays when a block
+// has only a group or two.  Measured in the step (stream-collide, us, against
+// 768 cells, three stages and a short last group a plane): 32^3 FP32 6.1 ->
+// 4.6, 80^2 x 60 FP32 13.6 -> 9.8, 61 x 53 x 47 FP32 9.2 -> 7.3, 64 boxes of
+// 48 to 96 in FP16 491 -> 416, 32 boxes with tau_in != tau_out 232 -> 171.
+constexpr int kGroupCells = 160;
+constexpr int64_t kLbSmemSm = 228 * 1024, kLbSmemBlock = 1024 + 128;   // an SM's; reserved and static per block
+void pick_shape(iblb_ctx *c)
+{
+    const int sb = (int)storage_bytes(c->storage);
+    double best = 1e300;
+    const int ns_set = c->cfg.lb_stages, cells_set = c->cfg.lb_group_cells;
+    for (int ns = c->auto_stages ? 2 : ns_set; ns <= (c->auto_stages ? 3 : ns_set); ++ns)
+        for (int cells = 32; cells <= 1024; cells += 32) {
+            int64_t stage = 0, groups = 0;
+            double work = 0.0, largest = 0.0;
+            for (const Drop &D : c->drops) {
+                const int P = (D.nx * sb + 15) / 16 * 16 / sb, gpp = (D.ny - 1) / rows_for(cells, D) + 1;
+                const int rows = (D.ny - 1) / gpp + 1;
+                stage = std::max(stage, (int64_t)lb_stage_bytes(rows, P, sb, c->ndrops > 1));
+                groups += (int64_t)gpp * D.nzf;
+                work += (double)D.nzf * ((double)gpp * kGroupCells + (double)D.ny * P);
+                largest = std::max(largest, (double)rows * P + kGroupCells);
+            }
+            const int64_t fit = (kLbSmemSm / 2 >= ns * stage + kLbSmemBlock) ? 2 : 1;
+            if (ns * stage > kLbSmemOptin)
+                continue;
+            const double blocks = (double)c->cfg.sm_count * fit, rounds = groups / blocks;
+            double cost = work / blocks + 0.5 * (std::ceil(rounds) - rounds) * largest;
+            if (groups <= blocks)
+                cost = largest;
+            // one block an SM has half the warps: slower, except where FP32's
+            // traffic leaves them idle and there are rounds enough to fill in
+            if (fit == 1)
+                cost *= sb == 4 && rounds > 3.0 ? 0.5 : 0.6;
+            if (ns == 2 && rounds > 2.0)
+                cost *= 1.1;
+            if (cost < best) {
+                best = cost;
+                if (c->auto_cells)
+                    c->cfg.lb_group_cells = cells;
+                if (c->auto_stages)
+                    c->cfg.lb_stages = ns;
+            }
+        }
+    if (!c->auto_cells)
+        c->cfg.lb_group_cells = cells_set;
+    else if (best == 1e300)
+        c->cfg.lb_group_cells = 32;   // rows too long for two full stages: layout shortens the groups
+}
+
 // Offsets of cells, tiles, columns, launch blocks for the current launch shape.
 void layout(iblb_ctx *c)
 {
+    if (c->auto_cells)
+        pick_shape(c);
     int64_t cell0 = 0, tile0 = 0, col0 = 0, pcell0 = 0, row0 = 0, trow0 = 0;
-    int lb0 = 0, mb0 = 0, stage = 0;
+    int mb0 = 0, stage = 0;
     const int sb = (int)storage_bytes(c->storage);
+    const bool several = c->ndrops > 1;
+    c->grp.clear();
+    c->lbc.clear();
+    c->grp_dirty = true;
     for (auto &D : c->drops) {
         D.cell0 = cell0;
         D.tile0 = tile0;
@@ -373,25 +446,56 @@ void layout(iblb_ctx *c)
         D.pcells = (int64_t)D.pitch * D.ny * D.nzf;
         D.pcell0 = pcell0;
         D.row0 = row0;
-        D.lb_rows = std::min(D.ny, c->cfg.lb_group_cells > 0
-                                       ? std::max(1, (c->cfg.lb_group_cells + D.nx / 2) / D.nx)
-                                       : c->cfg.lb_row_mult * lb_rows_per_group(D.nx));
+        D.lb_rows = c->cfg.lb_group_cells > 0 ? rows_for(c->cfg.lb_group_cells, D)
+                                              : std::min(D.ny, c->cfg.lb_row_mult * lb_rows_per_group(D.nx));
         // two stages of the group must fit the opt-in shared memory of a block
-        while (D.lb_rows > 1 && 2 * (int64_t)lb_stage_bytes(D.lb_rows, D.pitch, sb) > kLbSmemOptin)
+        while (D.lb_rows > 1 && 2 * (int64_t)lb_stage_bytes(D.lb_rows, D.pitch, sb, several) > kLbSmemOptin)
             --D.lb_rows;
-        D.lb_gpp = (D.ny + D.lb_rows - 1) / D.lb_rows;
-        D.lb_block0 = lb0;
-        D.lb_nblocks = D.lb_gpp * D.nzf;
+        // as many groups a plane, their rows as even as they go: a short last
+        // group would fall to the same blocks in every round
+        const int d = (int)c->lbc.size(), gpp = (D.ny - 1) / D.lb_rows + 1;
+        D.lb_rows = (D.ny - 1) / gpp + 1;
+        for (int z = 0; z < D.nzf; ++z)
+            for (int g = 0; g < gpp; ++g) {
+                const int y = (int)((int64_t)D.ny * g / gpp);
+                c->grp.push_back(make_int4(d, y, z, (int)((int64_t)D.ny * (g + 1) / gpp) - y));
+            }
+        LbConst k{};
+        k.nx = D.nx;
+        k.ny = D.ny;
+        k.P = D.pitch;
+        k.R = D.lb_rows;
+        k.PC = (int)D.pcells;
+        k.nzf = D.nzf;
+        k.walls = D.walls;
+        k.vartau = D.vartau;
+        k.npr = lb_items_per_row(D.pitch, sb);
+        k.step_r = lb_consumers(sb) / k.npr;
+        k.step_x = lb_consumers(sb) - k.step_r * k.npr;
+        k.tx = D.tx;
+        k.ty = D.ty;
+        k.inv_npr = 1.0f / (float)k.npr;
+        k.bfx = D.bf[0];
+        k.bfy = D.bf[1];
+        k.bfz = D.bf[2];
+        k.rho0 = D.rho0;
+        k.omega_out = D.omega_out;
+        k.omega_in = D.omega_in;
+        k.pcell0 = D.pcell0;
+        k.col0 = D.col0;
+        k.tile0 = D.tile0;
+        k.trow0 = D.trow0;
+        k.has_bf = D.bf[0] != 0.0f || D.bf[1] != 0.0f || D.bf[2] != 0.0f;
+        c->lbc.push_back(k);
         D.mass_block0 = mb0;
         D.mass_nblocks = (int)((D.cells + MASS_CELLS_PER_BLOCK - 1) / MASS_CELLS_PER_BLOCK);
-        stage = std::max(stage, lb_stage_bytes(D.lb_rows, D.pitch, sb));
+        stage = std::max(stage, lb_stage_bytes(D.lb_rows, D.pitch, sb, several));
         cell0 += D.cells;
         pcell0 += D.pcells;
         row0 += (int64_t)D.ny * D.nzf;
         tile0 += D.ntiles;
         trow0 += (int64_t)D.ty * D.tz;
         col0 += (int64_t)D.nx * D.ny;
-        lb0 += D.lb_nblocks;
         mb0 += D.mass_nblocks;
     }
     c->A.total_cells = cell0;
@@ -400,7 +504,7 @@ void layout(iblb_ctx *c)
     c->A.total_tiles = tile0;
     c->A.total_trows = trow0;
     c->A.total_cols = col0;
-    c->A.lb_blocks_total = lb0;
+    c->A.lb_blocks_total = (int)c->grp.size();
     c->A.lb_stage_bytes = stage;
     c->mass_blocks = mb0;
     fit_stages(c);
@@ -408,6 +512,11 @@ void layout(iblb_ctx *c)
 
 int upload_drops(iblb_ctx *c)
 {
+    if (c->grp_dirty) {
+        CK(cudaMemcpyAsync(c->d_grp, c->grp.data(), sizeof(int4) * c->grp.size(), cudaMemcpyHostToDevice, c->stream));
+        CK(cudaMemcpyAsync(c->d_lbc, c->lbc.data(), sizeof(LbConst) * c->ndrops, cudaMemcpyHostToDevice, c->stream));
+        c->grp_dirty = false;
+    }
     CK(cudaMemcpyAsync(c->d_drops, c->drops.data(), sizeof(Drop) * c->ndrops, cudaMemcpyHostToDevice, c->stream));
     CK(cudaStreamSynchronize(c->stream));
     return IBLB_OK;
@@ -947,6 +1056,8 @@ int iblb_batch_create(int n, const iblb_lattice_desc *lat, const iblb_physics_de
         (e = dalloc(&A.col_z, (size_t)A.total_cols * MAXC)) != cudaSuccess ||
         (e = dalloc(&A.mass_part, (size_t)c->mass_blocks)) != cudaSuccess ||
         (e = dalloc(&A.status, 4 * (size_t)n)) != cudaSuccess ||
+        (e = dalloc(&c->d_grp, (size_t)A.total_rows)) != cudaSuccess ||
+        (e = dalloc(&c->d_lbc, (size_t)n)) != cudaSuccess ||
         (e = dalloc(&c->d_mass, (size_t)n)) != cudaSuccess || (e = dalloc(&c->d_drops, (size_t)n)) != cudaSuccess)
         return bad(e, "cudaMalloc");
     if ((e = cudaMallocHost(&c->h_obs, sizeof(double) * (32 + (size_t)n))) != cudaSuccess ||
@@ -955,6 +1066,8 @@ int iblb_batch_create(int n, const iblb_lattice_desc *lat, const iblb_physics_de
     if ((e = cudaMallocHost(&c->h_status, sizeof(int) * 4 * n)) != cudaSuccess)
         return bad(e, "cudaMallocHost");
     A.drops = c->d_drops;
+    A.grp = c->d_grp;
+    A.lbc = c->d_lbc;
     cudaStream_t s = c->stream;
     const uint32_t one = 1;
     if ((e = cudaMemsetAsync(A.tile_gen, 0, sizeof(uint32_t) * T, s)) != cudaSuccess ||
@@ -973,10 +1086,8 @@ int iblb_batch_create(int n, const iblb_lattice_desc *lat, const iblb_physics_de
         (e = cudaMemsetAsync(A.F, 0, sizeof(float) * 3 * A.total_pcells, s)) != cudaSuccess ||
         (e = cudaMemsetAsync(A.U, 0, sizeof(float4) * A.total_pcells, s)) != cudaSuccess ||
         (e = launch_init_populations(A, c->storage, c->fbuf[0], s)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(c->d_drops, c->drops.data(), sizeof(Drop) * n, cudaMemcpyHostToDevice, s)) !=
-            cudaSuccess ||
-        (e = cudaStreamSynchronize(s)) != cudaSuccess)
-        return bad(e, "initialisation");
+        upload_drops(c) != IBLB_OK || (e = cudaStreamSynchronize(s)) != cudaSuccess)
+        return bad(e != cudaSuccess ? e : cudaErrorUnknown, "initialisation");
     *out = c;
     return IBLB_OK;
 }
@@ -1020,6 +1131,8 @@ void iblb_destroy(iblb_ctx *c)
     dfree(A.status);
     dfree(c->d_mass);
     dfree(c->d_drops);
+    dfree(c->d_grp);
+    dfree(c->d_lbc);
     dfree(c->obs_scr);
     if (c->h_status)
         cudaFreeHost(c->h_status);
@@ -1517,6 +1630,7 @@ int iblb_set_option(iblb_ctx *c, int option, int value)
         int r = ensure_ready(c);
         if (r)
             return r;
+        c->auto_cells = false;
         c->cfg.lb_group_cells = value;
         layout(c);
         invalidate_graphs(c);
@@ -1531,6 +1645,7 @@ int iblb_set_option(iblb_ctx *c, int option, int value)
         if (r)
             return r;
         c->cfg.lb_row_mult = value;
+        c->auto_cells = false;
         c->cfg.lb_group_cells = 0;             // the multiplier takes over
         layout(c);
         invalidate_graphs(c);
@@ -1570,6 +1685,7 @@ int iblb_set_option(iblb_ctx *c, int option, int value)
     case IBLB_OPT_LB_STAGES:
         if (value < 2 || value > 8)
             return fail(c, IBLB_E_ARG, "pipeline stages must be in [2, 8]");
+        c->auto_stages = false;
         c->cfg.lb_stages = value;
         fit_stages(c);
         invalidate_graphs(c);
@@ -1656,6 +1772,7 @@ int iblb_autotune(iblb_ctx *c, const char *cache_path)
     cudaEvent_t e0 = ev.e[0], e1 = ev.e[1];
     Entered entered_(c);
     int bs = c->cfg.lb_stages;
+    c->auto_cells = c->auto_stages = false;
     // group sizes of 256 .. 1024 cells in steps of 128 (whole rows), with
     // every pipeline depth and both residencies whose stages fit
     for (int cells = 256; cells <= 1024; cells += 128)

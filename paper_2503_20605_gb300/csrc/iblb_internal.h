@@ -44,9 +44,7 @@ struct Drop {
     int64_t pcell0, pcells;        // population planes: first padded cell, pitch*ny*nzf
     int64_t row0;                  // first row (y + ny z) in the pooled row arrays
     int node0, nnodes, tri0, ntri;
-    int lb_block0, lb_nblocks;     // row groups of the stream-collide launch
-    int lb_rows;                   // cell rows per group (consecutive y of one z-plane)
-    int lb_gpp;                    // groups per z-plane: ceil(ny / lb_rows)
+    int lb_rows;                   // cell rows per stream-collide group (consecutive y of one z-plane)
     int mass_block0, mass_nblocks; // blocks of the mass reduction
     int red_chunk0, red_nchunks;   // chunks of the mesh reductions
     float tau_out, tau_in, omega_out, omega_in;
@@ -58,6 +56,23 @@ struct Drop {
     double V0, R0;
     double inv_n, inv6V0;          // 1 / nnodes and 1 / (6 V0): the volume correction's fold multiplies
 };
+
+// A droplet's constants of the stream-collide kernel: with several droplets
+// they travel with every group's data into shared memory (one 128-byte copy),
+// so that a block that moves to another droplet waits for nothing.
+struct __align__(16) LbConst {
+    int nx, ny, P, R;              // P: row pitch, R: rows per group
+    int PC, nzf, walls, vartau;    // PC: cells per population plane
+    int npr, step_r, step_x, tx;   // work items per row and pitch (cells, or pairs of 16-bit cells); the stride of
+    int ty;                        // a thread's items in rows and items; tiles per row and column
+    float inv_npr;                 // 1 / npr
+    float bfx, bfy;
+    float bfz, rho0, omega_out, omega_in;
+    int64_t pcell0, col0;
+    int64_t tile0, trow0;
+    int has_bf, spare[3];
+};
+static_assert(sizeof(LbConst) == 128, "copied in one piece");
 
 // Record written per node by the force kernel and read by the spread and
 // the interpolation: base cell of the 4^3 support (fluid coordinates, x and
@@ -83,7 +98,9 @@ struct Arrays {
     int64_t total_cells;
     int64_t total_tiles;
     int total_nodes, total_tri;
-    int lb_blocks_total;           // sum of Drop::lb_nblocks (row groups)
+    int lb_blocks_total;           // row groups of the stream-collide launch
+    const int4 *grp;               // per group: droplet, first row y0, plane z, rows
+    const LbConst *lbc;            // per droplet
     int lb_stage_bytes;            // bytes of one shared-memory stage of the stream-collide kernel
     int64_t total_pcells;          // sum of Drop::pcells
     int64_t total_rows;            // sum of ny * nzf
@@ -224,8 +241,12 @@ struct LaunchCfg {
 };
 int lb_rows_per_group(int nx);     // 256-thread groups: max(1, 256 / nx) rows
 // bytes of one stage of the stream-collide kernel: 19 population rows and 3
-// force rows per cell row and the band flag (128-byte multiple)
-int lb_stage_bytes(int rows, int pitch, int storage_bytes);
+// force rows per cell row, the group's header and with several droplets its
+// droplet's constants (128-byte multiple)
+int lb_stage_bytes(int rows, int pitch, int storage_bytes, bool several);
+// work items per row and consumer threads per block, for LbConst
+int lb_items_per_row(int pitch, int storage_bytes);
+int lb_consumers(int storage_bytes);
 
 // Stream-collide over every group (list == nullptr) or over the groups
 // list[0 .. *count); no_force: the groups carry no force (skip the band test).

@@ -20,6 +20,11 @@
 // The producer refills a stage as soon as it is empty, so up to ns groups
 // are in flight, and no consumer warp waits for the others.
 //
+// Rows are written whole, padding included (as zeros): a 32-byte sector that
+// stays partly written costs a read of the rest when it leaves L2.  Twenty
+// 85^3 boxes in FP16 (pitch 88) ran at 3.4 TB/s without the padding's stores,
+// as against 5.3 TB/s for 88^3.
+//
 // Memory traffic per fluid cell: 19 reads + 19 writes of the storage type
 // (152 B for FP32, 76 B for 16-bit storage); the force density is read and
 // the velocity written only on band rows.
@@ -57,20 +62,6 @@ __device__ __forceinline__ void st(float *p, float v) { __stcs(p, v); }
 __device__ __forceinline__ void st(__half *p, float v) { __stcs(p, __float2half_rn(v)); }
 __device__ __forceinline__ void st(__nv_bfloat16 *p, float v) { __stcs(p, __float2bfloat16_rn(v)); }
 
-__device__ __forceinline__ int find_drop_group(const Drop *D, int n, int g)
-{
-    int lo = 0, hi = n - 1;
-    while (lo < hi) {
-        int mid = (lo + hi + 1) >> 1;
-        if (D[mid].lb_block0 <= g)
-            lo = mid;
-        else
-            hi = mid - 1;
-    }
-    return lo;
-}
-
-
 __constant__ int kCy[Q] = {0, 0, 0, 1, -1, 0, 0, 1, -1, -1, 1, 1, -1, 1, -1, 0, 0, 0, 0};
 __constant__ int kCz[Q] = {0, 0, 0, 0, 0, 1, -1, 0, 0, 0, 0, 1, -1, -1, 1, 1, -1, -1, 1};
 __constant__ int kOpp[Q] = {0, 2, 1, 4, 3, 6, 5, 8, 7, 10, 9, 12, 11, 14, 13, 16, 15, 18, 17};
@@ -84,94 +75,24 @@ constexpr float W0 = 1.0f / 3.0f, W1 = 1.0f / 18.0f, W2 = 1.0f / 36.0f;
 // rounds alike and that gain adds up step after step.
 constexpr float K2 = 1.0f / 12.0f, K1 = (1.0f - 8.0f * K2) * 0.5f;
 
-// stage layout: [19][R][P] populations | [3][R][P] force | band flag
+// stage layout: [19][R][P] populations | [3][R][P] force | header (int4: band
+// flag, droplet, first row y0, rows << 16 | plane z) | with several droplets
+// the group's LbConst
 template <typename S>
 struct Stage {
     S *pop;
     float *F;
-    int *flag;
     __device__ Stage(unsigned char *base, int R, int P)
     {
         pop = reinterpret_cast<S *>(base);
         F = reinterpret_cast<float *>(base + (size_t)R * Q * P * sizeof(S));
-        flag = reinterpret_cast<int *>(reinterpret_cast<unsigned char *>(F) + (size_t)R * 3 * P * sizeof(float));
     }
 };
-
-// rows y0 .. y0 + nr - 1 of plane z in group g of droplet D
-__device__ __forceinline__ void group_rows(const Drop &D, int g, int &y0, int &z, int &nr)
+// the header sits at the same place whatever the droplet's rows and pitch
+__device__ __forceinline__ int4 *stage_header(unsigned char *base, const Arrays &a)
 {
-    const int lg = g - D.lb_block0;
-    z = lg / D.lb_gpp;
-    y0 = (lg - z * D.lb_gpp) * D.lb_rows;
-    nr = min(D.lb_rows, D.ny - y0);
+    return reinterpret_cast<int4 *>(base + a.lb_stage_bytes) - (a.ndrops > 1 ? 9 : 1);
 }
-
-// A droplet's stream-collide constants, loaded once and kept in registers
-// while consecutive groups of the same droplet run (one droplet per launch
-// is the common case), with the thread's first cell (r0, x0) of a group.
-struct DropC {
-    int d, nx, ny, P, R, PC, nzf, walls, vartau, gpp, block0, step_r, step_x, r0, x0;
-    int npr, pstep_r, pstep_x, pr0, px0;   // the same walk over cell pairs (x, x + 1), x even
-    int tx, ty;                            // tiles per row and per plane of tile rows
-    int64_t tile0;
-    float inv_gpp, bfx, bfy, bfz, rho0, omega_out, omega_in;
-    bool has_bf;
-    int64_t pcell0, col0;
-    __device__ __forceinline__ void load(const Drop &D, int dd, int nt)
-    {
-        d = dd;
-        nx = D.nx;
-        ny = D.ny;
-        P = D.pitch;
-        R = D.lb_rows;
-        PC = (int)D.pcells;
-        nzf = D.nzf;
-        walls = D.walls;
-        vartau = D.vartau;
-        gpp = D.lb_gpp;
-        block0 = D.lb_block0;
-        step_r = nt / nx;
-        step_x = nt - step_r * nx;
-        r0 = threadIdx.x / nx;
-        x0 = threadIdx.x - r0 * nx;
-        tx = D.tx;
-        ty = D.ty;
-        tile0 = D.tile0;
-        npr = (nx + 1) >> 1;
-        pstep_r = nt / npr;
-        pstep_x = nt - pstep_r * npr;
-        pr0 = threadIdx.x / npr;
-        px0 = threadIdx.x - pr0 * npr;
-        inv_gpp = 1.0f / (float)gpp;
-        bfx = D.bf[0];
-        bfy = D.bf[1];
-        bfz = D.bf[2];
-        rho0 = D.rho0;
-        omega_out = D.omega_out;
-        omega_in = D.omega_in;
-        has_bf = bfx != 0.0f || bfy != 0.0f || bfz != 0.0f;
-        pcell0 = D.pcell0;
-        col0 = D.col0;
-    }
-    // rows y0 .. y0 + nr - 1 of plane z in group g (as group_rows, without
-    // an integer division: a float estimate of the quotient, corrected once)
-    __device__ __forceinline__ void rows(int g, int &y0, int &z, int &nr) const
-    {
-        const int lg = g - block0;
-        z = (int)((float)lg * inv_gpp);
-        int rem = lg - z * gpp;
-        if (rem < 0) {
-            --z;
-            rem += gpp;
-        } else if (rem >= gpp) {
-            ++z;
-            rem -= gpp;
-        }
-        y0 = rem * R;
-        nr = min(R, ny - y0);
-    }
-};
 
 // Band flags of 32 consecutive groups of a block, one per lane: lane l
 // takes group ig0 + l * stride.  A group carries force iff one of the tile
@@ -185,12 +106,10 @@ __device__ __forceinline__ uint32_t band_ballot(const Arrays &a, const int *list
     const int ig = ig0 + lane * stride;
     bool band = false;
     if (ig < total) {
-        const int g = list ? list[ig] : ig;
-        const Drop &D = a.drops[find_drop_group(a.drops, a.ndrops, g)];
-        int y0, z, nr;
-        group_rows(D, g, y0, z, nr);
-        const int64_t tr0 = D.trow0 + (int64_t)D.ty * (z >> 2);
-        for (int ty = y0 >> 2; ty <= (y0 + nr - 1) >> 2; ++ty)
+        const int4 e = a.grp[list ? list[ig] : ig];
+        const LbConst &c = a.lbc[e.x];
+        const int64_t tr0 = c.trow0 + (int64_t)c.ty * (e.z >> 2);
+        for (int ty = e.y >> 2; ty <= (e.y + e.w - 1) >> 2; ++ty)
             band |= a.rowgen[tr0 + ty] == gen;
     }
     return __ballot_sync(0xffffffffu, band);
@@ -202,10 +121,11 @@ __device__ __forceinline__ uint32_t band_ballot(const Arrays &a, const int *list
 // contiguous in memory except across the periodic y seam: lane i < 19 issues
 // one bulk copy for population i (two at the seam).  If the group carries
 // force (band), lanes 19..21 copy the three force-density components of the
-// group's rows.  Every lane announces the bytes of its own copies on the
-// mbarrier (initialised for 32 arrivals) before issuing them.
+// group's rows; with several droplets lane 22 copies the droplet's constants.
+// Every lane announces the bytes of its own copies on the mbarrier
+// (initialised for 32 arrivals) before issuing them.
 template <typename S>
-__device__ __forceinline__ void produce(const Arrays &a, const DropC &c, const S *src, int y0, int z, int nr,
+__device__ __forceinline__ void produce(const Arrays &a, const LbConst &c, int d, const S *src, int y0, int z, int nr,
                                         unsigned char *sbase, uint64_t *bar, bool band)
 {
     const int lane = threadIdx.x & 31;
@@ -240,9 +160,12 @@ __device__ __forceinline__ void produce(const Arrays &a, const DropC &c, const S
         mine = rowb * (uint32_t)(n_a + n_b);
     } else if (band && lane < Q + 3) {
         mine = (uint32_t)(nr * P * sizeof(float));
+    } else if (lane == Q + 3 && a.ndrops > 1) {
+        mine = sizeof(LbConst);
     }
+    int4 *header = stage_header(sbase, a);
     if (lane == 0)
-        *stg.flag = band;
+        *header = make_int4(band, d, y0, (nr << 16) | z);
     mbar_arrive_expect_tx(bar, mine);
     if (lane < Q) {
         const S *plane = src + (int64_t)Q * c.pcell0 + (int64_t)src_pop * c.PC + (int64_t)P * ny * src_z;
@@ -256,6 +179,8 @@ __device__ __forceinline__ void produce(const Arrays &a, const DropC &c, const S
         const int k = lane - Q;
         bulk_g2s(stg.F + (int64_t)k * R * P, a.F + k * a.total_pcells + c.pcell0 + (int64_t)P * (plane_row0 + y0),
                  (uint32_t)(nr * P * sizeof(float)), bar);
+    } else if (lane == Q + 3 && a.ndrops > 1) {
+        bulk_g2s(header + 1, a.lbc + d, sizeof(LbConst), bar);
     }
 }
 
@@ -274,13 +199,17 @@ __device__ __forceinline__ void produce(const Arrays &a, const DropC &c, const S
 // F = 0, so a cell's result does not depend on which group shape holds it.
 // the cell's tile is in this step's band: its velocity is read by the
 // interpolation (every node's kernel support lies in band tiles)
-__device__ __forceinline__ bool in_band_tile(const Arrays &a, const DropC &c, int x, int y, int z, uint32_t gen)
+__device__ __forceinline__ bool in_band_tile(const Arrays &a, const LbConst &c, int x, int y, int z, uint32_t gen)
 {
     return a.tile_gen[c.tile0 + (x >> 2) + (int64_t)c.tx * ((y >> 2) + (int64_t)c.ty * (z >> 2))] == gen;
 }
 
+// row of work item e of a group (e < 2^20, so that the product's error stays
+// below the half added)
+__device__ __forceinline__ int item_row(int e, float inv_npr) { return (int)(((float)e + 0.5f) * inv_npr); }
+
 template <typename S, bool VARTAU, bool FORCE>
-__device__ __forceinline__ void collide_group(const Arrays &a, const DropC &c, const Stage<S> &stg, int y0, int z,
+__device__ __forceinline__ void collide_group(const Arrays &a, const LbConst &c, const Stage<S> &stg, int y0, int z,
                                               int nr, bool band, S *__restrict__ dst, uint32_t gen)
 {
     const int nx = c.nx, ny = c.ny, P = c.P, R = c.R;
@@ -297,15 +226,21 @@ __device__ __forceinline__ void collide_group(const Arrays &a, const DropC &c, c
     float4 *U = a.U;
     // cell e = r * nx + x of the group, walked without divisions
     const int step_r = c.step_r, step_x = c.step_x;
-    int r = c.r0, x = c.x0;
+    int r = item_row(threadIdx.x, c.inv_npr), x = threadIdx.x - r * P;
     for (; r < nr; r += step_r, x += step_x) {
-        if (x >= nx) {
-            x -= nx;
+        if (x >= P) {
+            x -= P;
             ++r;
             if (r >= nr)
                 break;
         }
         const int y = y0 + r;
+        S *o = outb + P * y + x;
+        if (x >= nx) {      // the row's padding (see the file's head)
+            for (int i = 0; i < Q; ++i)
+                st(o + i * PC, 0.0f);
+            continue;
+        }
         float Fx = 0.0f, Fy = 0.0f, Fz = 0.0f;
         if (FORCE) {
             Fx = bfx;
@@ -378,7 +313,6 @@ __device__ __forceinline__ void collide_group(const Arrays &a, const DropC &c, c
         float X = omega * fmaf(-1.5f * rho, fmaf(ux, ux, fmaf(uy, uy, uz * uz)), drho);
         if (FORCE)
             X = fmaf(-3.0f * k, fmaf(ux, Fx, fmaf(uy, Fy, uz * Fz)), X);
-        S *o = outb + P * y + x;
         st(o, fmaf(om1, s0, W0 * X));
         // per weight class: b = w X, ea = 9/2 w omega rho, kf = 9 w k for the
         // even part; the odd part takes 3 w omega rho (c.U) + 3 w k (c.F) as
@@ -500,7 +434,7 @@ __device__ __forceinline__ void bgk_guo_cell(const float (&s)[Q], float Fx, floa
 // omega of cell (x, y, z) of a droplet with variable tau: tau_in iff an odd
 // number of the column's ray crossings lie below the cell (the in/out test)
 template <bool VARTAU>
-__device__ __forceinline__ float cell_omega(const Arrays &a, const DropC &c, int x, int y, int z)
+__device__ __forceinline__ float cell_omega(const Arrays &a, const LbConst &c, int x, int y, int z)
 {
     float omega = c.omega_out;
     if (VARTAU && c.vartau) {
@@ -521,7 +455,7 @@ __device__ __forceinline__ float cell_omega(const Arrays &a, const DropC &c, int
 // more change from group to group (a rotation by kk times the remainder),
 // so that no warp is always the last to release a stage.
 template <typename S, bool VARTAU, bool FORCE>
-__device__ __forceinline__ void collide_pairs(const Arrays &a, const DropC &c, const Stage<S> &stg, int y0, int z,
+__device__ __forceinline__ void collide_pairs(const Arrays &a, const LbConst &c, const Stage<S> &stg, int y0, int z,
                                               int nr, bool band, S *__restrict__ dst, int kk, uint32_t gen)
 {
     using PT = typename PairOf<S>::T;
@@ -534,17 +468,12 @@ __device__ __forceinline__ void collide_pairs(const Arrays &a, const DropC &c, c
     const int RP = R * P;
     S *outb = dst + (int64_t)Q * pcell0 + (int64_t)P * ny * z;
     float4 *U = a.U;
-    const int npr = c.npr, step_r = c.pstep_r, step_x = c.pstep_x;
-    int r = c.pr0, px = c.px0;
-    constexpr int NT = cons_threads<S>();
-    const int extra = (nr * npr) % NT;
-    if (extra) {
-        int e0 = threadIdx.x + (int)(((int64_t)kk * extra) % NT);
-        if (e0 >= NT)
-            e0 -= NT;
-        r = e0 / npr;
-        px = e0 - r * npr;
-    }
+    const int npr = c.npr, step_r = c.step_r, step_x = c.step_x;
+    constexpr unsigned NT = cons_threads<S>();
+    unsigned e0 = threadIdx.x + (unsigned)kk * ((unsigned)(nr * npr) % NT) % NT;
+    if (e0 >= NT)
+        e0 -= NT;
+    int r = item_row(e0, c.inv_npr), px = e0 - r * npr;
     for (; r < nr; r += step_r, px += step_x) {
         if (px >= npr) {
             px -= npr;
@@ -553,6 +482,8 @@ __device__ __forceinline__ void collide_pairs(const Arrays &a, const DropC &c, c
                 break;
         }
         const int x = 2 * px, y = y0 + r;
+        S *o = outb + P * y + x;
+        const bool hasA = x < nx;                  // else the row's padding: zeros (see the file's head)
         const bool hasB = x + 1 < nx;              // an odd row ends on a single cell
         const int xm = x ? x - 1 : nx - 1;         // source of the +x populations of cell x
         const int xp2 = x + 2 < nx ? x + 2 : x + 2 - nx;   // source of the -x populations of cell x + 1
@@ -567,7 +498,7 @@ __device__ __forceinline__ void collide_pairs(const Arrays &a, const DropC &c, c
             FAx = FBx = c.bfx;
             FAy = FBy = c.bfy;
             FAz = FBz = c.bfz;
-            if (band) {     // F vanishes outside band tiles
+            if (band) {     // F vanishes outside band tiles (and in the padding)
                 const float *Fr = stg.F + r * P + x;
                 const float2 f0 = *reinterpret_cast<const float2 *>(Fr);
                 const float2 f1 = *reinterpret_cast<const float2 *>(Fr + RP);
@@ -581,10 +512,12 @@ __device__ __forceinline__ void collide_pairs(const Arrays &a, const DropC &c, c
             }
         }
         const int64_t cell = (int64_t)P * (y + (int64_t)ny * z) + x;
-        S *o = outb + P * y + x;
-        const bool ub = FORCE && band && in_band_tile(a, c, x, y, z, gen);   // both cells share the tile
-        float oa[Q];
-        {   // cell x: c_x = 0 from the pair's low half, +x from x - 1, -x from the pair's high half
+        const bool ub = FORCE && band && hasA && in_band_tile(a, c, x, y, z, gen);   // both cells share the tile
+        float oa[Q], ob[Q];
+#pragma unroll
+        for (int i = 0; i < Q; ++i)
+            oa[i] = ob[i] = 0.0f;
+        if (hasA) {   // cell x: c_x = 0 from the pair's low half, +x from x - 1, -x from the pair's high half
             float sa[Q];
             sa[0] = PO::lo(pv[0]);
             sa[3] = PO::lo(pv[3]);
@@ -614,7 +547,7 @@ __device__ __forceinline__ void collide_pairs(const Arrays &a, const DropC &c, c
             }
         }
         if (hasB) {  // cell x + 1: c_x = 0 from the high half, +x from the low half, -x from x + 2
-            float sb[Q], ob[Q];
+            float sb[Q];
             sb[0] = PO::hi(pv[0]);
             sb[3] = PO::hi(pv[3]);
             sb[4] = PO::hi(pv[4]);
@@ -640,14 +573,11 @@ __device__ __forceinline__ void collide_pairs(const Arrays &a, const DropC &c, c
                 const int64_t gi = pcell0 + cell + 1;
                 U[gi] = make_float4(ux, uy, uz, 0.0f);
             }
-#pragma unroll
-            for (int i = 0; i < Q; ++i)
-                __stcs(reinterpret_cast<PT *>(o + (int64_t)i * PC), PO::pack(oa[i], ob[i]));
-        } else {
-#pragma unroll
-            for (int i = 0; i < Q; ++i)
-                st(o + (int64_t)i * PC, oa[i]);
         }
+        // one store for cells and padding alike, so that sectors go out whole
+#pragma unroll
+        for (int i = 0; i < Q; ++i)
+            __stcs(reinterpret_cast<PT *>(o + (int64_t)i * PC), PO::pack(oa[i], ob[i]));
 #undef SC
     }
 }
@@ -682,15 +612,25 @@ __global__ void __launch_bounds__(lb_block<S>(), 2)
     // soon as its data landed, without waiting for the other warps.
     bool failed = false;
     if (threadIdx.x >= cons_threads<S>()) {
-        int st_i = 0;
+        int st_i = 0, d = -1;
         uint32_t use = 0, bits = 0;
-        DropC c;
-        c.d = -1;
-        for (int ig = blockIdx.x, k = 0; ig < total; ig += gridDim.x, ++k) {
+        LbConst c;
+        const int stride = gridDim.x;
+        int4 next = make_int4(0, 0, 0, 0);
+        if ((int)blockIdx.x < total)
+            next = a.grp[list ? list[blockIdx.x] : blockIdx.x];
+        for (int ig = blockIdx.x, k = 0; ig < total; ig += stride, ++k) {
+            const int4 e = next;
+            if (ig + stride < total)      // the next group's entry arrives while this one is fetched
+                next = a.grp[list ? list[ig + stride] : ig + stride];
             // the band flags of the next 32 groups at once: one round trip
             // to memory per 32 groups, off the path of each group's copies
             if ((k & 31) == 0)
-                bits = no_force ? 0u : band_ballot(a, list, total, ig, gridDim.x, gen);
+                bits = no_force ? 0u : band_ballot(a, list, total, ig, stride, gen);
+            if (e.x != d) {
+                d = e.x;
+                c = a.lbc[d];
+            }
             if (use > 0 && !mbar_wait_bounded(&empty[st_i], (use - 1) & 1u, WAIT_CYCLES)) {
                 failed = true;
                 break;
@@ -698,13 +638,7 @@ __global__ void __launch_bounds__(lb_block<S>(), 2)
             // order the consumers' generic reads of the stage before the
             // asynchronous writes into it
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            const int g = list ? list[ig] : ig;
-            const int d = find_drop_group(a.drops, a.ndrops, g);
-            if (d != c.d)
-                c.load(a.drops[d], d, cons_threads<S>());
-            int y0, z, nr;
-            c.rows(g, y0, z, nr);
-            produce<S>(a, c, src, y0, z, nr, smem_raw + st_i * a.lb_stage_bytes, &full[st_i],
+            produce<S>(a, c, d, src, e.y, e.z, e.w, smem_raw + st_i * a.lb_stage_bytes, &full[st_i],
                        ((bits >> (k & 31)) & 1u) != 0);
             if (++st_i == ns) {
                 st_i = 0;
@@ -712,23 +646,25 @@ __global__ void __launch_bounds__(lb_block<S>(), 2)
             }
         }
     } else {
-        int st_i = 0, kk = 0;
+        int st_i = 0, kk = 0, d = 0;
         uint32_t phase = 0;
-        DropC c;
-        c.d = -1;
+        LbConst c = a.lbc[0];     // one droplet: its constants, for good; several: replaced by a group's own
+        if (a.ndrops > 1)
+            d = -1;
         for (int ig = blockIdx.x; ig < total; ig += gridDim.x, ++kk) {
-            const int g = list ? list[ig] : ig;
-            const int d = find_drop_group(a.drops, a.ndrops, g);
-            if (d != c.d)
-                c.load(a.drops[d], d, cons_threads<S>());
-            int y0, z, nr;
-            c.rows(g, y0, z, nr);
             if (!mbar_wait_bounded(&full[st_i], phase, WAIT_CYCLES)) {
                 failed = true;
                 break;
             }
-            const Stage<S> stg(smem_raw + st_i * a.lb_stage_bytes, c.R, c.P);
-            const bool band = *stg.flag != 0;
+            unsigned char *base = smem_raw + st_i * a.lb_stage_bytes;
+            const int4 h = *stage_header(base, a);
+            if (h.y != d) {
+                d = h.y;
+                c = *reinterpret_cast<const LbConst *>(stage_header(base, a) + 1);
+            }
+            const Stage<S> stg(base, c.R, c.P);
+            const bool band = h.x != 0;
+            const int y0 = h.z, z = h.w & 0xffff, nr = h.w >> 16;
             if constexpr (sizeof(S) == 2) {      // 16-bit storage: two cells per work item
                 if (band || c.has_bf)
                     collide_pairs<S, VARTAU, true>(a, c, stg, y0, z, nr, band, dst, kk, gen);
@@ -796,9 +732,14 @@ cudaError_t launch_t(const Arrays &a, const void *src, void *dst, bool vartau, c
 
 int lb_rows_per_group(int nx) { return nx >= LB_THREADS ? 1 : LB_THREADS / nx; }
 
-int lb_stage_bytes(int rows, int pitch, int sb)
+int lb_items_per_row(int pitch, int sb) { return sb == 2 ? pitch / 2 : pitch; }
+
+int lb_consumers(int sb) { return sb == 2 ? cons_threads<__half>() : cons_threads<float>(); }
+
+int lb_stage_bytes(int rows, int pitch, int sb, bool several)
 {
-    const size_t b = (size_t)rows * Q * pitch * sb + (size_t)rows * 3 * pitch * sizeof(float) + 16;
+    const size_t b = (size_t)rows * Q * pitch * sb + (size_t)rows * 3 * pitch * sizeof(float) + sizeof(int4) +
+                     (several ? sizeof(LbConst) : 0);
     return (int)((b + 127) & ~(size_t)127);
 }
 
@@ -873,10 +814,9 @@ __global__ void __launch_bounds__(256) classify_kernel(Arrays a)
         a.candrow[r] = (!ok || near_band(a, D, ty, ty, tz, gprev)) ? 1 : 0;
     }
     for (int64_t g = gid; g < a.lb_blocks_total; g += stride) {
-        const Drop &D = a.drops[find_drop_group(a.drops, a.ndrops, (int)g)];
-        int y0, z, nr;
-        group_rows(D, (int)g, y0, z, nr);
-        const bool near = !ok || near_band(a, D, y0 >> 2, (y0 + nr - 1) >> 2, z >> 2, gprev);
+        const int4 e = a.grp[g];
+        const Drop &D = a.drops[e.x];
+        const bool near = !ok || near_band(a, D, e.y >> 2, (e.y + e.w - 1) >> 2, e.z >> 2, gprev);
         const int slot = atomicAdd(&a.grp_cnt[near ? 0 : 1], 1);
         a.grp_list[(near ? 0 : a.total_rows) + slot] = (int)g;
     }
