@@ -728,10 +728,35 @@ __device__ void spread_finish(const Arrays &a, uint32_t gen, int cur, SpreadSmem
     }
 }
 
+// 4 x 4 transpose over four consecutive lanes: v[i] of lane j <-> v[j] of lane i
+__device__ __forceinline__ void transpose4(float (&v)[4])
+{
+    const bool b0 = threadIdx.x & 1, b1 = threadIdx.x & 2;
+#pragma unroll
+    for (int i = 0; i < 4; i += 2) {
+        const float got = __shfl_xor_sync(0xffffffffu, b0 ? v[i] : v[i + 1], 1);
+        v[i] = b0 ? got : v[i];
+        v[i + 1] = b0 ? v[i + 1] : got;
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const float got = __shfl_xor_sync(0xffffffffu, b1 ? v[i] : v[i + 2], 2);
+        v[i] = b1 ? got : v[i];
+        v[i + 2] = b1 ? v[i + 2] : got;
+    }
+}
+
 // Interpolation and advection of the IB_THREADS / 16 nodes of one block
 // (base: the global index of its thread 0, a multiple of IB_THREADS).
-// 16 lanes per node: lane l covers support row (dy, dz) = (l & 3, l >> 2)
-// and the four cells of that row; partial sums meet in a fixed shuffle tree.
+// 16 lanes per node.  Lane (y, k) = (l >> 2, l & 3) loads the cells x = k of
+// the support rows (y, z), z = 0 .. 3: a warp's load covers eight rows of 64
+// consecutive bytes (one lane per row, as the sums want it, touches 32 lines
+// a load and L1 was what bound the kernel: 0.90 of its throughput).  A 4 x 4
+// transpose over the four lanes of a row then gives lane (y, k) the whole row
+// (y, z = k), whose four cells it adds in order; the rows meet in a fixed
+// shuffle tree.  Measured in the step: 10 242 nodes 5.5 -> 4.3 us, 163 842
+// nodes 50 -> 41 us, 250 368 nodes in 64 boxes 75 -> 66 us (now L2 latency and
+// issue in equal parts; 40 or 32 registers for more warps: no gain).
 // The FP64 advection then runs on the block's first 3 IB_THREADS / 16
 // threads, one coordinate each, so that its FP64 operations fill whole
 // warps (on this GPU they issue at a small fraction of the FP32 rate); each
@@ -748,36 +773,49 @@ __device__ __forceinline__ void interp_block(const Arrays &a, int64_t base)
     double q = 0.0;
     if (adv)
         q = (an == 0 ? a.px : (an == 1 ? a.py : a.pz))[jn];
-    float ax = 0.f, ay = 0.f, az = 0.f;
     int d = 0;
+    float ux[4] = {0.f, 0.f, 0.f, 0.f}, uy[4] = {0.f, 0.f, 0.f, 0.f}, uz[4] = {0.f, 0.f, 0.f, 0.f};
+    float4 wx = make_float4(0.f, 0.f, 0.f, 0.f);
+    float wyz = 0.f;
     if (valid) {
         d = a.ndrops == 1 ? 0 : a.node_drop[j];
         const NodeRec &r = a.rec[j];
         const Drop &D = a.drops[d];
-        if (r.key > 0) {
-            const int dy = l & 3, dz = l >> 2;
-            int Z = r.bz - 1 + dz;
-            bool fluid = true;
-            if (D.walls)
-                fluid = Z >= 0 && Z < D.nzf;
-            else
-                Z = wrapi(Z, D.nzf);
-            if (fluid) {
-                const int Y = wrapi(r.by - 1 + dy, D.ny);
-                const float wyz = r.wy[dy] * r.wz[dz];
-                const int64_t row = D.pcell0 + (int64_t)D.pitch * (Y + (int64_t)D.ny * Z);
-                for (int dx = 0; dx < 4; ++dx) {
-                    const int64_t g = row + wrapi(r.bx - 1 + dx, D.nx);
-                    const float w = r.wx[dx] * wyz;
-                    const float4 u = a.U[g];
-                    ax = fmaf(u.x, w, ax);
-                    ay = fmaf(u.y, w, ay);
-                    az = fmaf(u.z, w, az);
+        const int4 base4 = *reinterpret_cast<const int4 *>(&r);      // bx, by, bz, key
+        if (base4.w > 0) {
+            const int y = l >> 2, k = l & 3;
+            wx = *reinterpret_cast<const float4 *>(r.wx);
+            wyz = r.wy[y] * r.wz[k];
+            const int X = wrapi(base4.x - 1 + k, D.nx), Y = wrapi(base4.y - 1 + y, D.ny);
+            const int64_t at = D.pcell0 + X + (int64_t)D.pitch * Y, plane = (int64_t)D.pitch * D.ny;
+#pragma unroll
+            for (int z = 0; z < 4; ++z) {
+                int Z = base4.z - 1 + z;
+                if (!D.walls)
+                    Z = wrapi(Z, D.nzf);
+                if (Z >= 0 && Z < D.nzf) {       // cells outside the fluid supply U = 0
+                    const float4 u = a.U[at + plane * Z];
+                    ux[z] = u.x;
+                    uy[z] = u.y;
+                    uz[z] = u.z;
                 }
             }
         }
     }
-    for (int o = 8; o >= 1; o >>= 1) {
+    transpose4(ux);
+    transpose4(uy);
+    transpose4(uz);
+    float ax = 0.f, ay = 0.f, az = 0.f;
+#pragma unroll
+    for (int x = 0; x < 4; ++x) {
+        const float w = (&wx.x)[x] * wyz;
+        ax = fmaf(ux[x], w, ax);
+        ay = fmaf(uy[x], w, ay);
+        az = fmaf(uz[x], w, az);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int o = i == 0 ? 2 : (i == 1 ? 1 : (i == 2 ? 8 : 4));      // z (lanes' low bits), then y
         ax += __shfl_xor_sync(0xffffffffu, ax, o);
         ay += __shfl_xor_sync(0xffffffffu, ay, o);
         az += __shfl_xor_sync(0xffffffffu, az, o);
