@@ -63,6 +63,7 @@ struct iblb_ctx {
     std::vector<int4> grp;         // stream-collide groups and constants of the current layout
     std::vector<LbConst> lbc;
     bool grp_dirty = true;         // not yet on the device
+    int64_t mask_bytes = 0;        // inside bits of every droplet with two viscosities
     int4 *d_grp = nullptr;
     LbConst *d_lbc = nullptr;
     void *fbuf[2] = {nullptr, nullptr};
@@ -361,6 +362,9 @@ void fit_stages(iblb_ctx *c)
         --c->cfg.lb_stages;
 }
 
+// bytes per row of a droplet's inside bits
+int mask_pitch(const Drop &D) { return D.vartau ? (D.nx + 127) / 128 * 16 : 0; }
+
 // rows per stream-collide group for about `cells` cells, of ny rows of pitch P
 int rows_for(int cells, const Drop &D) { return std::min(D.ny, std::max(1, (cells + D.nx / 2) / D.nx)); }
 
@@ -390,7 +394,7 @@ void pick_shape(iblb_ctx *c)
             for (const Drop &D : c->drops) {
                 const int P = (D.nx * sb + 15) / 16 * 16 / sb, gpp = (D.ny - 1) / rows_for(cells, D) + 1;
                 const int rows = (D.ny - 1) / gpp + 1;
-                stage = std::max(stage, (int64_t)lb_stage_bytes(rows, P, sb, c->ndrops > 1));
+                stage = std::max(stage, (int64_t)lb_stage_bytes(rows, P, sb, c->ndrops > 1, mask_pitch(D)));
                 groups += (int64_t)gpp * D.nzf;
                 work += (double)D.nzf * ((double)gpp * kGroupCells + (double)D.ny * P);
                 largest = std::max(largest, (double)rows * P + kGroupCells);
@@ -427,7 +431,8 @@ void layout(iblb_ctx *c)
 {
     if (c->auto_cells)
         pick_shape(c);
-    int64_t cell0 = 0, tile0 = 0, col0 = 0, pcell0 = 0, row0 = 0, trow0 = 0;
+    int64_t cell0 = 0, tile0 = 0, col0 = 0, pcell0 = 0, row0 = 0, trow0 = 0, mask0 = 0;
+    int mask_cols = 0;
     int mb0 = 0, stage = 0;
     const int sb = (int)storage_bytes(c->storage);
     const bool several = c->ndrops > 1;
@@ -444,12 +449,18 @@ void layout(iblb_ctx *c)
         const int align = 16 / sb;
         D.pitch = (D.nx + align - 1) / align * align;
         D.pcells = (int64_t)D.pitch * D.ny * D.nzf;
+        D.mask_pitch = mask_pitch(D);
+        D.mask0 = mask0;
+        D.mask_col0 = mask_cols;
+        mask0 += (int64_t)D.mask_pitch * D.ny * D.nzf;
+        mask_cols += D.mask_pitch / 4 * D.ny;
         D.pcell0 = pcell0;
         D.row0 = row0;
         D.lb_rows = c->cfg.lb_group_cells > 0 ? rows_for(c->cfg.lb_group_cells, D)
                                               : std::min(D.ny, c->cfg.lb_row_mult * lb_rows_per_group(D.nx));
         // two stages of the group must fit the opt-in shared memory of a block
-        while (D.lb_rows > 1 && 2 * (int64_t)lb_stage_bytes(D.lb_rows, D.pitch, sb, several) > kLbSmemOptin)
+        while (D.lb_rows > 1 &&
+               2 * (int64_t)lb_stage_bytes(D.lb_rows, D.pitch, sb, several, D.mask_pitch) > kLbSmemOptin)
             --D.lb_rows;
         // as many groups a plane, their rows as even as they go: a short last
         // group would fall to the same blocks in every round
@@ -482,14 +493,15 @@ void layout(iblb_ctx *c)
         k.omega_out = D.omega_out;
         k.omega_in = D.omega_in;
         k.pcell0 = D.pcell0;
-        k.col0 = D.col0;
+        k.mask0 = D.mask0;
+        k.mask_pitch = D.mask_pitch;
         k.tile0 = D.tile0;
         k.trow0 = D.trow0;
         k.has_bf = D.bf[0] != 0.0f || D.bf[1] != 0.0f || D.bf[2] != 0.0f;
         c->lbc.push_back(k);
         D.mass_block0 = mb0;
         D.mass_nblocks = (int)((D.cells + MASS_CELLS_PER_BLOCK - 1) / MASS_CELLS_PER_BLOCK);
-        stage = std::max(stage, lb_stage_bytes(D.lb_rows, D.pitch, sb, several));
+        stage = std::max(stage, lb_stage_bytes(D.lb_rows, D.pitch, sb, several, D.mask_pitch));
         cell0 += D.cells;
         pcell0 += D.pcells;
         row0 += (int64_t)D.ny * D.nzf;
@@ -504,6 +516,8 @@ void layout(iblb_ctx *c)
     c->A.total_tiles = tile0;
     c->A.total_trows = trow0;
     c->A.total_cols = col0;
+    c->A.total_mask_cols = mask_cols;
+    c->mask_bytes = mask0;
     c->A.lb_blocks_total = (int)c->grp.size();
     c->A.lb_stage_bytes = stage;
     c->mass_blocks = mb0;
@@ -572,6 +586,10 @@ void free_membrane_arrays(iblb_ctx *c)
     dfree(c->A.qh);
     dfree(c->A.ql);
     c->A.qh = c->A.ql = nullptr;
+    dfree(c->A.ni);
+    dfree(c->A.nf);
+    c->A.ni = nullptr;
+    c->A.nf = nullptr;
     dfree(c->A.node_drop);
     dfree(c->d_tri);
     dfree(c->A.face_drop);
@@ -682,6 +700,10 @@ int rebuild_membranes(iblb_ctx *c)
     CK(dalloc(&c->A.pz, N));
     CK(dalloc(&c->A.qh, N));
     CK(dalloc(&c->A.ql, N));
+    if (c->any_vartau) {
+        CK(dalloc(&c->A.ni, N));
+        CK(dalloc(&c->A.nf, N));
+    }
     CK(dalloc(&c->A.node_drop, N));
     CK(dalloc(&c->d_tri, 3 * (size_t)NT));
     CK(dalloc(&c->A.face_drop, NT));
@@ -1052,8 +1074,10 @@ int iblb_batch_create(int n, const iblb_lattice_desc *lat, const iblb_physics_de
         (e = dalloc(&A.candrow, (size_t)A.total_trows)) != cudaSuccess ||
         (e = dalloc(&A.grp_list, 2 * (size_t)A.total_rows)) != cudaSuccess ||
         (e = dalloc(&A.grp_cnt, 3)) != cudaSuccess || (e = dalloc(&A.split_ok, 1)) != cudaSuccess ||
-        (e = dalloc(&A.col_cnt, (size_t)A.total_cols)) != cudaSuccess ||
-        (e = dalloc(&A.col_z, (size_t)A.total_cols * MAXC)) != cudaSuccess ||
+        (e = dalloc(&A.col_cnt, c->any_vartau ? (size_t)A.total_cols : 1)) != cudaSuccess ||
+        (e = dalloc(&A.col_t, c->any_vartau ? (size_t)A.total_cols * MAXC : 1)) != cudaSuccess ||
+        (e = dalloc(&A.mask, (size_t)c->mask_bytes)) != cudaSuccess ||
+        (e = dalloc(&A.mask_any, (size_t)A.total_mask_cols)) != cudaSuccess ||
         (e = dalloc(&A.mass_part, (size_t)c->mass_blocks)) != cudaSuccess ||
         (e = dalloc(&A.status, 4 * (size_t)n)) != cudaSuccess ||
         (e = dalloc(&c->d_grp, (size_t)A.total_rows)) != cudaSuccess ||
@@ -1081,7 +1105,9 @@ int iblb_batch_create(int n, const iblb_lattice_desc *lat, const iblb_physics_de
         (e = cudaMemsetAsync(A.grp_cnt, 0, 3 * sizeof(int), s)) != cudaSuccess ||
         (e = cudaMemsetAsync(A.split_ok, 0, sizeof(int), s)) != cudaSuccess ||
         (e = cudaMemsetAsync(A.bin_cnt, 0, sizeof(int) * T, s)) != cudaSuccess ||
-        (e = cudaMemsetAsync(A.col_cnt, 0, sizeof(int) * A.total_cols, s)) != cudaSuccess ||
+        (e = cudaMemsetAsync(A.col_cnt, 0, sizeof(int) * (c->any_vartau ? A.total_cols : 1), s)) != cudaSuccess ||
+        (e = cudaMemsetAsync(A.mask, 0, c->mask_bytes, s)) != cudaSuccess ||
+        (e = cudaMemsetAsync(A.mask_any, 0, A.total_mask_cols, s)) != cudaSuccess ||
         (e = cudaMemsetAsync(A.status, 0, sizeof(int) * 4 * n, s)) != cudaSuccess ||
         (e = cudaMemsetAsync(A.F, 0, sizeof(float) * 3 * A.total_pcells, s)) != cudaSuccess ||
         (e = cudaMemsetAsync(A.U, 0, sizeof(float4) * A.total_pcells, s)) != cudaSuccess ||
@@ -1126,7 +1152,9 @@ void iblb_destroy(iblb_ctx *c)
     dfree(A.grp_cnt);
     dfree(A.split_ok);
     dfree(A.col_cnt);
-    dfree(A.col_z);
+    dfree(A.col_t);
+    dfree(A.mask);
+    dfree(A.mask_any);
     dfree(A.mass_part);
     dfree(A.status);
     dfree(c->d_mass);

@@ -123,13 +123,8 @@ __global__ void inside_kernel(Arrays a, int d, uint8_t *inside)
     const int ci = (int)c;
     const int x = ci % D.nx, y = (ci / D.nx) % D.ny, z = ci / (D.nx * D.ny);
     int par = 0;
-    if (D.vartau) {
-        const int64_t col = D.col0 + x + (int64_t)D.nx * y;
-        const int cnt = min(a.col_cnt[col], MAXC);
-        const double Z = (double)(z + D.walls);
-        for (int k = 0; k < cnt; ++k)
-            par ^= a.col_z[col * MAXC + k] < Z;
-    }
+    if (D.vartau)
+        par = (a.mask[D.mask0 + D.mask_pitch * (y + (int64_t)D.ny * z) + (x >> 3)] >> (x & 7)) & 1;
     inside[c] = (uint8_t)par;
 }
 

@@ -298,9 +298,15 @@ __device__ __forceinline__ void node_forces(const Arrays &a, int64_t gid, uint32
                       __shfl_sync(0xffffffffu, sane_l, qb | 2);
     int b = 0, nt = 0, t0 = -1, t1 = -1, t2 = -1;
     float w[4] = {0.f, 0.f, 0.f, 0.f};
+    if (a.ni && valid && l == 3)
+        a.ni[j].w = sane ? 1 : 0;
     if (valid && l < 3 && sane) {
         const double fb = floor(q);
         const float f = dtof_rn(q - fb);
+        if (a.ni) {     // for the in/out test
+            (&a.ni[j].x)[ax] = (int)fb;
+            (&a.nf[j].x)[ax] = f;
+        }
         const int n = ax == 0 ? D.nx : (ax == 1 ? D.ny : D.nzf);
         if (ax < 2) {
             b = wrapi((int)fb % n, n);
@@ -1128,6 +1134,13 @@ __global__ void __launch_bounds__(IB_THREADS) corrected_positions_kernel(Arrays 
     a.px[j] = x;
     a.py[j] = y;
     a.pz[j] = z;
+    if (a.ni) {
+        const bool sane = fabs(x) < 1e8 && fabs(y) < 1e8 && fabs(z) < 1e8;
+        const double fx = floor(x), fy = floor(y), fz = floor(z);
+        a.ni[j] = sane ? make_int4((int)fx, (int)fy, (int)fz, 1) : make_int4(0, 0, 0, 0);
+        a.nf[j] = sane ? make_float4(dtof_rn(x - fx), dtof_rn(y - fy), dtof_rn(z - fz), 0.0f)
+                       : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
     if (xyz && j >= node0 && j < node0 + n) {
         double *o = xyz + 3 * (int64_t)(j - node0);
         o[0] = x;

@@ -40,6 +40,8 @@ struct Drop {
     int64_t tile0;                 // first tile in the pooled tile arrays
     int64_t trow0;                 // first tile row (ty + tyc * tz) in the pooled tile-row arrays
     int64_t col0;                  // first column (nx*ny per droplet)
+    int64_t mask0;                 // inside bits: first byte; row (y, z) at mask0 + mask_pitch (y + ny z)
+    int mask_pitch, mask_col0;     // bytes per row (a multiple of 16; 0: one viscosity), first word column
     int pitch;                     // population row pitch: nx rounded up to 16 elements
     int64_t pcell0, pcells;        // population planes: first padded cell, pitch*ny*nzf
     int64_t row0;                  // first row (y + ny z) in the pooled row arrays
@@ -68,9 +70,9 @@ struct __align__(16) LbConst {
     float inv_npr;                 // 1 / npr
     float bfx, bfy;
     float bfz, rho0, omega_out, omega_in;
-    int64_t pcell0, col0;
+    int64_t pcell0, mask0;
     int64_t tile0, trow0;
-    int has_bf, spare[3];
+    int has_bf, mask_pitch, spare[2];
 };
 static_assert(sizeof(LbConst) == 128, "copied in one piece");
 
@@ -148,9 +150,14 @@ struct Arrays {
                                    // the force kernel needs no adj_start lookup first
     NodeRec *rec;                  // total_nodes
     // in/out
-    int *col_cnt;                  // crossings per column
-    double *col_z;                 // MAXC crossings per column (sorted)
+    int *col_cnt;                  // crossings per column (0 between steps)
+    int *col_t;                    // MAXC crossings per column: the first layer above each (arrival order)
     int64_t total_cols;
+    uint8_t *mask;                 // one bit per cell: inside (rows of Drop::mask_pitch bytes)
+    uint8_t *mask_any;             // per word column: some word is not 0
+    int total_mask_cols;           // 32-column words of one layer, over all droplets with two viscosities
+    int4 *ni;                      // per node: integer parts of its (corrected) position, w = 1 if it is a
+    float4 *nf;                    // sane number, and the fractions; null without a viscosity ratio
     int *face_drop;                // droplet of each face
     const float4 *fref;            // per face, from the mesh given at set-up: S = H^-1 of the
                                    // reference edge Gram matrix H (x = S11, y = S12, z = S22)
@@ -241,9 +248,9 @@ struct LaunchCfg {
 };
 int lb_rows_per_group(int nx);     // 256-thread groups: max(1, 256 / nx) rows
 // bytes of one stage of the stream-collide kernel: 19 population rows and 3
-// force rows per cell row, the group's header and with several droplets its
-// droplet's constants (128-byte multiple)
-int lb_stage_bytes(int rows, int pitch, int storage_bytes, bool several);
+// force rows per cell row, its inside bits with two viscosities, the group's
+// header and with several droplets its droplet's constants (128-byte multiple)
+int lb_stage_bytes(int rows, int pitch, int storage_bytes, bool several, int mask_pitch);
 // work items per row and consumer threads per block, for LbConst
 int lb_items_per_row(int pitch, int storage_bytes);
 int lb_consumers(int storage_bytes);

@@ -75,17 +75,19 @@ constexpr float W0 = 1.0f / 3.0f, W1 = 1.0f / 18.0f, W2 = 1.0f / 36.0f;
 // rounds alike and that gain adds up step after step.
 constexpr float K2 = 1.0f / 12.0f, K1 = (1.0f - 8.0f * K2) * 0.5f;
 
-// stage layout: [19][R][P] populations | [3][R][P] force | header (int4: band
-// flag, droplet, first row y0, rows << 16 | plane z) | with several droplets
+// stage layout: [19][R][P] populations | [3][R][P] force | with two
+// viscosities [R][mask_pitch] inside bits | header (int4: band flag, droplet, first row y0, rows << 16 | plane z) | with several droplets
 // the group's LbConst
 template <typename S>
 struct Stage {
     S *pop;
     float *F;
+    unsigned char *mask;
     __device__ Stage(unsigned char *base, int R, int P)
     {
         pop = reinterpret_cast<S *>(base);
         F = reinterpret_cast<float *>(base + (size_t)R * Q * P * sizeof(S));
+        mask = reinterpret_cast<unsigned char *>(F + (size_t)R * 3 * P);
     }
 };
 // the header sits at the same place whatever the droplet's rows and pitch
@@ -121,10 +123,11 @@ __device__ __forceinline__ uint32_t band_ballot(const Arrays &a, const int *list
 // contiguous in memory except across the periodic y seam: lane i < 19 issues
 // one bulk copy for population i (two at the seam).  If the group carries
 // force (band), lanes 19..21 copy the three force-density components of the
-// group's rows; with several droplets lane 22 copies the droplet's constants.
+// group's rows; with several droplets lane 22 copies the droplet's constants,
+// with two viscosities lane 23 the rows' inside bits.
 // Every lane announces the bytes of its own copies on the mbarrier
 // (initialised for 32 arrivals) before issuing them.
-template <typename S>
+template <typename S, bool VARTAU>
 __device__ __forceinline__ void produce(const Arrays &a, const LbConst &c, int d, const S *src, int y0, int z, int nr,
                                         unsigned char *sbase, uint64_t *bar, bool band)
 {
@@ -162,6 +165,8 @@ __device__ __forceinline__ void produce(const Arrays &a, const LbConst &c, int d
         mine = (uint32_t)(nr * P * sizeof(float));
     } else if (lane == Q + 3 && a.ndrops > 1) {
         mine = sizeof(LbConst);
+    } else if (VARTAU && lane == Q + 4) {
+        mine = (uint32_t)(nr * c.mask_pitch);
     }
     int4 *header = stage_header(sbase, a);
     if (lane == 0)
@@ -181,6 +186,8 @@ __device__ __forceinline__ void produce(const Arrays &a, const LbConst &c, int d
                  (uint32_t)(nr * P * sizeof(float)), bar);
     } else if (lane == Q + 3 && a.ndrops > 1) {
         bulk_g2s(header + 1, a.lbc + d, sizeof(LbConst), bar);
+    } else if (VARTAU && lane == Q + 4 && c.mask_pitch) {
+        bulk_g2s(stg.mask, a.mask + c.mask0 + c.mask_pitch * (plane_row0 + y0), (uint32_t)(nr * c.mask_pitch), bar);
     }
 }
 
@@ -217,8 +224,7 @@ __device__ __forceinline__ void collide_group(const Arrays &a, const LbConst &c,
     const int64_t pcell0 = c.pcell0;
     const float bfx = c.bfx, bfy = c.bfy, bfz = c.bfz, rho0 = c.rho0;
     const float omega_out = c.omega_out, omega_in = c.omega_in;
-    const int vartau = c.vartau, walls = c.walls;
-    const int64_t col0 = c.col0;
+    const int walls = c.walls;
     const bool bbm = walls && z == 0;              // rows pulled from z-1 bounced at the bottom
     const bool bbp = walls && z == c.nzf - 1;      // rows pulled from z+1 bounced at the top
     const int RP = R * P;
@@ -254,14 +260,9 @@ __device__ __forceinline__ void collide_group(const Arrays &a, const LbConst &c,
             }
         }
         float omega = omega_out;
-        if (VARTAU && vartau) {
-            const int64_t col = col0 + x + (int64_t)nx * y;
-            const int cnt = min(a.col_cnt[col], MAXC);
-            const double Z = (double)(z + walls);
-            int par = 0;
-            for (int q = 0; q < cnt; ++q)
-                par ^= a.col_z[col * MAXC + q] < Z;
-            if (par)
+        if (VARTAU && c.mask_pitch) {
+            const uint32_t m = *reinterpret_cast<const uint32_t *>(stg.mask + r * c.mask_pitch + (x >> 5) * 4);
+            if ((m >> (x & 31)) & 1u)
                 omega = omega_in;
         }
         const int xm = x ? x - 1 : nx - 1, xp = x + 1 < nx ? x + 1 : 0;
@@ -431,25 +432,6 @@ __device__ __forceinline__ void bgk_guo_cell(const float (&s)[Q], float Fx, floa
 #undef PAIR
 }
 
-// omega of cell (x, y, z) of a droplet with variable tau: tau_in iff an odd
-// number of the column's ray crossings lie below the cell (the in/out test)
-template <bool VARTAU>
-__device__ __forceinline__ float cell_omega(const Arrays &a, const LbConst &c, int x, int y, int z)
-{
-    float omega = c.omega_out;
-    if (VARTAU && c.vartau) {
-        const int64_t col = c.col0 + x + (int64_t)c.nx * y;
-        const int cnt = min(a.col_cnt[col], MAXC);
-        const double Z = (double)(z + c.walls);
-        int par = 0;
-        for (int q = 0; q < cnt; ++q)
-            par ^= a.col_z[col * MAXC + q] < Z;
-        if (par)
-            omega = c.omega_in;
-    }
-    return omega;
-}
-
 // kk: the block's count of groups so far.  When the group's pairs do not
 // divide evenly among the consumer threads, the threads that take one pair
 // more change from group to group (a rotation by kk times the remainder),
@@ -513,6 +495,12 @@ __device__ __forceinline__ void collide_pairs(const Arrays &a, const LbConst &c,
         }
         const int64_t cell = (int64_t)P * (y + (int64_t)ny * z) + x;
         const bool ub = FORCE && band && hasA && in_band_tile(a, c, x, y, z, gen);   // both cells share the tile
+        float omegaA = c.omega_out, omegaB = c.omega_out;
+        if (VARTAU && c.mask_pitch) {      // x is even: both cells' bits in one word
+            const uint32_t m = *reinterpret_cast<const uint32_t *>(stg.mask + r * c.mask_pitch + (x >> 5) * 4) >> (x & 31);
+            omegaA = (m & 1u) ? c.omega_in : omegaA;
+            omegaB = (m & 2u) ? c.omega_in : omegaB;
+        }
         float oa[Q], ob[Q];
 #pragma unroll
         for (int i = 0; i < Q; ++i)
@@ -540,7 +528,7 @@ __device__ __forceinline__ void collide_pairs(const Arrays &a, const LbConst &c,
             sa[16] = bbp ? PO::lo(pv[16]) : (hasB ? PO::hi(pv[16]) : SC(16, 0));
             sa[18] = bbm ? PO::lo(pv[18]) : (hasB ? PO::hi(pv[18]) : SC(18, 0));
             float ux, uy, uz;
-            bgk_guo_cell<FORCE>(sa, FAx, FAy, FAz, cell_omega<VARTAU>(a, c, x, y, z), c.rho0, oa, ux, uy, uz);
+            bgk_guo_cell<FORCE>(sa, FAx, FAy, FAz, omegaA, c.rho0, oa, ux, uy, uz);
             if (FORCE && ub) {
                 const int64_t gi = pcell0 + cell;
                 U[gi] = make_float4(ux, uy, uz, 0.0f);
@@ -568,7 +556,7 @@ __device__ __forceinline__ void collide_pairs(const Arrays &a, const LbConst &c,
             sb[16] = bbp ? PO::hi(pv[16]) : SC(16, xp2);
             sb[18] = bbm ? PO::hi(pv[18]) : SC(18, xp2);
             float ux, uy, uz;
-            bgk_guo_cell<FORCE>(sb, FBx, FBy, FBz, cell_omega<VARTAU>(a, c, x + 1, y, z), c.rho0, ob, ux, uy, uz);
+            bgk_guo_cell<FORCE>(sb, FBx, FBy, FBz, omegaB, c.rho0, ob, ux, uy, uz);
             if (FORCE && ub) {
                 const int64_t gi = pcell0 + cell + 1;
                 U[gi] = make_float4(ux, uy, uz, 0.0f);
@@ -638,7 +626,7 @@ __global__ void __launch_bounds__(lb_block<S>(), 2)
             // order the consumers' generic reads of the stage before the
             // asynchronous writes into it
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            produce<S>(a, c, d, src, e.y, e.z, e.w, smem_raw + st_i * a.lb_stage_bytes, &full[st_i],
+            produce<S, VARTAU>(a, c, d, src, e.y, e.z, e.w, smem_raw + st_i * a.lb_stage_bytes, &full[st_i],
                        ((bits >> (k & 31)) & 1u) != 0);
             if (++st_i == ns) {
                 st_i = 0;
@@ -736,10 +724,10 @@ int lb_items_per_row(int pitch, int sb) { return sb == 2 ? pitch / 2 : pitch; }
 
 int lb_consumers(int sb) { return sb == 2 ? cons_threads<__half>() : cons_threads<float>(); }
 
-int lb_stage_bytes(int rows, int pitch, int sb, bool several)
+int lb_stage_bytes(int rows, int pitch, int sb, bool several, int mask_pitch)
 {
-    const size_t b = (size_t)rows * Q * pitch * sb + (size_t)rows * 3 * pitch * sizeof(float) + sizeof(int4) +
-                     (several ? sizeof(LbConst) : 0);
+    const size_t b = (size_t)rows * Q * pitch * sb + (size_t)rows * 3 * pitch * sizeof(float) +
+                     (size_t)rows * mask_pitch + sizeof(int4) + (several ? sizeof(LbConst) : 0);
     return (int)((b + 127) & ~(size_t)127);
 }
 
