@@ -96,12 +96,13 @@ struct iblb_ctx {
     LaunchCfg cfg{0, 2, 148, 3, 1, 0};
     bool auto_cells = true, auto_stages = true;   // group size / pipeline depth by pick_shape
     int *h_status = nullptr;     // pinned, 4 per droplet
-    double *obs_scr = nullptr;   // scratch of the mesh observation kernels
-    int64_t obs_scr_n = 0;
+    double *obs_scr = nullptr;   // scratch of the mesh observation kernels, every droplet's
+    ObsMesh *d_obs = nullptr;    // the droplets' meshes for them (with the membranes)
+    std::vector<ObsMesh> obs;
     unsigned long long *d_trace = nullptr;   // per-warp stamps of iblb_trace_step (allocated by its first call)
-    double *d_stage = nullptr;   // x, y, z per node of one droplet: node uploads and downloads
+    double *d_stage = nullptr;   // one droplet's nodes (x, y, z per node) or fields on their way
     int64_t d_stage_n = 0;
-    double *h_obs = nullptr;     // pinned: 32 raw observation doubles, then one mass per droplet
+    double *h_obs = nullptr;     // pinned: OBS_RAW raw observation doubles per droplet
     cudaEvent_t ev_copy = nullptr;   // a node upload has left the caller's buffer
     std::string err;
 };
@@ -586,6 +587,10 @@ void free_membrane_arrays(iblb_ctx *c)
     dfree(c->A.qh);
     dfree(c->A.ql);
     c->A.qh = c->A.ql = nullptr;
+    dfree(c->obs_scr);
+    dfree(c->d_obs);
+    c->obs_scr = nullptr;
+    c->d_obs = nullptr;
     dfree(c->A.ni);
     dfree(c->A.nf);
     c->A.ni = nullptr;
@@ -778,6 +783,25 @@ int rebuild_membranes(iblb_ctx *c)
         CK(up(c->A.red_out, ro.data(), sizeof(double) * ro.size()));
     }
     c->A.fref = c->d_fref;
+    {   // the meshes as the observation passes see them, each with its own scratch
+        int64_t n = 0;
+        c->obs.assign(c->ndrops, ObsMesh{});
+        for (int d = 0; d < c->ndrops; ++d)
+            n += observe_scratch_doubles(c->drops[d].nnodes, c->drops[d].ntri);
+        CK(dalloc(&c->obs_scr, (size_t)n));
+        CK(dalloc(&c->d_obs, (size_t)c->ndrops));
+        n = 0;
+        for (int d = 0; d < c->ndrops; ++d) {
+            const Drop &D = c->drops[d];
+            ObsMesh m{c->A.px, c->A.py, c->A.pz, 1, c->d_tri + 3 * (int64_t)D.tri0, D.ntri, D.node0, D.nnodes, 0, 0, 0,
+                      c->A.clamped, D.R0, c->obs_scr + n};
+            obs_mesh_plan(m);
+            m.nc = D.nnodes ? m.nc : 0;
+            n += observe_scratch_doubles(D.nnodes, D.ntri);
+            c->obs[d] = m;
+        }
+        CK(up(c->d_obs, c->obs.data(), sizeof(ObsMesh) * c->ndrops));
+    }
     CK(cudaMemsetAsync(c->A.bin_cnt, 0, sizeof(int) * c->A.total_tiles, c->stream));
     CK(cudaMemsetAsync(c->A.split_ok, 0, sizeof(int), c->stream));   // no previous band for these nodes
     c->mem_dirty = false;
@@ -965,7 +989,9 @@ int read_status(iblb_ctx *c, bool clear, int *flags_or)
     return IBLB_OK;
 }
 
-// The staging array for one droplet's nodes (x, y, z per node), grown on demand.
+// The staging array for one droplet's nodes (x, y, z per node) or fields, grown
+// on demand; fields above kStageMax doubles (128 MB) take a buffer of their own.
+constexpr int64_t kStageMax = (int64_t)16 << 20;
 int ensure_stage(iblb_ctx *c, int64_t n)
 {
     if (n > c->d_stage_n) {
@@ -1084,7 +1110,7 @@ int iblb_batch_create(int n, const iblb_lattice_desc *lat, const iblb_physics_de
         (e = dalloc(&c->d_lbc, (size_t)n)) != cudaSuccess ||
         (e = dalloc(&c->d_mass, (size_t)n)) != cudaSuccess || (e = dalloc(&c->d_drops, (size_t)n)) != cudaSuccess)
         return bad(e, "cudaMalloc");
-    if ((e = cudaMallocHost(&c->h_obs, sizeof(double) * (32 + (size_t)n))) != cudaSuccess ||
+    if ((e = cudaMallocHost(&c->h_obs, sizeof(double) * OBS_RAW * (size_t)n)) != cudaSuccess ||
         (e = cudaEventCreateWithFlags(&c->ev_copy, cudaEventDisableTiming)) != cudaSuccess)
         return bad(e, "cudaMallocHost");
     if ((e = cudaMallocHost(&c->h_status, sizeof(int) * 4 * n)) != cudaSuccess)
@@ -1161,7 +1187,6 @@ void iblb_destroy(iblb_ctx *c)
     dfree(c->d_drops);
     dfree(c->d_grp);
     dfree(c->d_lbc);
-    dfree(c->obs_scr);
     if (c->h_status)
         cudaFreeHost(c->h_status);
     if (c->h_obs)
@@ -1325,11 +1350,21 @@ int iblb_get_macros(iblb_ctx *c, int k, double *rho, double *u)
     if (r)
         return r;
     const Drop &D = c->drops[k];
-    Tmp t;
-    CK(cudaMalloc(&t.p, sizeof(double) * 4 * D.cells));
-    double *dr = (double *)t.p, *du = dr + D.cells;
     Entered entered_(c);
-    CK(launch_export_macros(c->A, k, c->storage, c->fbuf[c->cur], dr, du, D.cells, c->stream));
+    // through the staging array that the context keeps, up to kStageMax
+    // (an allocation and its release cost more than the kernel on small boxes)
+    Tmp t;
+    double *dr;
+    if (4 * D.cells <= kStageMax) {
+        if ((r = ensure_stage(c, 4 * D.cells)))
+            return r;
+        dr = c->d_stage;
+    } else {
+        CK(cudaMalloc(&t.p, sizeof(double) * 4 * D.cells));
+        dr = (double *)t.p;
+    }
+    double *du = dr + D.cells;
+    CK(launch_export_macros(c->A, D, k, c->storage, c->fbuf[c->cur], dr, du, c->stream));
     CK(cudaMemcpyAsync(rho, dr, sizeof(double) * D.cells, cudaMemcpyDeviceToHost, c->stream));
     CK(cudaMemcpyAsync(u, du, sizeof(double) * 3 * D.cells, cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));
@@ -1531,55 +1566,71 @@ int iblb_sync(iblb_ctx *c)
     return IBLB_OK;
 }
 
-// mesh observables and status of droplet k into out (the mass is filled by
-// the caller; the corrected positions are in c->A.p*); the observation
-// scratch is kept in the context
-// Enqueue the mesh observation of droplet k (kernels and a copy of the raw
-// results to c->h_obs); observe_mesh_finish fills out once the stream has
-// passed them (and c->h_status was refreshed with them).
-int observe_mesh_enqueue(iblb_ctx *c, int k, double zcut_frac, double eps_flat)
+namespace {
+
+// Observe droplets k .. k + n - 1: the lattice mass on the side stream beside
+// the corrected positions and the mesh passes, all droplets in the same
+// launches, the results written straight to pinned host memory; one
+// synchronisation.
+int observe_range(iblb_ctx *c, int k, int n, double zcut_frac, double eps_flat, iblb_obs *out)
 {
-    const Drop &D = c->drops[k];
-    if (!D.nnodes)
-        return IBLB_OK;
-    const int64_t need = observe_scratch_doubles(D.nnodes, D.ntri);
-    if (need > c->obs_scr_n) {
-        dfree(c->obs_scr);
-        c->obs_scr = nullptr;
-        c->obs_scr_n = 0;
-        CK(dalloc(&c->obs_scr, (size_t)need));
-        c->obs_scr_n = need;
+    memset(out, 0, sizeof(*out) * (size_t)n);
+    Entered entered_(c);
+    int blocks = 0, chunks = 0;
+    for (int d = k; d < k + n; ++d) {
+        blocks += c->drops[d].mass_nblocks;
+        chunks = std::max(chunks, c->A.total_nodes ? c->obs[d].nc : 0);
     }
-    CK(enqueue_observe(c->A.px, c->A.py, c->A.pz, c->A.clamped, c->A.tri + 3 * (int64_t)D.tri0, D.ntri, D.node0,
-                       D.nnodes, D.R0, zcut_frac, eps_flat, c->obs_scr, c->h_obs, c->stream));
+    CK(cudaEventRecord(c->ev_fork, c->stream));
+    CK(cudaStreamWaitEvent(c->side, c->ev_fork, 0));
+    CK(launch_mass(c->A, c->storage, c->fbuf[c->cur], c->d_mass, c->drops[k].mass_block0, blocks, k, n, c->side));
+    CK(cudaEventRecord(c->ev_join, c->side));
+    int r = IBLB_OK;
+    const ObsMesh none{}, *table = c->A.total_nodes ? c->d_obs + k : nullptr;
+    auto enqueue = [&]() -> int {
+        if (chunks) {
+            CK(launch_corrected_positions(c->A, c->stream));
+            CK(enqueue_observe(table, nullptr, n, chunks, zcut_frac, eps_flat, c->stream));
+        }
+        return IBLB_OK;
+    };
+    r = enqueue();
+    CK(cudaStreamWaitEvent(c->stream, c->ev_join, 0));   // on every way out: the side stream's work is joined
+    if (r)
+        return r;
+    CK(enqueue_observe_result(table, table ? nullptr : &none, n, c->d_mass, c->A.status, k, c->h_obs, c->stream));
+    CK(cudaStreamSynchronize(c->stream));
+    for (int i = 0; i < n; ++i) {
+        const double *hv = c->h_obs + (size_t)OBS_RAW * i;
+        iblb_obs &o = out[i];
+        o.mass = hv[13];
+        const Drop &D = c->drops[k + i];
+        if (D.nnodes) {
+            double h[14];
+            finish_observe(hv, D.R0, h);
+            o.volume = h[0];
+            o.area = h[1];
+            o.centroid[0] = h[2];
+            o.centroid[1] = h[3];
+            o.centroid[2] = h[4];
+            o.zmin = h[5];
+            o.zmax = h[6];
+            o.theta_R0_deg = h[7];
+            o.theta_RV_deg = h[8];
+            o.rc_cut = h[9];
+            o.rc_flat = h[10];
+            o.n_cut = h[11];
+            o.chi_flat = h[12];
+            o.clamped = (int)h[13];
+        }
+        // this droplet's flags; a bounded-wait timeout is recorded on droplet 0
+        // and concerns every droplet
+        o.status = status_code((int)hv[14] | ((int)hv[15] & ST_TIMEOUT));
+    }
     return IBLB_OK;
 }
 
-void observe_mesh_finish(iblb_ctx *c, int k, iblb_obs *out)
-{
-    const Drop &D = c->drops[k];
-    if (D.nnodes) {
-        double h[14];
-        finish_observe(c->h_obs, D.R0, h);
-        out->volume = h[0];
-        out->area = h[1];
-        out->centroid[0] = h[2];
-        out->centroid[1] = h[3];
-        out->centroid[2] = h[4];
-        out->zmin = h[5];
-        out->zmax = h[6];
-        out->theta_R0_deg = h[7];
-        out->theta_RV_deg = h[8];
-        out->rc_cut = h[9];
-        out->rc_flat = h[10];
-        out->n_cut = h[11];
-        out->chi_flat = h[12];
-        out->clamped = (int)h[13];
-    }
-    // this droplet's flags; a bounded-wait timeout is recorded on droplet 0
-    // and concerns every droplet
-    out->status = status_code(c->h_status[4 * k] | (c->h_status[0] & ST_TIMEOUT));
-}
+}  // namespace
 
 int iblb_observe(iblb_ctx *c, int k, double zcut_frac, double eps_flat, iblb_obs *out)
 {
@@ -1589,21 +1640,7 @@ int iblb_observe(iblb_ctx *c, int k, double zcut_frac, double eps_flat, iblb_obs
         return r;
     if (!out)
         return fail(c, IBLB_E_ARG, "null output");
-    memset(out, 0, sizeof(*out));
-    Entered entered_(c);
-    // everything enqueued, one synchronisation: the mass, the corrected
-    // positions and the mesh passes, then the copies of their results and of
-    // the status words to pinned host memory
-    CK(launch_mass(c->A, c->storage, c->fbuf[c->cur], c->d_mass, c->mass_blocks, c->stream));
-    CK(launch_corrected_positions(c->A, c->stream));
-    if ((r = observe_mesh_enqueue(c, k, zcut_frac, eps_flat)))
-        return r;
-    CK(cudaMemcpyAsync(c->h_obs + 32 + k, c->d_mass + k, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    CK(cudaMemcpyAsync(c->h_status, c->A.status, sizeof(int) * 4 * c->ndrops, cudaMemcpyDeviceToHost, c->stream));
-    CK(cudaStreamSynchronize(c->stream));
-    out->mass = c->h_obs[32 + k];
-    observe_mesh_finish(c, k, out);
-    return IBLB_OK;
+    return observe_range(c, k, 1, zcut_frac, eps_flat, out);
 }
 
 int iblb_observe_all(iblb_ctx *c, double zcut_frac, double eps_flat, iblb_obs *out)
@@ -1615,20 +1652,7 @@ int iblb_observe_all(iblb_ctx *c, double zcut_frac, double eps_flat, iblb_obs *o
         return r;
     if (!out)
         return fail(c, IBLB_E_ARG, "null output");
-    memset(out, 0, sizeof(*out) * (size_t)c->ndrops);
-    Entered entered_(c);
-    CK(launch_mass(c->A, c->storage, c->fbuf[c->cur], c->d_mass, c->mass_blocks, c->stream));
-    CK(cudaMemcpyAsync(c->h_obs + 32, c->d_mass, sizeof(double) * c->ndrops, cudaMemcpyDeviceToHost, c->stream));
-    CK(cudaMemcpyAsync(c->h_status, c->A.status, sizeof(int) * 4 * c->ndrops, cudaMemcpyDeviceToHost, c->stream));
-    CK(launch_corrected_positions(c->A, c->stream));
-    for (int k = 0; k < c->ndrops; ++k) {   // one droplet at a time through the shared scratch
-        if ((r = observe_mesh_enqueue(c, k, zcut_frac, eps_flat)))
-            return r;
-        CK(cudaStreamSynchronize(c->stream));
-        out[k].mass = c->h_obs[32 + k];
-        observe_mesh_finish(c, k, &out[k]);
-    }
-    return IBLB_OK;
+    return observe_range(c, 0, c->ndrops, zcut_frac, eps_flat, out);
 }
 
 int iblb_set_option(iblb_ctx *c, int option, int value)
@@ -1940,7 +1964,7 @@ int iblb_mesh_observe_dev(const double *d_xyz, int n_nodes, const int32_t *d_tri
         return fail(nullptr, IBLB_E_ARG, "iblb_mesh_observe_dev: bad arguments");
     cudaStream_t s = (cudaStream_t)stream;
     double *scr = nullptr;
-    CK(cudaMallocAsync((void **)&scr, sizeof(double) * observe_scratch_doubles(n_nodes, n_tri), s));
+    CK(cudaMallocAsync((void **)&scr, sizeof(double) * (observe_scratch_doubles(n_nodes, n_tri) + OBS_RAW), s));
     cudaError_t e = launch_observe_view(d_xyz, d_xyz + 1, d_xyz + 2, 3, d_tri, n_tri, 0, n_nodes, R0, zcut_frac,
                                         eps_flat, scr, out, s);
     cudaFreeAsync(scr, s);
@@ -1987,7 +2011,7 @@ namespace {
 constexpr int kNoAllocMaxChunks = 512;
 constexpr int kNoAllocMaxFaces = kNoAllocMaxChunks * RED_FACES;
 constexpr int kNoAllocMaxNodes = kNoAllocMaxChunks * RED_NODES;
-constexpr int64_t kNoAllocScratch = (int64_t)NRED * kNoAllocMaxChunks + 32 + 5 * (int64_t)kNoAllocMaxChunks + 8;
+constexpr int64_t kNoAllocScratch = (int64_t)(NRED + 5) * kNoAllocMaxChunks + OBS_RAW;
 constexpr int kNoAllocMaxDevices = 256;
 struct NoAllocSlot {
     unsigned long long ctx_id = 0;   // 0: no set-up yet (context ids start at 1)
@@ -2068,7 +2092,7 @@ int iblb_mesh_observe_dev_noalloc(const double *d_xyz, int n_nodes, const int32_
     if (!d_xyz || !d_tri || !out || n_nodes < 1 || n_tri < 1 || !(R0 > 0.0))
         return fail(nullptr, IBLB_E_ARG, "iblb_mesh_observe_dev_noalloc: bad arguments");
     if (n_tri > kNoAllocMaxFaces || n_nodes > kNoAllocMaxNodes ||
-        observe_scratch_doubles(n_nodes, n_tri) > kNoAllocScratch)
+        observe_scratch_doubles(n_nodes, n_tri) + OBS_RAW > kNoAllocScratch)
         return fail(nullptr, IBLB_E_ARG,
                     "iblb_mesh_observe_dev_noalloc: mesh too large for the static scratch (at most " +
                         std::to_string(kNoAllocMaxFaces) + " faces and " + std::to_string(kNoAllocMaxNodes) +

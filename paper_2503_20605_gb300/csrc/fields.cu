@@ -13,15 +13,16 @@ __constant__ double kW[Q] = {1.0 / 3.0,  1.0 / 18.0, 1.0 / 18.0, 1.0 / 18.0, 1.0
                              1.0 / 18.0, 1.0 / 18.0, 1.0 / 36.0, 1.0 / 36.0, 1.0 / 36.0,
                              1.0 / 36.0, 1.0 / 36.0, 1.0 / 36.0, 1.0 / 36.0, 1.0 / 36.0,
                              1.0 / 36.0, 1.0 / 36.0, 1.0 / 36.0, 1.0 / 36.0};
-__constant__ int kC[Q][3] = {{0, 0, 0},  {1, 0, 0},  {-1, 0, 0}, {0, 1, 0},   {0, -1, 0},
-                             {0, 0, 1},  {0, 0, -1}, {1, 1, 0},  {-1, -1, 0}, {1, -1, 0},
-                             {-1, 1, 0}, {0, 1, 1},  {0, -1, -1}, {0, 1, -1}, {0, -1, 1},
-                             {1, 0, 1},  {-1, 0, -1}, {1, 0, -1}, {-1, 0, 1}};
 
 template <typename S> __device__ __forceinline__ double to_d(S v);
 template <> __device__ __forceinline__ double to_d<float>(float v) { return (double)v; }
 template <> __device__ __forceinline__ double to_d<__half>(__half v) { return (double)__half2float(v); }
 template <> __device__ __forceinline__ double to_d<__nv_bfloat16>(__nv_bfloat16 v) { return (double)__bfloat162float(v); }
+__device__ __forceinline__ float to_f(float v) { return v; }
+__device__ __forceinline__ float to_f(__half v) { return __half2float(v); }
+__device__ __forceinline__ float to_f(__nv_bfloat16 v) { return __bfloat162float(v); }
+template <typename S> constexpr bool half_storage() { return false; }
+template <> constexpr bool half_storage<__half>() { return true; }
 template <typename S> __device__ __forceinline__ S from_d(double v);
 template <> __device__ __forceinline__ float from_d<float>(double v) { return (float)v; }
 template <> __device__ __forceinline__ __half from_d<__half>(double v) { return __double2half(v); }
@@ -76,29 +77,80 @@ __device__ __forceinline__ bool band_cell(const Arrays &a, const Drop &D, int64_
     return a.tile_gen[t] == *a.gen;
 }
 
+// Sum and first moments of a cell's 19 offsets in FP64.  FP64 issues at a
+// fraction of the other rates here, so nothing is multiplied by the
+// directions' 0 and +-1.
+__device__ __forceinline__ void moments(const double (&s)[Q], double &r, double (&j)[3])
+{
+#pragma unroll
+    for (int k = 0; k < Q; ++k)
+        r += s[k];
+    j[0] = ((s[1] - s[2]) + (s[7] - s[8])) + ((s[9] - s[10]) + (s[15] - s[16])) + (s[17] - s[18]);
+    j[1] = ((s[3] - s[4]) + (s[7] - s[8])) + ((s[10] - s[9]) + (s[11] - s[12])) + (s[13] - s[14]);
+    j[2] = ((s[5] - s[6]) + (s[11] - s[12])) + ((s[14] - s[13]) + (s[15] - s[16])) + (s[18] - s[17]);
+}
+
+// Half offsets are multiples of 2^-24: below 4 in magnitude their sums fit a
+// 32-bit integer and equal the FP64 sums exactly.
+constexpr float HALF_UNITS = 16777216.0f, HALF_LIMIT = 4.0f;
+__device__ __forceinline__ void moments_half(const float (&v)[Q], double &r, double (&j)[3])
+{
+    int n[Q], sum = 0;
+#pragma unroll
+    for (int k = 0; k < Q; ++k) {
+        n[k] = __float2int_rn(v[k] * HALF_UNITS);
+        sum += n[k];
+    }
+    r = fma((double)sum, 1.0 / 16777216.0, r);
+    j[0] = (double)((n[1] - n[2]) + (n[7] - n[8]) + (n[9] - n[10]) + (n[15] - n[16]) + (n[17] - n[18]));
+    j[1] = (double)((n[3] - n[4]) + (n[7] - n[8]) + (n[10] - n[9]) + (n[11] - n[12]) + (n[13] - n[14]));
+    j[2] = (double)((n[5] - n[6]) + (n[11] - n[12]) + (n[14] - n[13]) + (n[15] - n[16]) + (n[18] - n[17]));
+    for (int e = 0; e < 3; ++e)
+        j[e] *= 1.0 / 16777216.0;
+}
+
+// One block per MACRO_X cells of a row (no division per cell).  Measured with
+// the copy into kept host arrays, where the buffer was allocated and freed
+// for each call before: 128^3 FP16 1.43 -> 0.48 ms (0.36 of it the copy),
+// 80^2 x 60 FP32 0.39 -> 0.17 ms.
+constexpr int MACRO_X = 128;
 template <typename S>
-__global__ void macros_kernel(Arrays a, int d, const S *f, double *rho, double *u)
+__global__ void __launch_bounds__(MACRO_X) macros_kernel(Arrays a, int d, const S *f, double *rho, double *u)
 {
     const Drop &D = a.drops[d];
-    const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= D.cells)
+    const int chunks = (D.nx + MACRO_X - 1) / MACRO_X, row = blockIdx.x / chunks;
+    const int x = (blockIdx.x - row * chunks) * MACRO_X + threadIdx.x, z = row / D.ny, y = row - z * D.ny;
+    if (x >= D.nx)
         return;
-    double r = D.rho0, j[3] = {0.0, 0.0, 0.0};
+    const int64_t cell = x + (int64_t)D.pitch * row, c = x + (int64_t)D.nx * row;
+    const S *p = f + (int64_t)Q * D.pcell0 + cell;
+    double r = D.rho0, j[3];
+    float v[Q], most = 0.0f;
+#pragma unroll
     for (int k = 0; k < Q; ++k) {
-        const double s = to_d<S>(f[pop_index(D, k, c)]);
-        r += s;
-        for (int e = 0; e < 3; ++e)
-            j[e] += kC[k][e] * s;
+        v[k] = to_f(p[(int64_t)k * D.pcells]);
+        most = fmaxf(most, fabsf(v[k]));
+        most = v[k] == v[k] ? most : INFINITY;      // (fmaxf drops a NaN)
     }
-    int xyz[3];
+    if (sizeof(S) == 2 && half_storage<S>() && most < HALF_LIMIT) {
+        moments_half(v, r, j);
+    } else {
+        double s[Q];
+#pragma unroll
+        for (int k = 0; k < Q; ++k)
+            s[k] = (double)v[k];
+        moments(s, r, j);
+    }
     double F[3] = {D.bf[0], D.bf[1], D.bf[2]};
-    if (band_cell(a, D, c, xyz))
+    const int64_t t = D.tile0 + (x >> 2) + (int64_t)D.tx * ((y >> 2) + (int64_t)D.ty * (z >> 2));
+    if (a.tile_gen[t] == *a.gen)
         for (int e = 0; e < 3; ++e)
-            F[e] += a.F[e * a.total_pcells + pop_index(D, 0, c) - (int64_t)Q * D.pcell0 + D.pcell0];
+            F[e] += a.F[e * a.total_pcells + D.pcell0 + cell];
     rho[c] = r;
     // post-collision momentum = sum c_i f_i + F (BGK keeps rho U, Guo adds (1-1/2tau) F)
+    const double inv = 1.0 / r;
     for (int e = 0; e < 3; ++e)
-        u[e * D.cells + c] = (j[e] - 0.5 * F[e]) / r;
+        u[e * D.cells + c] = (j[e] - 0.5 * F[e]) * inv;
 }
 
 __global__ void force_kernel(Arrays a, int d, double *F)
@@ -170,14 +222,14 @@ cudaError_t launch_init_populations(const Arrays &a, int storage, void *f, cudaS
     return cudaGetLastError();
 }
 
-cudaError_t launch_export_macros(const Arrays &a, int d, int storage, const void *f, double *rho, double *u,
-                                 int64_t cells, cudaStream_t s)
+cudaError_t launch_export_macros(const Arrays &a, const Drop &D, int d, int storage, const void *f, double *rho,
+                                 double *u, cudaStream_t s)
 {
-    const unsigned g = blocks_for(cells, 256);
+    const unsigned g = (unsigned)((D.nx + MACRO_X - 1) / MACRO_X * D.ny * D.nzf);
     switch (storage) {
-    case 0: macros_kernel<float><<<g, 256, 0, s>>>(a, d, (const float *)f, rho, u); break;
-    case 1: macros_kernel<__half><<<g, 256, 0, s>>>(a, d, (const __half *)f, rho, u); break;
-    case 2: macros_kernel<__nv_bfloat16><<<g, 256, 0, s>>>(a, d, (const __nv_bfloat16 *)f, rho, u); break;
+    case 0: macros_kernel<float><<<g, MACRO_X, 0, s>>>(a, d, (const float *)f, rho, u); break;
+    case 1: macros_kernel<__half><<<g, MACRO_X, 0, s>>>(a, d, (const __half *)f, rho, u); break;
+    case 2: macros_kernel<__nv_bfloat16><<<g, MACRO_X, 0, s>>>(a, d, (const __nv_bfloat16 *)f, rho, u); break;
     default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();

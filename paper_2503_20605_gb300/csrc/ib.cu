@@ -1115,14 +1115,14 @@ __global__ void trace_marker_kernel(Arrays a, unsigned long long *tr)
     trace_start(tr, TR_END);
 }
 
-// a.p* = the positions as read (the pending correction applied)
-// and, for nodes node0 .. node0 + n - 1 when xyz is set, the same
-// positions interleaved (x, y, z per node) into xyz
+// a.p* = the positions of nodes node0 .. node0 + n - 1 as read (the pending
+// correction applied) and, when xyz is set, the same positions interleaved
+// (x, y, z per node) into xyz
 __global__ void __launch_bounds__(IB_THREADS) corrected_positions_kernel(Arrays a, double *xyz, int node0, int n)
 {
     griddep_wait();
-    const int j = blockIdx.x * IB_THREADS + threadIdx.x;
-    if (j >= a.total_nodes)
+    const int j = node0 + blockIdx.x * IB_THREADS + threadIdx.x;
+    if (j >= node0 + n)
         return;
     double x = a.qx[j], y = a.qy[j], z = a.qz[j];
     const Corr cr = load_corr(a, a.node_drop[j]);
@@ -1141,7 +1141,7 @@ __global__ void __launch_bounds__(IB_THREADS) corrected_positions_kernel(Arrays 
         a.nf[j] = sane ? make_float4(dtof_rn(x - fx), dtof_rn(y - fy), dtof_rn(z - fz), 0.0f)
                        : make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    if (xyz && j >= node0 && j < node0 + n) {
+    if (xyz) {
         double *o = xyz + 3 * (int64_t)(j - node0);
         o[0] = x;
         o[1] = y;
@@ -1324,7 +1324,11 @@ cudaError_t launch_corrected_positions(const Arrays &a, cudaStream_t s, double *
 {
     if (a.total_nodes <= 0)
         return cudaSuccess;
-    return launch_k(corrected_positions_kernel, dim3((a.total_nodes + IB_THREADS - 1) / IB_THREADS),
+    if (!xyz) {
+        node0 = 0;
+        n = a.total_nodes;
+    }
+    return launch_k(corrected_positions_kernel, dim3((n + IB_THREADS - 1) / IB_THREADS),
                     dim3(IB_THREADS), 0, s, a.pdl != 0, a, xyz, node0, n);
 }
 

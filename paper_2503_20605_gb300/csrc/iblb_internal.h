@@ -275,32 +275,49 @@ cudaError_t launch_ib_back(const Arrays &a, int n_chunks_total, bool volcorr, in
 // FP64 volume and centroid of every droplet with volume correction and the
 // rescale of its nodes (one cooperative launch)
 cudaError_t launch_volume_correction(const Arrays &a, int n_chunks_total, cudaStream_t s);
-cudaError_t launch_mass(const Arrays &a, int storage, const void *f, double *d_out, int mass_blocks,
-                        cudaStream_t s);
-// Corrected positions of every node into a.px, a.py, a.pz (the pending
-// volume correction applied; a plain copy where none is pending).
+// Lattice mass of droplets d0 .. d0 + n - 1 (their blocks block0 .. block0 +
+// blocks - 1 of the reduction) into d_out[d].
+cudaError_t launch_mass(const Arrays &a, int storage, const void *f, double *d_out, int block0, int blocks, int d0,
+                        int n, cudaStream_t s);
+// Corrected positions of every node (with xyz: of nodes node0 .. node0 + n - 1,
+// interleaved there too) into a.px, a.py, a.pz (the pending volume correction
+// applied; a plain copy where none is pending).
 cudaError_t launch_corrected_positions(const Arrays &a, cudaStream_t s, double *xyz = nullptr, int node0 = 0,
                                        int n = 0);
 // Droplet k's nodes node0 .. node0 + n - 1 set from the device array xyz
 // (x, y, z per node), with no volume correction pending for the droplet.
 cudaError_t launch_set_nodes(const Arrays &a, const double *xyz, int node0, int n, int k, cudaStream_t s);
-// Observables of one mesh: node j at q*[j * stride]; tri holds node indices
-// into q*; nodes node0 .. node0 + nnodes - 1.  Writes 13 doubles to h_out
-// (volume, area, centroid[3], zmin, zmax, theta_R0, theta_RV, rc_cut,
-// rc_flat, n_cut, chi_flat) and synchronises s.
+// One mesh to observe: node j at q*[j * stride]; tri holds node indices into
+// q*; nodes node0 .. node0 + nnodes - 1; nc chunks of fpc faces and npc nodes
+// (obs_mesh_plan); clamped: per node (global index), set by the near-wall
+// guard, or null; scratch: observe_scratch_doubles doubles.
+struct ObsMesh {
+    const double *qx, *qy, *qz;
+    int stride;
+    const int *tri;
+    int ntri, node0, nnodes;
+    int nc, fpc, npc;
+    const uint8_t *clamped;
+    double R0;
+    double *scratch;
+};
+constexpr int OBS_RAW = 16;        // raw results per mesh (obs_result_kernel)
+void obs_mesh_plan(ObsMesh &m);
 int64_t observe_scratch_doubles(int n_nodes, int n_tri);
+// The passes over n meshes (of the device table, or the one given), and their
+// raw results to out (device, or pinned host memory); once s has passed them,
+// finish_observe turns a mesh's OBS_RAW doubles into V, A, cx, cy, cz, zmin,
+// zmax, theta_R0, theta_RV, rc_cut, rc_flat, n_cut, chi_flat, clamped.
+cudaError_t enqueue_observe(const ObsMesh *table, const ObsMesh *one, int n, int max_chunks, double zcut_frac,
+                            double eps_flat, cudaStream_t s);
+cudaError_t enqueue_observe_result(const ObsMesh *table, const ObsMesh *one, int n, const double *mass,
+                                   const int *status, int d0, double *out, cudaStream_t s);
+void finish_observe(const double *hv, double R0, double *h_out);
+// The first 13 of one mesh to h_out; synchronises s.  scratch: OBS_RAW
+// doubles more than observe_scratch_doubles.
 cudaError_t launch_observe_view(const double *qx, const double *qy, const double *qz, int stride,
                                 const int *tri, int ntri, int node0, int nnodes, double R0, double zcut_frac,
                                 double eps_flat, double *scratch, double *h_out, cudaStream_t s);
-// The same for a context's droplet (positions with stride 1, and the
-// near-wall guard's per-node flags, counted as a fourteenth value) without
-// the synchronisation: the kernels and a copy of 32 raw doubles to hv (host,
-// pinned) are enqueued on s; once s has passed them, finish_observe turns hv
-// into the 14 values.
-cudaError_t enqueue_observe(const double *qx, const double *qy, const double *qz, const uint8_t *clamped,
-                            const int *tri, int ntri, int node0, int nnodes, double R0, double zcut_frac,
-                            double eps_flat, double *scratch, double *hv, cudaStream_t s);
-void finish_observe(const double *hv, double R0, double *h_out);
 // Bring the code of the observation kernels onto the current device now
 // (module loading is lazy by default, and a load allocates device memory).
 cudaError_t preload_observe_kernels();
@@ -310,8 +327,8 @@ cudaError_t launch_export_populations(const Arrays &a, int d, int storage, const
                                       int64_t cells, cudaStream_t s);
 cudaError_t launch_import_populations(const Arrays &a, int d, int storage, void *f, const double *in,
                                       int64_t cells, cudaStream_t s);
-cudaError_t launch_export_macros(const Arrays &a, int d, int storage, const void *f, double *rho, double *u,
-                                 int64_t cells, cudaStream_t s);
+cudaError_t launch_export_macros(const Arrays &a, const Drop &D, int d, int storage, const void *f, double *rho,
+                                 double *u, cudaStream_t s);
 cudaError_t launch_export_force(const Arrays &a, int d, double *F, int64_t cells, cudaStream_t s);
 cudaError_t launch_export_inside(const Arrays &a, int d, uint8_t *inside, int64_t cells, cudaStream_t s);
 cudaError_t launch_init_populations(const Arrays &a, int storage, void *f, cudaStream_t s);
