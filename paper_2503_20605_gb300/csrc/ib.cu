@@ -114,6 +114,45 @@ __device__ __forceinline__ float dtof_rn(double x)
     return __uint_as_float(s | b);
 }
 
+// v 2^e, v != 0, rounded to nearest (ties to even) FP32 by integer operations
+// (the result normal)
+__device__ __forceinline__ float fixed_to_float(uint64_t v, int e)
+{
+    const int lz = __clzll((long long)v);
+    v <<= lz;
+    const uint32_t h = (uint32_t)(v >> 32), l = (uint32_t)v, m = h >> 8, r = h & 0xffu;
+    const uint32_t up = (r > 0x80u || (r == 0x80u && (l != 0u || (m & 1u)))) ? 1u : 0u;
+    return __uint_as_float(((uint32_t)(190 + e - lz) << 23) + (m - 0x800000u) + up);
+}
+
+// floor(q) and q - floor(q) in units of 2^-64 (bits below that collected in the
+// last one, so that roundings of it are those of q) for |q| < 2^31, by integer
+// operations: FP64's floor, difference and conversions each occupy the
+// pipe for as long as some dozens of these.
+__device__ __forceinline__ int split_floor(double q, uint64_t &frac)
+{
+    const uint32_t h = (uint32_t)__double2hiint(q);
+    const int be = (int)((h >> 20) & 0x7ffu);
+    uint64_t M = ((uint64_t)((h & 0xfffffu) | (be ? 0x100000u : 0u)) << 32) | (uint32_t)__double2loint(q);
+    const int e = (be ? be : 1) - 1023;                  // q = M 2^(e - 52)
+    int ip = 0;
+    if (e >= 0) {
+        ip = (int)(M >> (52 - e));
+        M <<= 12 + e;                                    // the integer bits leave at the top
+    } else if (e >= -12) {
+        M <<= 12 + e;
+    } else {
+        const int r = -12 - e;
+        M = r > 63 ? (M ? 1u : 0u) : ((M >> r) | ((M & ((1ull << r) - 1)) ? 1u : 0u));
+    }
+    if ((int)h < 0) {
+        ip = M ? -ip - 1 : -ip;
+        M = 0ull - M;
+    }
+    frac = M;
+    return ip;
+}
+
 // One coordinate of q_a - q_j from the FP32 pairs of the two positions: the
 // hi parts of nearby positions differ exactly, the lo parts carry the rest.
 __device__ __forceinline__ float rel_coord(float ah, float al, float jh, float jl)
@@ -202,6 +241,12 @@ __device__ __forceinline__ void psi4(float f, float *w)
 // [0, n) otherwise; at most 3 (a partial last tile of a periodic axis).
 __device__ __forceinline__ int support_tiles3(int b, int n, bool periodic, int &t0, int &t1, int &t2)
 {
+    if (b >= 1 && b + 2 < n) {       // away from the ends
+        t0 = (b - 1) >> 2;
+        t1 = (b + 2) >> 2;
+        t2 = -1;
+        return t0 == t1 ? 1 : 2;
+    }
     int cnt = 0;
     t0 = t1 = t2 = -1;
 #pragma unroll
@@ -293,43 +338,42 @@ __device__ __forceinline__ void node_forces(const Arrays &a, int64_t gid, uint32
     if (cr.on)
         q = corr1(q, ax == 0 ? cr.cx : (ax == 1 ? cr.cy : cr.cz), cr.k);
     const int qb = threadIdx.x & 28;      // the quad's first lane
-    const int sane_l = fabs(q) < 1e8 ? 1 : 0;
-    const bool sane = __shfl_sync(0xffffffffu, sane_l, qb | 0) && __shfl_sync(0xffffffffu, sane_l, qb | 1) &&
-                      __shfl_sync(0xffffffffu, sane_l, qb | 2);
-    int b = 0, nt = 0, t0 = -1, t1 = -1, t2 = -1;
+    // |q| < 1e8, by the high word (1e8's low word is 0)
+    const bool sane_l = ((uint32_t)__double2hiint(q) & 0x7fffffffu) < 0x4197d784u;
+    const bool sane = ((__ballot_sync(0xffffffffu, sane_l) >> qb) & 7u) == 7u;
+    int b = 0, nt = 0, t0 = 0, t1 = 0, t2 = 0;
     float w[4] = {0.f, 0.f, 0.f, 0.f};
+    float hz = -1.0f;                  // lane 2: height over the wall plane, z - 1/2 (-1: below it)
     if (a.ni && valid && l == 3)
         a.ni[j].w = sane ? 1 : 0;
     if (valid && l < 3 && sane) {
-        const double fb = floor(q);
-        const float f = dtof_rn(q - fb);
+        uint64_t frac;
+        const int ib = split_floor(q, frac);
+        const float f = frac ? fixed_to_float(frac, -64) : 0.0f;
         if (a.ni) {     // for the in/out test
-            (&a.ni[j].x)[ax] = (int)fb;
+            (&a.ni[j].x)[ax] = ib;
             (&a.nf[j].x)[ax] = f;
         }
         const int n = ax == 0 ? D.nx : (ax == 1 ? D.ny : D.nzf);
-        if (ax < 2) {
-            b = wrapi((int)fb % n, n);
-            nt = support_tiles3(b, n, true, t0, t1, t2);
-        } else {
-            b = (int)fb - D.walls;
-            if (!D.walls)
-                b = wrapi(b % D.nz, D.nz);
-            nt = support_tiles3(b, n, !D.walls, t0, t1, t2);
-        }
+        const bool periodic = ax < 2 || !D.walls;
+        b = ax == 2 ? ib - D.walls : ib;
+        if (periodic && (b < 0 || b >= n))
+            b = wrapi(b % n, n);
+        nt = support_tiles3(b, n, periodic, t0, t1, t2);
         psi4(f, w);
+        const int I = ib - (frac >> 63 ? 0 : 1);
+        const uint64_t G = frac ^ (1ull << 63);          // z - 1/2 = I + G 2^-64
+        if (I > 0)
+            hz = fixed_to_float(((uint64_t)(uint32_t)I << 32) | (G >> 32) | ((uint32_t)G ? 1u : 0u), -32);
+        else if (I == 0)
+            hz = G ? fixed_to_float(G, -64) : 0.0f;
     }
-    // the z coordinate (lane 2) for the wall interaction; the tile counts
-    // and tiles of every axis for the listing
-    const double qz = __shfl_sync(0xffffffffu, q, qb | 2);
-    const int ntx = __shfl_sync(0xffffffffu, nt, qb | 0), nty = __shfl_sync(0xffffffffu, nt, qb | 1),
-              ntz = __shfl_sync(0xffffffffu, nt, qb | 2);
-    const int tx0 = __shfl_sync(0xffffffffu, t0, qb | 0), tx1 = __shfl_sync(0xffffffffu, t1, qb | 0),
-              tx2 = __shfl_sync(0xffffffffu, t2, qb | 0);
-    const int ty0 = __shfl_sync(0xffffffffu, t0, qb | 1), ty1 = __shfl_sync(0xffffffffu, t1, qb | 1),
-              ty2 = __shfl_sync(0xffffffffu, t2, qb | 1);
-    const int tz0 = __shfl_sync(0xffffffffu, t0, qb | 2), tz1 = __shfl_sync(0xffffffffu, t1, qb | 2),
-              tz2 = __shfl_sync(0xffffffffu, t2, qb | 2);
+    // the height (lane 2) for the wall interaction; every axis' tiles for the listing
+    const float hwall = __shfl_sync(0xffffffffu, hz, qb | 2);
+    const uint32_t pk = ((uint32_t)t0 & 2047u) | (((uint32_t)t1 & 2047u) << 11) | ((uint32_t)nt << 22);
+    const uint32_t pkx = __shfl_sync(0xffffffffu, pk, qb | 0), pky = __shfl_sync(0xffffffffu, pk, qb | 1),
+                   pkz = __shfl_sync(0xffffffffu, pk, qb | 2);
+    const int ntx = (int)(pkx >> 22), nty = (int)(pky >> 22), ntz = (int)(pkz >> 22);
     const int ncombo = ntx * nty * ntz;
     NodeRec &rec = a.rec[valid ? j : 0];
     if (valid && l < 3) {
@@ -339,49 +383,56 @@ __device__ __forceinline__ void node_forces(const Arrays &a, int64_t gid, uint32
         float *rw = ax == 0 ? rec.wx : (ax == 1 ? rec.wy : rec.wz);
         *reinterpret_cast<float4 *>(rw) = make_float4(w[0], w[1], w[2], w[3]);
     }
-    // the node's tiles, shared by the four lanes: every counter's atomic is
-    // issued before any result is used (a support across a partial periodic
-    // tile can touch up to 27 tiles)
+    // the node's tiles, shared by the four lanes: both of a lane's counters'
+    // atomics are issued before any result is used
     const int cur = (int)(gen & 1u);
-    for (int c0 = l; valid && c0 < ncombo; c0 += 2 * NL) {
-        int64_t tl[2], trw[2];
-        int rk[2], tc[2];
+    auto list_node = [&](const int (&tx)[2], const bool (&on)[2], int ty, int tz) {
+        const int row = ty + D.ty * tz;
+        const int64_t tl = D.tile0 + (int64_t)D.tx * row;
+        int rk[2];
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+            if (on[i])
+                rk[i] = atomicAdd(&a.bin_cnt[tl + tx[i]], 1);
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
-            const int c = c0 + i * NL;
-            if (c < ncombo) {
-                const int ix = c % ntx, iy = (c / ntx) % nty, iz = c / (ntx * nty);
-                const int tx = ix == 0 ? tx0 : (ix == 1 ? tx1 : tx2);
-                const int ty = iy == 0 ? ty0 : (iy == 1 ? ty1 : ty2);
-                const int tz = iz == 0 ? tz0 : (iz == 1 ? tz1 : tz2);
-                tl[i] = D.tile0 + tx + (int64_t)D.tx * (ty + (int64_t)D.ty * tz);
-                trw[i] = D.trow0 + ty + (int64_t)D.ty * tz;
-                tc[i] = tile_coords(tx, ty, tz);
-                rk[i] = atomicAdd(&a.bin_cnt[tl[i]], 1);
-            }
-        }
-#pragma unroll
-        for (int i = 0; i < 2; ++i) {
-            if (c0 + i * NL >= ncombo)
+            if (!on[i])
                 continue;
-            const int64_t t = tl[i];
-            const int rank = rk[i];
-            if (rank == 0) {        // first node of the tile: the tile joins the band
+            const int64_t t = tl + tx[i];
+            if (rk[i] == 0) {        // first node of the tile: the tile joins the band
                 a.tile_gen[t] = gen;
                 const int slot = atomicAdd(&a.n_active[cur], 1);
                 if (slot < a.active_cap)
-                    a.active[(int64_t)cur * a.active_cap + slot] = make_int2((int)t, tc[i]);
+                    a.active[(int64_t)cur * a.active_cap + slot] = make_int2((int)t, tile_coords(tx[i], ty, tz));
                 // its tile row too; the stream-collide rows run before this
                 // step's band was known assumed that this row could not hold
                 // band tiles
-                a.rowgen[trw[i]] = gen;
-                if (a.grp_cnt[2] && !a.candrow[trw[i]])
+                a.rowgen[D.trow0 + row] = gen;
+                if (a.grp_cnt[2] && !a.candrow[D.trow0 + row])
                     atomicOr(&a.status[4 * d], ST_BAND_MISS);
             }
-            if (rank < TILE_CAP)
-                a.tile_list[t * TILE_CAP + rank] = j;
+            if (rk[i] < TILE_CAP)
+                a.tile_list[t * TILE_CAP + rk[i]] = j;
             else
                 atomicOr(&a.status[4 * d], ST_SPREAD_OVF);
+        }
+    };
+    if (!__any_sync(0xffffffffu, nt > 2)) {
+        // at most two tiles an axis: lane l takes the y and z tile of its bits
+        // and both x tiles
+        const int iy = l & 1, iz = l >> 1;
+        const bool mine = valid && iy < nty && iz < ntz;
+        list_node({(int)(pkx & 2047u), (int)((pkx >> 11) & 2047u)}, {mine && ntx > 0, mine && ntx > 1},
+                  (int)((iy ? pky >> 11 : pky) & 2047u), (int)((iz ? pkz >> 11 : pkz) & 2047u));
+    } else {
+        // a support across a partial periodic tile: up to three tiles an axis
+        const int tx2 = __shfl_sync(0xffffffffu, t2, qb | 0), ty2 = __shfl_sync(0xffffffffu, t2, qb | 1),
+                  tz2 = __shfl_sync(0xffffffffu, t2, qb | 2);
+        for (int c = l; valid && c < ncombo; c += NL) {
+            const int ix = c % ntx, iy = (c / ntx) % nty, iz = c / (ntx * nty);
+            const int tx = ix == 2 ? tx2 : (int)((ix ? pkx >> 11 : pkx) & 2047u);
+            list_node({tx, 0}, {true, false}, iy == 2 ? ty2 : (int)((iy ? pky >> 11 : pky) & 2047u),
+                      iz == 2 ? tz2 : (int)((iz ? pkz >> 11 : pkz) & 2047u));
         }
     }
     // the faces: the first pass from the positions loaded above, then any
@@ -456,7 +507,7 @@ __device__ __forceinline__ void node_forces(const Arrays &a, int64_t gid, uint32
                 pz += ez;
             }
             if (D.wetting) {
-                float h = dtof_rn(qz - 0.5);
+                float h = hwall;
                 if (h < D.hmin) {
                     h = D.hmin;
                     clamped = 1;
