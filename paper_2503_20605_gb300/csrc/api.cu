@@ -873,7 +873,8 @@ int enqueue_step(iblb_ctx *c, int par, bool forces_only)
         CK(launch_lb(a, c->storage, c->fbuf[par], c->fbuf[par ^ 1], c->any_vartau, c->cfg, s, a.grp_list,
                      a.grp_cnt, false));
     else
-        CK(launch_lb(a, c->storage, c->fbuf[par], c->fbuf[par ^ 1], nodes && c->any_vartau, c->cfg, s));
+        CK(launch_lb(a, c->storage, c->fbuf[par], c->fbuf[par ^ 1], nodes && c->any_vartau, c->cfg, s, nullptr, nullptr,
+                     false, -1, nodes && a.pdl));   // after the forces and the spread
     CK(mark(4));
     if (nodes && c->fused_ib) {
         CK(launch_ib_back(a, c->n_red_chunks, c->any_volcorr, c->cfg.ib_blocks_per_sm, s));   // advection, volume correction

@@ -54,19 +54,6 @@ __device__ __forceinline__ float ipow(float r, int k)
     return p;
 }
 
-__device__ __forceinline__ int find_drop_tile(const Drop *D, int n, int64_t t)
-{
-    int lo = 0, hi = n - 1;
-    while (lo < hi) {
-        int mid = (lo + hi + 1) >> 1;
-        if (D[mid].tile0 <= t)
-            lo = mid;
-        else
-            hi = mid - 1;
-    }
-    return lo;
-}
-
 // The volume correction of a step (not in the paper) is kept pending: the
 // stored positions q are those after advection, and the correction
 // q' = c + (q - c) k computed from them is applied wherever positions are
@@ -288,8 +275,11 @@ __device__ __forceinline__ int support_tiles3(int b, int n, bool periodic, int &
 // neighbour positions are in flight.  Every lane of the warp takes part
 // (the shuffles span whole quads).
 constexpr int NL = 4;
-template <bool EL>     // EL: some droplet of the launch has an elastic membrane (a.fref set)
-__device__ __forceinline__ void node_forces(const Arrays &a, int64_t gid, uint32_t gen)
+// EL: some droplet of the launch has an elastic membrane (a.fref set).  WAIT:
+// the node's faces and droplet, which no kernel writes, are read before the
+// wait for the previous kernel, the step's generation after it.
+template <bool EL, bool WAIT, bool TR = false>
+__device__ __forceinline__ void node_forces(const Arrays &a, int64_t gid, uint32_t gen, unsigned long long *tr = nullptr)
 {
     const int j = (int)(gid >> 2), l = (int)(gid & 3);
     const bool valid = j < a.total_nodes;
@@ -308,15 +298,23 @@ __device__ __forceinline__ void node_forces(const Arrays &a, int64_t gid, uint32
     float4 a0h = zero4, a0l = zero4, b0h = zero4, b0l = zero4, a1h = zero4, a1l = zero4, b1h = zero4, b1l = zero4;
     if (valid) {
         d = a.ndrops == 1 ? 0 : a.node_drop[j];   // (one droplet: no lookup on the critical path)
+        f0 = a.ring8[(int64_t)RING8 * j + l];
+        f1 = a.ring8[(int64_t)RING8 * j + l + NL];
+        nfaces = f0.w;
+    }
+    if (WAIT) {
+        griddep_wait();
+        if constexpr (TR)
+            trace_start(tr, TR_FORCE);
+        gen = *a.gen + 1u;                        // committed by the spread
+    }
+    if (valid) {
         cr = load_corr(a, d);
         qx0 = a.qx[j];
         qy0 = a.qy[j];
         qz0 = a.qz[j];
         jh = a.qh[j];
         jl = a.ql[j];
-        f0 = a.ring8[(int64_t)RING8 * j + l];
-        f1 = a.ring8[(int64_t)RING8 * j + l + NL];
-        nfaces = f0.w;
         if (l < nfaces) {
             a0h = a.qh[f0.x];
             a0l = a.ql[f0.x];
@@ -403,7 +401,7 @@ __device__ __forceinline__ void node_forces(const Arrays &a, int64_t gid, uint32
                 a.tile_gen[t] = gen;
                 const int slot = atomicAdd(&a.n_active[cur], 1);
                 if (slot < a.active_cap)
-                    a.active[(int64_t)cur * a.active_cap + slot] = make_int2((int)t, tile_coords(tx[i], ty, tz));
+                    a.active[(int64_t)cur * a.active_cap + slot] = make_int4((int)t, tile_coords(tx[i], ty, tz), d, 0);
                 // its tile row too; the stream-collide rows run before this
                 // step's band was known assumed that this row could not hold
                 // band tiles
@@ -576,7 +574,7 @@ __device__ __forceinline__ void tile_weights(int T0, int b, int n, bool periodic
 // does not matter.
 struct LeftTile {
     int64_t T = -1;
-    int coords = 0;
+    int coords = 0, d = 0;
     uint32_t g = 0;
 };
 template <int NT>
@@ -586,9 +584,10 @@ __device__ __forceinline__ LeftTile zero_left_first(const Arrays &a, int cur, in
     LeftTile lt;
     const int it = bid * TPB + threadIdx.x / TILE_CELLS;
     if (it < min(a.n_active[cur ^ 1], a.active_cap)) {
-        const int2 e = a.active[(int64_t)(cur ^ 1) * a.active_cap + it];
+        const int4 e = a.active[(int64_t)(cur ^ 1) * a.active_cap + it];
         lt.T = e.x;
         lt.coords = e.y;
+        lt.d = e.z;
         lt.g = a.tile_gen[lt.T];
     }
     return lt;
@@ -600,15 +599,14 @@ __device__ void zero_left_tiles(const Arrays &a, uint32_t gen, int cur, int bid,
     constexpr int TPB = NT / TILE_CELLS;
     const int tid = threadIdx.x;
     const int nprev = min(a.n_active[cur ^ 1], a.active_cap);
-    const int2 *plist = a.active + (int64_t)(cur ^ 1) * a.active_cap;
+    const int4 *plist = a.active + (int64_t)(cur ^ 1) * a.active_cap;
     for (int it = bid * TPB + tid / TILE_CELLS; it < nprev; it += nb * TPB) {
         const bool pre = it == bid * TPB + tid / TILE_CELLS && first.T >= 0;
-        const int2 e = pre ? make_int2((int)first.T, first.coords) : plist[it];
+        const int4 e = pre ? make_int4((int)first.T, first.coords, first.d, 0) : plist[it];
         const int64_t T = e.x;
         if ((pre ? first.g : a.tile_gen[T]) == gen)
             continue;
-        const int d = a.ndrops == 1 ? 0 : find_drop_tile(a.drops, a.ndrops, T);
-        const Drop &D = a.drops[d];
+        const Drop &D = a.drops[e.z];
         const int cell = tid & (TILE_CELLS - 1);
         const int X = 4 * (e.y & 2047) + (cell & 3);
         const int Y = 4 * ((e.y >> 11) & 2047) + ((cell >> 2) & 3);
@@ -639,20 +637,19 @@ __device__ void spread_tiles(const Arrays &a, uint32_t gen, int cur, int bid, in
     constexpr int HK = TILE_CAP / NT;              // a tile's nodes per thread, at most
     const int tid = threadIdx.x;
     const int nact = min(a.n_active[cur], a.active_cap);
-    const int2 *list = a.active + (int64_t)cur * a.active_cap;
+    const int4 *list = a.active + (int64_t)cur * a.active_cap;
     // a block's next tile is looked up while it works on the current one:
     // its list entry at once, its count and first key once the entry is in
     // (a thread's first key slot is loaded whatever the count: the tile's
     // list has TILE_CAP slots, and slots beyond the count are not used)
-    int2 te_n = bid < nact ? list[bid] : make_int2(0, 0);
+    int4 te_n = bid < nact ? list[bid] : make_int4(0, 0, 0, 0);
     int cnt_n = -1, key0_n = 0x7fffffff;
     for (int it = bid; it < nact; it += nb) {
-        const int2 te = te_n;
+        const int4 te = te_n;
         if (it + nb < nact)
             te_n = list[it + nb];
         const int64_t T = te.x;
-        const int d = a.ndrops == 1 ? 0 : find_drop_tile(a.drops, a.ndrops, T);
-        const Drop &D = a.drops[d];
+        const Drop &D = a.drops[te.z];
         const int X0 = 4 * (te.y & 2047), Y0 = 4 * ((te.y >> 11) & 2047), Z0 = 4 * (te.y >> 22);
         const int64_t e0 = T * TILE_CAP;
         // (overflow was flagged by the force kernel)
@@ -818,7 +815,11 @@ __device__ __forceinline__ void transpose4(float (&v)[4])
 // threads, one coordinate each, so that its FP64 operations fill whole
 // warps (on this GPU they issue at a small fraction of the FP32 rate); each
 // thread reads its (corrected) coordinate when the kernel starts.
-__device__ __forceinline__ void interp_block(const Arrays &a, int64_t base)
+// WAIT: records, coordinates and droplets, which the force kernel wrote (the
+// spread and the stream-collide kernel waited in turn since) or no kernel
+// writes, are read before the wait for the stream-collide kernel.
+template <bool WAIT, bool TR = false>
+__device__ __forceinline__ void interp_block(const Arrays &a, int64_t base, unsigned long long *tr = nullptr)
 {
     constexpr int NPB = IB_THREADS / 16;
     __shared__ float inc_s[3 * NPB];
@@ -834,28 +835,41 @@ __device__ __forceinline__ void interp_block(const Arrays &a, int64_t base)
     float ux[4] = {0.f, 0.f, 0.f, 0.f}, uy[4] = {0.f, 0.f, 0.f, 0.f}, uz[4] = {0.f, 0.f, 0.f, 0.f};
     float4 wx = make_float4(0.f, 0.f, 0.f, 0.f);
     float wyz = 0.f;
+    bool on = false;
+    int z0 = 0, walls = 0, nzf = 0;
+    int64_t at = 0, plane = 0;
     if (valid) {
         d = a.ndrops == 1 ? 0 : a.node_drop[j];
         const NodeRec &r = a.rec[j];
         const Drop &D = a.drops[d];
         const int4 base4 = *reinterpret_cast<const int4 *>(&r);      // bx, by, bz, key
-        if (base4.w > 0) {
+        on = base4.w > 0;
+        if (on) {
             const int y = l >> 2, k = l & 3;
             wx = *reinterpret_cast<const float4 *>(r.wx);
             wyz = r.wy[y] * r.wz[k];
             const int X = wrapi(base4.x - 1 + k, D.nx), Y = wrapi(base4.y - 1 + y, D.ny);
-            const int64_t at = D.pcell0 + X + (int64_t)D.pitch * Y, plane = (int64_t)D.pitch * D.ny;
+            at = D.pcell0 + X + (int64_t)D.pitch * Y;
+            plane = (int64_t)D.pitch * D.ny;
+            z0 = base4.z - 1;
+            walls = D.walls;
+            nzf = D.nzf;
+        }
+    }
+    if (WAIT) {
+        griddep_wait();
+        if constexpr (TR)
+            trace_start(tr, TR_INTERP);
+    }
+    if (on) {
 #pragma unroll
-            for (int z = 0; z < 4; ++z) {
-                int Z = base4.z - 1 + z;
-                if (!D.walls)
-                    Z = wrapi(Z, D.nzf);
-                if (Z >= 0 && Z < D.nzf) {       // cells outside the fluid supply U = 0
-                    const float4 u = a.U[at + plane * Z];
-                    ux[z] = u.x;
-                    uy[z] = u.y;
-                    uz[z] = u.z;
-                }
+        for (int z = 0; z < 4; ++z) {
+            const int Z = walls ? z0 + z : wrapi(z0 + z, nzf);
+            if (Z >= 0 && Z < nzf) {             // cells outside the fluid supply U = 0
+                const float4 u = a.U[at + plane * Z];
+                ux[z] = u.x;
+                uy[z] = u.y;
+                uz[z] = u.z;
             }
         }
     }
@@ -1117,11 +1131,7 @@ constexpr int NF_THREADS = 64;   // block size of the force kernel (16 nodes): s
 template <bool EL, bool TR>
 __global__ void __launch_bounds__(NF_THREADS) node_force_kernel(Arrays a, unsigned long long *tr)
 {
-    griddep_wait();
-    if constexpr (TR)
-        trace_start(tr, TR_FORCE);
-    const uint32_t gen = *a.gen + 1u;                  // committed by the spread
-    node_forces<EL>(a, (int64_t)blockIdx.x * NF_THREADS + threadIdx.x, gen);
+    node_forces<EL, true, TR>(a, (int64_t)blockIdx.x * NF_THREADS + threadIdx.x, 0, tr);
 }
 
 template <bool TR>
@@ -1130,6 +1140,13 @@ __global__ void __launch_bounds__(SP_THREADS, SP_PER_SM) spread_kernel(Arrays a,
     griddep_wait();
     if constexpr (TR)
         trace_start(tr, TR_SPREAD);
+    // One droplet: the next kernel's blocks may take the SMs that finish first
+    // (the stream-collide kernel then requests its first populations while the
+    // last tiles are summed).  Every block of this launch is resident when the
+    // last one says so.  Measured (step, us): 32^3 17.3 -> 16.5, 128^3 FP16 53.6
+    // -> 52.1, 163 842 nodes 289 -> 286; but 64 boxes 647 -> 666, so not there.
+    if (a.ndrops == 1)
+        launch_dependents();
     __shared__ SpreadSmem sm;
     const uint32_t gen = *a.gen + 1u;
     const int cur = (int)(gen & 1u);
@@ -1142,10 +1159,7 @@ __global__ void __launch_bounds__(SP_THREADS, SP_PER_SM) spread_kernel(Arrays a,
 template <bool TR>
 __global__ void __launch_bounds__(IB_THREADS) interp_advect_kernel(Arrays a, unsigned long long *tr)
 {
-    griddep_wait();
-    if constexpr (TR)
-        trace_start(tr, TR_INTERP);
-    interp_block(a, (int64_t)blockIdx.x * IB_THREADS);
+    interp_block<true, TR>(a, (int64_t)blockIdx.x * IB_THREADS, tr);
 }
 
 // The volume correction of every droplet: FP64 volume and centroid
@@ -1235,7 +1249,7 @@ __global__ void __launch_bounds__(IB_THREADS) ib_front_kernel(Arrays a)
     const int64_t nf = ((int64_t)a.total_nodes * NL + 31) & ~(int64_t)31;   // whole warps
     const int64_t stride = (int64_t)gridDim.x * IB_THREADS;
     for (int64_t gid = (int64_t)blockIdx.x * IB_THREADS + threadIdx.x; gid < nf; gid += stride)
-        node_forces<EL>(a, gid, gen);
+        node_forces<EL, false>(a, gid, gen);
     if (!grid_barrier(a, sense))
         return;
     const LeftTile first = zero_left_first<IB_THREADS>(a, cur, blockIdx.x);
@@ -1253,7 +1267,7 @@ __global__ void __launch_bounds__(IB_THREADS) ib_back_kernel(Arrays a, int n_chu
     const int64_t ni = (int64_t)a.total_nodes * 16;
     const int64_t stride = (int64_t)gridDim.x * IB_THREADS;
     for (int64_t base = (int64_t)blockIdx.x * IB_THREADS; base < ni; base += stride) {   // block-uniform
-        interp_block(a, base);
+        interp_block<false>(a, base);
         __syncthreads();    // the next pass rewrites inc_s
     }
     if (!volcorr)

@@ -114,9 +114,10 @@ struct Arrays {
     uint32_t *tile_gen;            // tile is in the band of this step iff == *gen
     uint32_t *gen;                 // step generation counter (device)
     int *n_active;                 // 2: band tiles of this step / of the previous step
-    int2 *active;                  // 2 * active_cap: band tiles, indexed by generation parity: the
-                                   // pooled tile index and the tile's coordinates in its droplet
-                                   // (tile_coords), so that readers need no divisions
+    int4 *active;                  // 2 * active_cap: band tiles, indexed by generation parity: the
+                                   // pooled tile index, the tile's coordinates in its droplet
+                                   // (tile_coords) and the droplet, so that readers need neither
+                                   // divisions nor a search
     int active_cap;
     // per-tile node lists
     int *bin_cnt;                  // total_tiles: nodes listed in this step (returns to 0 in the spread)
@@ -206,10 +207,15 @@ cudaError_t launch_trace_marker(const Arrays &a, unsigned long long *trace, cuda
 
 // Programmatic dependent launch: a kernel of the step may be launched while
 // the previous one finishes; griddep_wait() returns once the previous kernel
-// has completed and its writes are visible, and it is the first statement of
-// every kernel of the step (a no-op for a kernel launched without the
-// attribute).
+// has completed and its writes are visible (a no-op for a kernel launched
+// without the attribute).  Every kernel of the step calls it, before it reads
+// what a kernel of the step writes: what no kernel writes (topology, droplets,
+// group table) may be read sooner, and so may results of a kernel before the
+// previous one, when that kernel waited in its turn.  launch_dependents() lets
+// the next kernel's blocks start where this one's have finished; without it
+// they start once all have.
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // Launch with or without programmatic dependent launch.
 template <typename... KArgs, typename... Args>
@@ -256,10 +262,13 @@ int lb_items_per_row(int pitch, int storage_bytes);
 int lb_consumers(int storage_bytes);
 
 // Stream-collide over every group (list == nullptr) or over the groups
-// list[0 .. *count); no_force: the groups carry no force (skip the band test).
+// list[0 .. *count); no_force: the groups carry no force (skip the band test);
+// early: the populations may be read before the previous kernel has finished
+// (two kernels that wait for their predecessors separate this launch from the
+// last one that wrote them).
 cudaError_t launch_lb(const Arrays &a, int storage, const void *src, void *dst, bool vartau,
                       const LaunchCfg &cfg, cudaStream_t s, const int *list = nullptr, const int *count = nullptr,
-                      bool no_force = false, int blocks_per_sm = -1);
+                      bool no_force = false, int blocks_per_sm = -1, bool early = false);
 // Split the stream-collide groups of the coming step into those whose rows
 // may meet its band (within one tile row of the previous step's band) and
 // the others; also marks the tile rows that may hold band tiles.

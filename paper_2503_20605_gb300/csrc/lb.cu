@@ -117,77 +117,81 @@ __device__ __forceinline__ uint32_t band_ballot(const Arrays &a, const int *list
     return __ballot_sync(0xffffffffu, band);
 }
 
-// Producer warp: fetch group g into a stage.  The source rows of population i
-// for rows y0 .. y0+nr-1 of plane z are rows y0-c_iy .. of plane z-c_iz
-// (or the group's own rows of the opposite population at a wall), which are
-// contiguous in memory except across the periodic y seam: lane i < 19 issues
-// one bulk copy for population i (two at the seam).  If the group carries
-// force (band), lanes 19..21 copy the three force-density components of the
-// group's rows; with several droplets lane 22 copies the droplet's constants,
-// with two viscosities lane 23 the rows' inside bits.
-// Every lane announces the bytes of its own copies on the mbarrier
-// (initialised for 32 arrivals) before issuing them.
+// Producer warp: fetch a group into a stage, in two parts.
+// The populations: the source rows of population i for rows y0 .. y0+nr-1 of
+// plane z are rows y0-c_iy .. of plane z-c_iz (or the group's own rows of the
+// opposite population at a wall), which are contiguous in memory except
+// across the periodic y seam: lane i < 19 issues one bulk copy for population
+// i (two at the seam) and adds its bytes to what the mbarrier expects.
+template <typename S>
+__device__ __forceinline__ void produce_populations(const LbConst &c, const S *src, int y0, int z, int nr,
+                                                    unsigned char *sbase, uint64_t *bar)
+{
+    const int i = threadIdx.x & 31;
+    if (i >= Q)
+        return;
+    const int P = c.P, ny = c.ny;
+    const uint32_t rowb = (uint32_t)(P * sizeof(S));
+    // up to two pieces (source row, destination row, rows)
+    int src_pop = i, zs = z - kCz[i], ys = y0 - kCy[i], y_a, n_a, n_b = 0, d_b = 0;
+    if (c.walls && (zs < 0 || zs >= c.nzf)) {
+        src_pop = kOpp[i];          // halfway bounce-back: own rows, opposite population
+        zs = z;
+        ys = y0;
+    } else {
+        zs = wrapi(zs, c.nzf);
+    }
+    if (ys < 0) {                   // first row wraps to y = ny - 1
+        y_a = ny - 1; n_a = 1;
+        n_b = nr - 1; d_b = 1;
+    } else if (ys + nr > ny) {      // last row wraps to y = 0
+        y_a = ys; n_a = ny - ys;
+        n_b = nr - n_a; d_b = n_a;
+    } else {
+        y_a = ys; n_a = nr;
+    }
+    mbar_expect_tx(bar, rowb * (uint32_t)(n_a + n_b));
+    const S *plane = src + (int64_t)Q * c.pcell0 + (int64_t)src_pop * c.PC + (int64_t)P * ny * zs;
+    S *dst = reinterpret_cast<S *>(sbase) + (int64_t)i * c.R * P;
+    const uint64_t pol = l2_evict_first();
+    if (n_a > 0)
+        bulk_g2s_hint(dst, plane + (int64_t)P * y_a, rowb * n_a, bar, pol);
+    if (n_b > 0)
+        bulk_g2s_hint(dst + (int64_t)d_b * P, plane, rowb * n_b, bar, pol);
+}
+
+// What this step's earlier kernels wrote, and the header: if the group carries
+// force (band), lanes 19..21 copy the three force-density components of its
+// rows; with several droplets lane 22 copies the droplet's constants, with
+// two viscosities lane 23 the rows' inside bits.  Every lane announces the
+// bytes of its own copies with its arrival on the mbarrier (initialised for
+// 32) before issuing them.
 template <typename S, bool VARTAU>
-__device__ __forceinline__ void produce(const Arrays &a, const LbConst &c, int d, const S *src, int y0, int z, int nr,
-                                        unsigned char *sbase, uint64_t *bar, bool band)
+__device__ __forceinline__ void produce_rest(const Arrays &a, const LbConst &c, int d, int y0, int z, int nr,
+                                             unsigned char *sbase, uint64_t *bar, bool band)
 {
     const int lane = threadIdx.x & 31;
-    const int P = c.P, ny = c.ny, R = c.R;
+    const int P = c.P, R = c.R;
     Stage<S> stg(sbase, R, P);
-    const int64_t plane_row0 = (int64_t)ny * z;
-    const uint32_t rowb = (uint32_t)(P * sizeof(S));
-    // copies of this lane: up to two pieces (source row, destination row, rows)
-    int src_pop = 0, src_z = 0, y_a = 0, n_a = 0, y_b = 0, n_b = 0, d_b = 0;
+    const int64_t row0 = (int64_t)c.ny * z + y0;
     uint32_t mine = 0;
-    if (lane < Q) {
-        const int i = lane;
-        int zs = z - kCz[i], ys = y0 - kCy[i];
-        src_pop = i;
-        if (c.walls && (zs < 0 || zs >= c.nzf)) {
-            src_pop = kOpp[i];          // halfway bounce-back: own rows, opposite population
-            zs = z;
-            ys = y0;
-        } else {
-            zs = wrapi(zs, c.nzf);
-        }
-        src_z = zs;
-        if (ys < 0) {                   // first row wraps to y = ny - 1
-            y_a = ny - 1; n_a = 1;
-            y_b = 0; n_b = nr - 1; d_b = 1;
-        } else if (ys + nr > ny) {      // last row wraps to y = 0
-            y_a = ys; n_a = ny - ys;
-            y_b = 0; n_b = nr - n_a; d_b = n_a;
-        } else {
-            y_a = ys; n_a = nr;
-        }
-        mine = rowb * (uint32_t)(n_a + n_b);
-    } else if (band && lane < Q + 3) {
+    if (band && lane >= Q && lane < Q + 3)
         mine = (uint32_t)(nr * P * sizeof(float));
-    } else if (lane == Q + 3 && a.ndrops > 1) {
+    else if (lane == Q + 3 && a.ndrops > 1)
         mine = sizeof(LbConst);
-    } else if (VARTAU && lane == Q + 4) {
+    else if (VARTAU && lane == Q + 4)
         mine = (uint32_t)(nr * c.mask_pitch);
-    }
     int4 *header = stage_header(sbase, a);
     if (lane == 0)
         *header = make_int4(band, d, y0, (nr << 16) | z);
     mbar_arrive_expect_tx(bar, mine);
-    if (lane < Q) {
-        const S *plane = src + (int64_t)Q * c.pcell0 + (int64_t)src_pop * c.PC + (int64_t)P * ny * src_z;
-        S *dst = stg.pop + (int64_t)lane * R * P;
-        const uint64_t pol = l2_evict_first();
-        if (n_a > 0)
-            bulk_g2s_hint(dst, plane + (int64_t)P * y_a, rowb * n_a, bar, pol);
-        if (n_b > 0)
-            bulk_g2s_hint(dst + (int64_t)d_b * P, plane + (int64_t)P * y_b, rowb * n_b, bar, pol);
-    } else if (band && lane < Q + 3) {
+    if (band && lane >= Q && lane < Q + 3) {
         const int k = lane - Q;
-        bulk_g2s(stg.F + (int64_t)k * R * P, a.F + k * a.total_pcells + c.pcell0 + (int64_t)P * (plane_row0 + y0),
-                 (uint32_t)(nr * P * sizeof(float)), bar);
+        bulk_g2s(stg.F + (int64_t)k * R * P, a.F + k * a.total_pcells + c.pcell0 + (int64_t)P * row0, mine, bar);
     } else if (lane == Q + 3 && a.ndrops > 1) {
         bulk_g2s(header + 1, a.lbc + d, sizeof(LbConst), bar);
     } else if (VARTAU && lane == Q + 4 && c.mask_pitch) {
-        bulk_g2s(stg.mask, a.mask + c.mask0 + c.mask_pitch * (plane_row0 + y0), (uint32_t)(nr * c.mask_pitch), bar);
+        bulk_g2s(stg.mask, a.mask + c.mask0 + c.mask_pitch * row0, mine, bar);
     }
 }
 
@@ -573,18 +577,13 @@ __device__ __forceinline__ void collide_pairs(const Arrays &a, const LbConst &c,
 template <typename S, bool VARTAU, bool TR>
 __global__ void __launch_bounds__(lb_block<S>(), 2)
     lb_kernel(Arrays a, const S *__restrict__ src, S *__restrict__ dst, int ns, const int *__restrict__ list,
-              const int *__restrict__ count, int no_force, unsigned long long *tr)
+              const int *__restrict__ count, int no_force, int early, unsigned long long *tr)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     // full[s]: the stage's bulk copies landed (32 producer lanes arrive with
     // the byte count); empty[s]: every consumer thread is done reading it
     __shared__ __align__(8) uint64_t full[LB_MAX_STAGES], empty[LB_MAX_STAGES];
-    griddep_wait();
-    if constexpr (TR)
-        lb_trace_start(tr);
-    const uint32_t gen = *a.gen;
-    // the groups of this launch: list[0 .. *count) or all of them
-    const int total = list ? *count : a.lb_blocks_total;
+    const bool producer = threadIdx.x >= cons_threads<S>();
     if (threadIdx.x == 0) {
         for (int i = 0; i < ns; ++i) {
             mbar_init(&full[i], 32);
@@ -598,12 +597,34 @@ __global__ void __launch_bounds__(lb_block<S>(), 2)
     // stage as soon as the consumers released its previous use, so up to ns
     // groups are in flight; each consumer warp moves on to the next group as
     // soon as its data landed, without waiting for the other warps.
+    // Before the wait for the previous kernel (early: at least two kernels of
+    // this step came between this one and the last writer of the populations,
+    // each of which waited for its predecessor, so that writer has completed),
+    // the populations of the first ns groups are requested: they travel while
+    // the previous kernel drains.  The group table and the droplets' constants
+    // are not written by any kernel.
+    const int stride = gridDim.x;
+    int total = a.lb_blocks_total, ahead = 0;
+    if (producer && early) {
+        asm volatile("fence.proxy.async;" ::: "memory");
+        for (int ig = blockIdx.x; ahead < ns && ig < total; ig += stride, ++ahead) {
+            const int4 e = a.grp[ig];
+            const LbConst c = a.lbc[e.x];
+            produce_populations<S>(c, src, e.y, e.z, e.w, smem_raw + ahead * a.lb_stage_bytes, &full[ahead]);
+        }
+    }
+    griddep_wait();
+    if constexpr (TR)
+        lb_trace_start(tr);
+    const uint32_t gen = *a.gen;
+    // the groups of this launch: list[0 .. *count) or all of them
+    if (list)
+        total = *count;
     bool failed = false;
-    if (threadIdx.x >= cons_threads<S>()) {
+    if (producer) {
         int st_i = 0, d = -1;
         uint32_t use = 0, bits = 0;
         LbConst c;
-        const int stride = gridDim.x;
         int4 next = make_int4(0, 0, 0, 0);
         if ((int)blockIdx.x < total)
             next = a.grp[list ? list[blockIdx.x] : blockIdx.x];
@@ -619,15 +640,18 @@ __global__ void __launch_bounds__(lb_block<S>(), 2)
                 d = e.x;
                 c = a.lbc[d];
             }
-            if (use > 0 && !mbar_wait_bounded(&empty[st_i], (use - 1) & 1u, WAIT_CYCLES)) {
-                failed = true;
-                break;
+            unsigned char *base = smem_raw + st_i * a.lb_stage_bytes;
+            if (k >= ahead) {
+                if (use > 0 && !mbar_wait_bounded(&empty[st_i], (use - 1) & 1u, WAIT_CYCLES)) {
+                    failed = true;
+                    break;
+                }
+                // order the consumers' generic reads of the stage before the
+                // asynchronous writes into it
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                produce_populations<S>(c, src, e.y, e.z, e.w, base, &full[st_i]);
             }
-            // order the consumers' generic reads of the stage before the
-            // asynchronous writes into it
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            produce<S, VARTAU>(a, c, d, src, e.y, e.z, e.w, smem_raw + st_i * a.lb_stage_bytes, &full[st_i],
-                       ((bits >> (k & 31)) & 1u) != 0);
+            produce_rest<S, VARTAU>(a, c, d, e.y, e.z, e.w, base, &full[st_i], ((bits >> (k & 31)) & 1u) != 0);
             if (++st_i == ns) {
                 st_i = 0;
                 ++use;
@@ -678,7 +702,7 @@ __global__ void __launch_bounds__(lb_block<S>(), 2)
 }
 template <typename S>
 cudaError_t launch_t(const Arrays &a, const void *src, void *dst, bool vartau, const LaunchCfg &cfg,
-                     cudaStream_t s, const int *list, const int *count, bool no_force, int blocks_per_sm)
+                     cudaStream_t s, const int *list, const int *count, bool no_force, int blocks_per_sm, bool early)
 {
     const int total = a.lb_blocks_total;      // at most this many groups in a list
     if (total <= 0)
@@ -702,18 +726,18 @@ cudaError_t launch_t(const Arrays &a, const void *src, void *dst, bool vartau, c
         per_sm = want;
     int grid = cfg.sm_count * per_sm;
     grid = grid < total ? grid : total;
-    const int nf = no_force ? 1 : 0;
+    const int nf = no_force ? 1 : 0, ea = early && !list ? 1 : 0;
     unsigned long long *tr = g_trace_lb;
     const dim3 g(grid), b(lb_block<S>());
     if (vartau)
         return traced ? launch_k(lb_kernel<S, true, true>, g, b, smem, s, a.pdl != 0, a, (const S *)src, (S *)dst, ns,
-                                 list, count, nf, tr)
+                                 list, count, nf, ea, tr)
                       : launch_k(lb_kernel<S, true, false>, g, b, smem, s, a.pdl != 0, a, (const S *)src, (S *)dst, ns,
-                                 list, count, nf, tr);
+                                 list, count, nf, ea, tr);
     return traced ? launch_k(lb_kernel<S, false, true>, g, b, smem, s, a.pdl != 0, a, (const S *)src, (S *)dst, ns, list,
-                             count, nf, tr)
+                             count, nf, ea, tr)
                   : launch_k(lb_kernel<S, false, false>, g, b, smem, s, a.pdl != 0, a, (const S *)src, (S *)dst, ns,
-                             list, count, nf, tr);
+                             list, count, nf, ea, tr);
 }
 
 }  // namespace
@@ -733,12 +757,12 @@ int lb_stage_bytes(int rows, int pitch, int sb, bool several, int mask_pitch)
 
 cudaError_t launch_lb(const Arrays &a, int storage, const void *src, void *dst, bool vartau,
                       const LaunchCfg &cfg, cudaStream_t s, const int *list, const int *count, bool no_force,
-                      int blocks_per_sm)
+                      int blocks_per_sm, bool early)
 {
     switch (storage) {
-    case 0: return launch_t<float>(a, src, dst, vartau, cfg, s, list, count, no_force, blocks_per_sm);
-    case 1: return launch_t<__half>(a, src, dst, vartau, cfg, s, list, count, no_force, blocks_per_sm);
-    case 2: return launch_t<__nv_bfloat16>(a, src, dst, vartau, cfg, s, list, count, no_force, blocks_per_sm);
+    case 0: return launch_t<float>(a, src, dst, vartau, cfg, s, list, count, no_force, blocks_per_sm, early);
+    case 1: return launch_t<__half>(a, src, dst, vartau, cfg, s, list, count, no_force, blocks_per_sm, early);
+    case 2: return launch_t<__nv_bfloat16>(a, src, dst, vartau, cfg, s, list, count, no_force, blocks_per_sm, early);
     }
     return cudaErrorInvalidValue;
 }
