@@ -79,6 +79,10 @@ struct Operand {
 };
 // K-major, row groups `sbo` apart (8 core matrices of K per 1024 bytes)
 __device__ __forceinline__ Operand k_major(const void *p, uint32_t sbo) { return {smem_addr(p), 128, sbo, 256}; }
+// activations: K-major with the 16 row groups of a K group adjacent (2048
+// bytes per K group), so that a CTA's units are one contiguous piece
+constexpr uint32_t A_KGROUP = TC_M * 16;
+__device__ __forceinline__ Operand activations(const void *p) { return {smem_addr(p), A_KGROUP, 128, 2 * A_KGROUP}; }
 // MN-major with mn elements along M or N
 __device__ __forceinline__ Operand mn_major(const void *p, int mn)
 {
@@ -188,54 +192,34 @@ __device__ __forceinline__ void stage_mn_major(uint8_t *dst, const __nv_bfloat16
     }
 }
 
-// The cluster barrier between two layers: operand writes to shared memory
-// (any CTA's) are visible to the tensor cores after it, accumulator reads and
-// writes are ordered across it.  In two halves, so that a thread's global
-// stores go out between them: before the arrival its release would wait for
-// them.
+// all threads of all CTAs of the cluster
 __device__ __forceinline__ void cluster_arrive()
 {
     __syncwarp();
-    asm volatile("fence.proxy.async.shared::cluster;" ::: "memory");
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
 }
 __device__ __forceinline__ void cluster_wait()
 {
     __syncwarp();
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    asm volatile("fence.proxy.async.shared::cluster;" ::: "memory");
 }
 
-// the thread's row, K columns from k0 (8 in a uint4, 4 in a uint2), into the
-// K-major operand at `buf` of every CTA of the cluster
-__device__ __forceinline__ uint32_t operand_at(uint8_t *buf, int k0)
+// the thread's row of an activation operand, from K column k0
+__device__ __forceinline__ uint8_t *row_at(uint8_t *buf, int k0)
 {
     const int r = threadIdx.x & 127;
-    return smem_addr(buf) + (r >> 3) * 4096 + (k0 >> 3) * 128 + (r & 7) * 16 + (k0 & 7) * 2;
+    return buf + (k0 >> 3) * A_KGROUP + (r >> 3) * 128 + (r & 7) * 16 + (k0 & 7) * 2;
 }
-__device__ __forceinline__ uint32_t in_cta(uint32_t addr, int c)
+// `bytes` at `src` to the same place in CTA c of the cluster; their arrival
+// counts on the same mbarrier there
+__device__ __forceinline__ void send(const uint8_t *src, uint32_t bytes, uint64_t *bar, int c)
 {
-    uint32_t dst;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(dst) : "r"(addr), "r"(c));
-    return dst;
-}
-__device__ __forceinline__ void broadcast(uint8_t *buf, int k0, uint4 v)
-{
-    const uint32_t at = operand_at(buf, k0);
-#pragma unroll
-    for (int c = 0; c < CLUSTER; ++c)
-        asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(in_cta(at, c)), "r"(v.x), "r"(v.y),
-                     "r"(v.z), "r"(v.w)
-                     : "memory");
-}
-__device__ __forceinline__ void broadcast(uint8_t *buf, int k0, uint2 v)
-{
-    const uint32_t at = operand_at(buf, k0);
-#pragma unroll
-    for (int c = 0; c < CLUSTER; ++c)
-        asm volatile("st.shared::cluster.v2.b32 [%0], {%1, %2};" ::"r"(in_cta(at, c)), "r"(v.x), "r"(v.y) : "memory");
+    uint32_t dst, rbar;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(dst) : "r"(smem_addr(src)), "r"(c));
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rbar) : "r"(smem_addr(bar)), "r"(c));
+    asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+                 "r"(smem_addr(src)), "r"(bytes), "r"(rbar)
+                 : "memory");
 }
 
 __device__ __forceinline__ uint32_t pack2(float a, float b)
@@ -303,24 +287,25 @@ static_assert(TRAIN_SMEM <= 226 * 1024, "shared memory of one CTA");
 
 // Forward pass (and with TRAIN the loss and the backward pass) of 128
 // samples per cluster.  A layer's product needs every unit of the previous
-// layer, so each CTA writes its 32 units' outputs straight into the operand
-// buffers of all eight CTAs (distributed shared memory) and one cluster
-// barrier separates the layers: seven barriers in place of ten launches with
-// their passes through global memory.  What bounds it is that chain of
-// barriers, products and tanh epilogues (8 per thread), not a throughput:
-// eight CTAs of 512 threads per 128 samples keep each link short, and
-// everything a thread reads from global memory (weights' slices by
-// asynchronous copies in the order of use, biases, labels) is requested
-// before the first barrier.
-// Measured: inference of 200 samples 262 -> 37 us a call (four launches and
-// three copies before); 27 us of a training step at batch 128, about 2.3 us a
-// layer of which 0.6 are the product, 0.7 the barrier and the rest the
-// epilogue and its 64 KB of stores into the other CTAs.
+// layer, so each CTA writes its 32 units' outputs into its own operand buffer
+// and sends that 8 KB piece to the seven others (bulk copies between shared
+// memories, counted on an mbarrier there): no launch, no pass through global
+// memory and no cluster barrier stands between the layers.  Two buffers
+// suffice: a CTA sends into a buffer only after every other one's next data
+// reached it, which they send after their last product from that buffer.
+// What bounds it is the chain of copies, products and tanh epilogues (8 per
+// thread), not a throughput: eight CTAs of 512 threads per 128 samples keep
+// each link short, and everything a thread reads from global memory (weights'
+// slices by asynchronous copies in the order of use, biases, labels) is
+// requested before the first layer.
+// Measured: a training step at batch 128 39 -> 32 us against stores into the
+// other CTAs and a cluster barrier per layer; inference of 200 samples 38 us
+// a call, 14 of them here (262 with four launches and three copies).
 template <bool TRAIN>
 __global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(NET_THREADS, 1) net_kernel(Net g)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
-    __shared__ __align__(8) uint64_t bar;
+    __shared__ __align__(8) uint64_t bar, full[2];     // a product is done; an operand buffer's pieces have arrived
     __shared__ uint32_t tslot;
     uint8_t *sa[2] = {smem + OFF_SA, smem + OFF_SA + A_BYTES};
     const int cta = blockIdx.x & (CLUSTER - 1), m0 = (blockIdx.x / CLUSTER) * TC_M, n0 = cta * UNITS;
@@ -331,7 +316,8 @@ __global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(NET_THREADS, 1
     const int o0 = (cta & (OUT_CTAS - 1)) * OUT_UNITS + 4 * quarter;   // its 4 outputs (CTAs below OUT_CTAS)
 
     if (threadIdx.x == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&bar)) : "memory");
+        for (uint64_t *m : {&bar, &full[0], &full[1]})
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(m)) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) {
@@ -372,16 +358,34 @@ __global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(NET_THREADS, 1
         if (TRAIN)
             load_floats(g.y + (int64_t)src * NOUT + o0, yl);
     }
-    uint32_t parity = 0;
+    uint32_t parity = 0, fparity[2] = {0, 0};
     bool failed = false;
     uint32_t tmem = 0;
-    // one product (the cluster barrier before it ordered everyone's operand
-    // writes): issue, wait for its completion
-    auto product = [&](Operand A, Operand B, int N, int ksteps, bool b_mn) {
+    // The CTA's piece of buffer b (kn columns from k0) is written: make it and
+    // the staged weights visible to the tensor core and the copies, order the
+    // accumulator's readers before its next use, and send it to the others.
+    auto publish = [&](int b, int k0, int kn) {
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncthreads();
+        if (kn && threadIdx.x < CLUSTER && (int)threadIdx.x != cta)
+            send(sa[b] + (k0 >> 3) * A_KGROUP, (uint32_t)(kn >> 3) * A_KGROUP, &full[b], threadIdx.x);
+    };
+    // the product of buffer b (`bytes` of it come from other CTAs) with B
+    auto product = [&](int b, uint32_t bytes, Operand B, int N, int ksteps, bool b_mn) {
         if (!failed) {
-            if (threadIdx.x == 0)
-                issue_mma(tmem, A, B, ksteps, instr_desc(N, false, b_mn), false, &bar);
-            const bool ok = mbar_wait_bounded(&bar, parity);
+            bool ok = true;
+            if (threadIdx.x == 0) {
+                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(&full[b])),
+                             "r"(bytes)
+                             : "memory");
+                ok = mbar_wait_bounded(&full[b], fparity[b]);
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                if (ok)
+                    issue_mma(tmem, activations(sa[b]), B, ksteps, instr_desc(N, false, b_mn), false, &bar);
+            }
+            fparity[b] ^= 1u;
+            ok = ok && mbar_wait_bounded(&bar, parity);
             parity ^= 1u;
             if (__syncthreads_or(!ok)) {
                 failed = true;
@@ -391,6 +395,7 @@ __global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(NET_THREADS, 1
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         }
     };
+    constexpr uint32_t OTHERS = (CLUSTER - 1) * (UNITS / 8) * A_KGROUP;
     uint4 hk1, hk2, hk3, w;              // its activations, kept for the backward pass
     float v[8] = {};
     // the backward pass's dz = dh (1 - h^2)
@@ -428,55 +433,54 @@ __global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(NET_THREADS, 1
         v[e] = live ? tanhf(z) : 0.0f;
     }
     hk1 = pack8(v);
-    cluster_wait();      // every CTA of the cluster runs: its shared memory may be written; TMEM is allocated
-    tmem = tslot;
-    broadcast(sa[0], c0, hk1);
+    *reinterpret_cast<uint4 *>(row_at(sa[0], c0)) = hk1;
     cp_wait<TRAIN ? 5 : 2>();
-    cluster_arrive();
+    cluster_wait();      // every CTA of the cluster runs: its shared memory and barriers may be written
+    publish(0, n0, UNITS);
+    tmem = tslot;
     if (TRAIN)
         store(g.h1, hk1);
-    cluster_wait();
     // hidden layers 2 and 3
-    product(k_major(sa[0], 4096), k_major(smem + OFF_SW1, 4096), UNITS, NH / 16, false);
+    product(0, OTHERS, k_major(smem + OFF_SW1, 4096), UNITS, NH / 16, false);
     if (!failed)
         read_acc(tmem, 8 * quarter, v);
 #pragma unroll
     for (int e = 0; e < 8; ++e)
         v[e] = tanhf(v[e] + b1[e]);
     hk2 = pack8(v);
-    broadcast(sa[1], c0, hk2);
+    *reinterpret_cast<uint4 *>(row_at(sa[1], c0)) = hk2;
     cp_wait<TRAIN ? 4 : 1>();
-    cluster_arrive();
+    publish(1, n0, UNITS);
     if (TRAIN)
         store(g.h2, hk2);
-    cluster_wait();
-    product(k_major(sa[1], 4096), k_major(smem + OFF_SW2, 4096), UNITS, NH / 16, false);
+    product(1, OTHERS, k_major(smem + OFF_SW2, 4096), UNITS, NH / 16, false);
     if (!failed)
         read_acc(tmem, 8 * quarter, v);
 #pragma unroll
     for (int e = 0; e < 8; ++e)
         v[e] = tanhf(v[e] + b2[e]);
     hk3 = pack8(v);
-    broadcast(sa[0], c0, hk3);
+    *reinterpret_cast<uint4 *>(row_at(sa[0], c0)) = hk3;
     cp_wait<TRAIN ? 3 : 0>();
-    cluster_arrive();
+    publish(0, n0, UNITS);
     if (TRAIN)
         store(g.h3, hk3);
-    cluster_wait();
     // output layer, loss gradient 2 (yhat - y) / (S 64) and squared errors
+    const bool out_cta = cta < OUT_CTAS;
     float o[4] = {}, q[4] = {};
-    uint2 t = make_uint2(0, 0);
-    if (cta < OUT_CTAS) {
-        product(k_major(sa[0], 4096), k_major(smem + OFF_SW3, 4096), OUT_UNITS, NH / 16, false);
+    product(0, OTHERS, k_major(smem + OFF_SW3, 4096), OUT_UNITS, out_cta ? NH / 16 : 0, false);
+    if (out_cta) {
         if (!failed)
             read_acc(tmem, 4 * quarter, o);
 #pragma unroll
         for (int e = 0; e < 4; ++e)
             o[e] = o[e] + b3[e];
-        if (!TRAIN) {
-            if (live)
-                store_floats(g.yhat + (int64_t)s * NOUT + o0, o);
-        } else {
+        if (!TRAIN && live)
+            store_floats(g.yhat + (int64_t)s * NOUT + o0, o);
+    }
+    if constexpr (TRAIN) {
+        uint2 t = make_uint2(0, 0);
+        if (out_cta) {
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 const float d = live ? o[e] - yl[e] : 0.0f;
@@ -484,49 +488,47 @@ __global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(NET_THREADS, 1
                 q[e] = d * d;
             }
             t = make_uint2(pack2(o[0], o[1]), pack2(o[2], o[3]));
-            broadcast(sa[1], o0, t);
+            *reinterpret_cast<uint2 *>(row_at(sa[1], o0)) = t;
         }
-    }
-    if constexpr (TRAIN) {
         cp_wait<2>();
-        cluster_arrive();
-        if (live && cta < OUT_CTAS) {
+        publish(1, cta * OUT_UNITS, out_cta ? OUT_UNITS : 0);
+        if (live && out_cta) {
             *reinterpret_cast<uint2 *>(g.dyb + (int64_t)s * NOUT + o0) = t;
             store_floats(g.dy + (int64_t)s * NOUT + o0, o);
             store_floats(g.sq + (int64_t)s * NOUT + o0, q);
         }
-        cluster_wait();
         // d3 = (dy W3) (1 - h3^2)
-        product(k_major(sa[1], 4096), mn_major(smem + OFF_TW3, UNITS), UNITS, NOUT / 16, true);
+        product(1, (OUT_CTAS - out_cta) * (OUT_UNITS / 8) * A_KGROUP, mn_major(smem + OFF_TW3, UNITS), UNITS, NOUT / 16,
+                true);
         if (!failed)
             read_acc(tmem, 8 * quarter, v);
         dtanh(hk3);
         w = pack8(v);
-        broadcast(sa[0], c0, w);
+        *reinterpret_cast<uint4 *>(row_at(sa[0], c0)) = w;
         cp_wait<1>();
-        cluster_arrive();
+        publish(0, n0, UNITS);
         store_f(g.d3);
         store(g.d3b, w);
-        cluster_wait();
         // d2 = (d3 W2) (1 - h2^2)
-        product(k_major(sa[0], 4096), mn_major(smem + OFF_TW2, UNITS), UNITS, NH / 16, true);
+        product(0, OTHERS, mn_major(smem + OFF_TW2, UNITS), UNITS, NH / 16, true);
         if (!failed)
             read_acc(tmem, 8 * quarter, v);
         dtanh(hk2);
         w = pack8(v);
-        broadcast(sa[1], c0, w);
+        *reinterpret_cast<uint4 *>(row_at(sa[1], c0)) = w;
         cp_wait<0>();
-        cluster_arrive();
+        publish(1, n0, UNITS);
         store_f(g.d2);
         store(g.d2b, w);
-        cluster_wait();
         // d1 = (d2 W1) (1 - h1^2)
-        product(k_major(sa[1], 4096), mn_major(smem + OFF_TW1, UNITS), UNITS, NH / 16, true);
+        product(1, OTHERS, mn_major(smem + OFF_TW1, UNITS), UNITS, NH / 16, true);
         if (!failed)
             read_acc(tmem, 8 * quarter, v);
         dtanh(hk1);
         store_f(g.d1);
     }
+    cluster_arrive();    // no CTA leaves while its pieces are read or its buffers written
+    cluster_wait();
     if (failed)   // give MMAs still in flight a bounded chance to finish before TMEM is freed
         mbar_wait_bounded(&bar, parity ^ 1u);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -730,7 +732,7 @@ __device__ __forceinline__ void unit_sums(const Update &g, const float *dz, int 
 // the tensor cores, the next 32 units' biases each (with the input layer's
 // weights), the last the loss.  Small tiles because the time of a CTA is its
 // loads and its divisions: 107 CTAs share both.  Measured: an Adam step at
-// batch 128 766 -> 40 us (15 launches before), 12 of them here.
+// batch 128 766 -> 32 us (15 launches before), 10 of them here.
 __global__ void __launch_bounds__(THREADS, 1) update_kernel(Update g)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
