@@ -932,19 +932,21 @@ __device__ __forceinline__ int find_drop_chunk(const Drop *D, int n, int c)
 // Sums of NV values over the NT threads of a block, in a fixed order: the
 // values go to shared memory, lane l of warp 0 adds entries l, l + 32, ...
 // and the warp's lanes are combined by a shuffle tree.  Few FP64
-// instructions (a warp-wide FP64 instruction is slow on this GPU).  Result
-// in thread 0.
+// instructions (a warp-wide FP64 instruction is slow on this GPU).  Only the
+// first nv values are summed (the others are 0 in every thread).  Result in
+// thread 0.
 template <int NV, int NT>
-__device__ __forceinline__ void block_sum(double *v)
+__device__ __forceinline__ void block_sum(double *v, int nv)
 {
     static_assert(NV * 32 <= NT, "one warp per value");
     __shared__ double sh[NV][NT];
     __shared__ double res[NV];
     for (int k = 0; k < NV; ++k)
-        sh[k][threadIdx.x] = v[k];
+        if (k < nv)
+            sh[k][threadIdx.x] = v[k];
     __syncthreads();
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (w < NV) {           // warp w sums value w
+    if (w < nv) {           // warp w sums value w
         double x = sh[w][lane];
         for (int i = lane + 32; i < NT; i += 32)
             x += sh[w][i];
@@ -954,7 +956,7 @@ __device__ __forceinline__ void block_sum(double *v)
     }
     __syncthreads();
     for (int k = 0; k < NV; ++k)
-        v[k] = res[k];
+        v[k] = k < nv ? res[k] : 0.0;
 }
 
 // (V/V0)^(-1/3) for s = V/V0 given as e = s - 1: the binomial series
@@ -1036,7 +1038,8 @@ __device__ void vc_chunk(const Arrays &a, int c, unsigned long long *tr = nullpt
         v[2] = a.qy[j];
         v[3] = a.qz[j];
     }
-    block_sum<4, NT>(v);
+    // (a chunk beyond the nodes has only the volume to sum)
+    block_sum<4, NT>(v, k * VC_RB < D.nnodes ? 4 : 1);
     double *part = a.red_part + (int64_t)NRED * c;
     if (threadIdx.x == 0) {
         for (int i = 0; i < 4; ++i)
@@ -1052,20 +1055,26 @@ __device__ void vc_chunk(const Arrays &a, int c, unsigned long long *tr = nullpt
         // warp q folds value q of every chunk of the droplet: lane l adds
         // chunks l, l + 32, ... in that order.  Thread 0's acquire and the
         // block barrier order these loads after every chunk's release; they
-        // read L2 (not the non-coherent L1), all of a pass issued at once.
+        // read L2 (not the non-coherent L1), all of a pass issued at once and
+        // the next pass's while this one's are added (2560 chunks: ten round
+        // trips would follow one another in the last block).
         constexpr int U = 8;
         const double *pp = a.red_part + (int64_t)NRED * D.red_chunk0 + w;
-        double x = 0.0;
-        for (int i0 = lane; i0 < D.red_nchunks; i0 += 32 * U) {
-            double t[U];
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const int i = i0 + 32 * u;
-                t[u] = i < D.red_nchunks ? __ldcg(pp + (int64_t)NRED * i) : 0.0;
-            }
+        double x = 0.0, t[U], next[U];
+        const int n = D.red_nchunks;
+        const auto load = [&](double (&r)[U], int i0) {
 #pragma unroll
             for (int u = 0; u < U; ++u)
+                r[u] = i0 + 32 * u < n ? __ldcg(pp + (int64_t)NRED * (i0 + 32 * u)) : 0.0;
+        };
+        load(t, lane);
+        for (int i0 = lane; i0 < n; i0 += 32 * U) {
+            load(next, i0 + 32 * U);
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
                 x += t[u];
+                t[u] = next[u];
+            }
         }
         x = warp_sum(x);
         if (lane == 0)
