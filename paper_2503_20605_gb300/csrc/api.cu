@@ -853,6 +853,8 @@ int enqueue_step(iblb_ctx *c, int par, bool forces_only)
                      a.grp_list + a.total_rows, a.grp_cnt + 1, true, c->lb_far_blocks_per_sm));
         CK(cudaEventRecord(c->ev_join, c->side));
     }
+    // (one kernel per stage: the spread's blocks take the crossings too)
+    const bool faces_in_spread = c->any_vartau && !split && !c->fused_ib;
     if (nodes && c->fused_ib) {
         CK(launch_ib_front(a, c->cfg.ib_blocks_per_sm, s));     // forces and spread: both in the forces phase
         CK(mark(1));
@@ -861,11 +863,11 @@ int enqueue_step(iblb_ctx *c, int par, bool forces_only)
             CK(launch_node_force(a, s));
         CK(mark(1));
         if (nodes)
-            CK(launch_spread(a, s));
+            CK(launch_spread(a, s, faces_in_spread));
     }
     CK(mark(2));
     if (nodes && c->any_vartau && !split)
-        CK(launch_inout(a, s));
+        CK(launch_inout(a, s, !faces_in_spread));
     CK(mark(3));
     if (forces_only)
         return IBLB_OK;

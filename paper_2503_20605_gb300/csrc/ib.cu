@@ -29,6 +29,7 @@
 #include <cuda/atomic>
 
 #include "iblb_internal.h"
+#include "inout.cuh"
 #include "reduce_util.cuh"
 
 namespace iblb {
@@ -1143,7 +1144,12 @@ __global__ void __launch_bounds__(NF_THREADS) node_force_kernel(Arrays a, unsign
     node_forces<EL, true, TR>(a, (int64_t)blockIdx.x * NF_THREADS + threadIdx.x, 0, tr);
 }
 
-template <bool TR>
+// FACES: with two viscosities the blocks go on to the in/out test's faces once
+// their tiles are done, those that had a tile less first: a launch less, and
+// the blocks' uneven ends are filled.  Measured with face_cross_kernel after
+// it -> with FACES (spread and in/out, us): 33.0 -> 28.0 (81 920 faces, step
+// 173.5 -> 171.2), 111 -> 106 (428 800 faces in 32 boxes, step 351 -> 347.6).
+template <bool TR, bool FACES>
 __global__ void __launch_bounds__(SP_THREADS, SP_PER_SM) spread_kernel(Arrays a, unsigned long long *tr)
 {
     griddep_wait();
@@ -1162,6 +1168,10 @@ __global__ void __launch_bounds__(SP_THREADS, SP_PER_SM) spread_kernel(Arrays a,
     const LeftTile first = zero_left_first<SP_THREADS>(a, cur, blockIdx.x);
     spread_tiles<SP_THREADS>(a, gen, cur, blockIdx.x, gridDim.x, sm);
     zero_left_tiles<SP_THREADS>(a, gen, cur, blockIdx.x, gridDim.x, first);
+    if (FACES)
+        for (int t = (gridDim.x - 1 - blockIdx.x) * SP_THREADS + threadIdx.x; t < a.total_tri;
+             t += gridDim.x * SP_THREADS)
+            face_cross(a, t);
     spread_finish(a, gen, cur, sm);
 }
 
@@ -1318,14 +1328,14 @@ cudaError_t launch_node_force(const Arrays &a, cudaStream_t s)
                                  (unsigned long long *)nullptr);
 }
 
-cudaError_t launch_spread(const Arrays &a, cudaStream_t s)
+cudaError_t launch_spread(const Arrays &a, cudaStream_t s, bool faces)
 {
     if (a.total_nodes <= 0)
         return cudaSuccess;
-    const dim3 grid(sm_count() * SP_PER_SM);
-    return g_trace_ib ? launch_k(spread_kernel<true>, grid, dim3(SP_THREADS), 0, s, a.pdl != 0, a, g_trace_ib)
-                      : launch_k(spread_kernel<false>, grid, dim3(SP_THREADS), 0, s, a.pdl != 0, a,
-                                 (unsigned long long *)nullptr);
+    const dim3 grid(sm_count() * SP_PER_SM), block(SP_THREADS);
+    auto *kernel = faces ? (g_trace_ib ? spread_kernel<true, true> : spread_kernel<false, true>)
+                         : (g_trace_ib ? spread_kernel<true, false> : spread_kernel<false, false>);
+    return launch_k(kernel, grid, block, 0, s, a.pdl != 0, a, g_trace_ib);
 }
 
 void set_trace_ib(unsigned long long *trace) { g_trace_ib = trace; }

@@ -274,8 +274,10 @@ cudaError_t launch_lb(const Arrays &a, int storage, const void *src, void *dst, 
 // the others; also marks the tile rows that may hold band tiles.
 cudaError_t launch_classify(const Arrays &a, cudaStream_t s);
 cudaError_t launch_node_force(const Arrays &a, cudaStream_t s);
-cudaError_t launch_spread(const Arrays &a, cudaStream_t s);
-cudaError_t launch_inout(const Arrays &a, cudaStream_t s);
+// faces: the spread's blocks also find the in/out test's crossings
+cudaError_t launch_spread(const Arrays &a, cudaStream_t s, bool faces = false);
+// in/out test; faces false: the crossings were found by the spread's launch
+cudaError_t launch_inout(const Arrays &a, cudaStream_t s, bool faces = true);
 cudaError_t launch_interp_advect(const Arrays &a, cudaStream_t s);
 // cooperative kernels: forces + tile lists + spread; advection + volume correction
 // (per_sm: resident blocks per SM of the cooperative grid, 0 = as many as fit)

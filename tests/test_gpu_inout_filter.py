@@ -80,3 +80,28 @@ def test_batch_with_one_viscosity_beside_two():
             np.testing.assert_array_equal(got, want)
     finally:
         iblb.iblb_destroy(c)
+
+
+@pytest.mark.parametrize("level,R,box,n", [(1, 6.0, 24, 1), (3, 8.0, 28, 2), (6, 34.0, 80, 4)])
+def test_crossings_from_the_spread_and_from_their_own_kernel(level, R, box, n):
+    """One kernel per stage lets the spread's blocks take the faces (from far
+    fewer faces than threads to several passes over them); with the fused
+    membrane kernels they have a launch of their own."""
+    meshes = [_rotated(level, R, (box / 2 + 0.3, box / 2, box / 2 - 0.2), k) for k in range(n)]
+    got = []
+    for fused in (0, 1):
+        c = iblb.iblb_batch_create([iblb.lattice_desc(box, box, box, tau_out=0.9, lam=2.0) for _ in meshes],
+                                   [iblb.physics_desc(sigma=0.01, theta_eq_deg=90.0, xi=2.0) for _ in meshes],
+                                   stream())
+        try:
+            iblb.iblb_set_option(c, iblb.IBLB_OPT_FUSED_IB, fused)
+            for k, m in enumerate(meshes):
+                iblb.iblb_set_membrane(c, k, *m)
+            iblb.iblb_step(c, 3)
+            got.append([(iblb.iblb_get_inside(c, k), iblb.iblb_get_nodes(c, k)) for k in range(n)])
+        finally:
+            iblb.iblb_destroy(c)
+    for (ia, na), (ib, nb) in zip(*got):
+        assert ia.any()
+        np.testing.assert_array_equal(ia, ib)
+        np.testing.assert_array_equal(na, nb)
