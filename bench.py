@@ -151,7 +151,7 @@ def launches_per_step(spec):
     specs = spec if isinstance(spec, list) else [spec]
     n = 1 + 1 + 1 + 1                # forces and tile lists; spread; stream-collide; interpolation + advection
     if any(w.lam != 1.0 for w in specs):
-        n += 3                       # column reset, face crossings, column sort
+        n += 1                       # inside bits of the crossings, which the spread's blocks found
     if any(w.volume_correction for w in specs):
         n += 1                       # FP64 volume and centroid, rescale (one cooperative launch)
     return n

@@ -59,8 +59,6 @@ __device__ __forceinline__ float cvt(__nv_bfloat16 v) { return __bfloat162float(
 // population stores are streamed (evict-first in L2): they are read again
 // only in the next step
 __device__ __forceinline__ void st(float *p, float v) { __stcs(p, v); }
-__device__ __forceinline__ void st(__half *p, float v) { __stcs(p, __float2half_rn(v)); }
-__device__ __forceinline__ void st(__nv_bfloat16 *p, float v) { __stcs(p, __float2bfloat16_rn(v)); }
 
 __constant__ int kCy[Q] = {0, 0, 0, 1, -1, 0, 0, 1, -1, -1, 1, 1, -1, 1, -1, 0, 0, 0, 0};
 __constant__ int kCz[Q] = {0, 0, 0, 0, 0, 1, -1, 0, 0, 0, 0, 1, -1, -1, 1, 1, -1, -1, 1};
