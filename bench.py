@@ -409,7 +409,7 @@ def run_mlp(I, iblb, torch):
     flop_step = 3 * flop_fwd * 256                            # forward + backward (two GEMMs per layer)
     return {"train_step_ms": dt / steps * 1e3, "train_tflops": flop_step * steps / dt / 1e12,
             "predict_200_ms": dp * 1e3, "bf16_peak_sustained_tflops": peaks_bf16(),
-            "note": "latency-bound: 128 x 256 x 256 tiles, one CTA per 128 rows"}
+            "note": "latency-bound: a chain of layers, eight CTAs per 128 samples"}
 
 
 def peaks_bf16():
