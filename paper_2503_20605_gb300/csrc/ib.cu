@@ -1138,10 +1138,27 @@ constexpr int NF_THREADS = 64;   // block size of the force kernel (16 nodes): s
                                  // mesh of ten thousand nodes spreads evenly over every SM (641
                                  // blocks; 128-thread blocks measured 0.1-0.3 us slower per step)
 
-template <bool EL, bool TR>
-__global__ void __launch_bounds__(NF_THREADS) node_force_kernel(Arrays a, unsigned long long *tr)
+// Order of the force kernel's blocks.  Block b works on piece b for small
+// meshes; from FORCE_SPREAD blocks an SM on (39 000 nodes on 152 SMs), blocks
+// b, b + sms, .. take consecutive pieces, so that the blocks in flight come
+// from sms distant parts of the meshes instead of one neighbourhood whose
+// nodes all count themselves into the same tiles at once.  Measured (force
+// kernel, us, in order -> spread out): 250 368 nodes in 64 boxes 55.7 -> 49.6,
+// 214 464 in 32 boxes 49.3 -> 43.9, 163 842 on one 35.7 -> 33.0, 40 962 on one
+// 12.2 -> 12.2; fewer make one wave, whose order does not matter.  The
+// interpolation, whose blocks share what they read, loses by it (53 -> 60), and
+so does a warp whose eight nodes lie apart (50 -> 66: their loads no longer
+coalesce).
+constexpr int FORCE_SPREAD = 16;
+__device__ __forceinline__ int64_t force_piece(int sms)
 {
-    node_forces<EL, true, TR>(a, (int64_t)blockIdx.x * NF_THREADS + threadIdx.x, 0, tr);
+    return sms ? (int64_t)(blockIdx.x % sms) * (gridDim.x / sms) + blockIdx.x / sms : (int64_t)blockIdx.x;
+}
+
+template <bool EL, bool TR>
+__global__ void __launch_bounds__(NF_THREADS) node_force_kernel(Arrays a, int sms, unsigned long long *tr)
+{
+    node_forces<EL, true, TR>(a, force_piece(sms) * NF_THREADS + threadIdx.x, 0, tr);
 }
 
 // FACES: with two viscosities the blocks go on to the in/out test's faces once
@@ -1316,15 +1333,17 @@ cudaError_t launch_node_force(const Arrays &a, cudaStream_t s)
 {
     if (a.total_nodes <= 0)
         return cudaSuccess;
-    const dim3 grid((unsigned)(((int64_t)a.total_nodes * NL + NF_THREADS - 1) / NF_THREADS));
+    const int64_t blocks = ((int64_t)a.total_nodes * NL + NF_THREADS - 1) / NF_THREADS;
+    const int sms = blocks >= FORCE_SPREAD * (int64_t)sm_count() ? sm_count() : 0;
+    const dim3 grid((unsigned)(sms ? (blocks + sms - 1) / sms * sms : blocks));     // whole pieces per SM
     if (a.fref)
-        return g_trace_ib ? launch_k(node_force_kernel<true, true>, grid, dim3(NF_THREADS), 0, s, a.pdl != 0, a,
+        return g_trace_ib ? launch_k(node_force_kernel<true, true>, grid, dim3(NF_THREADS), 0, s, a.pdl != 0, a, sms,
                                      g_trace_ib)
-                          : launch_k(node_force_kernel<true, false>, grid, dim3(NF_THREADS), 0, s, a.pdl != 0, a,
+                          : launch_k(node_force_kernel<true, false>, grid, dim3(NF_THREADS), 0, s, a.pdl != 0, a, sms,
                                      (unsigned long long *)nullptr);
-    return g_trace_ib ? launch_k(node_force_kernel<false, true>, grid, dim3(NF_THREADS), 0, s, a.pdl != 0, a,
+    return g_trace_ib ? launch_k(node_force_kernel<false, true>, grid, dim3(NF_THREADS), 0, s, a.pdl != 0, a, sms,
                                  g_trace_ib)
-                      : launch_k(node_force_kernel<false, false>, grid, dim3(NF_THREADS), 0, s, a.pdl != 0, a,
+                      : launch_k(node_force_kernel<false, false>, grid, dim3(NF_THREADS), 0, s, a.pdl != 0, a, sms,
                                  (unsigned long long *)nullptr);
 }
 

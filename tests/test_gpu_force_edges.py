@@ -11,7 +11,7 @@ import pytest
 import oracle.oracle as O
 from paper_2503_20605_gb300 import iblb
 from paper_2503_20605_gb300 import inputs as I
-from gpu_util import pair, rel_l2
+from gpu_util import pair, rel_l2, stream
 
 pytestmark = pytest.mark.gpu
 
@@ -54,3 +54,29 @@ def test_heights_near_the_wall_without_a_guard(gap):
     xyz, tri = I.icosphere(2, 3.0, (8.0, 8.0, 0.5 + 3.0 + gap))
     xyz[:, 2] = np.maximum(xyz[:, 2], 0.5 + gap)
     _check(xyz, tri, nx=16, ny=16, nz=16, theta=120.0, xi=1.5, h_min_frac=0.0)
+
+
+@pytest.mark.parametrize("n", [3, 4, 5])
+def test_block_order_of_large_batches(n):
+    """From 16 blocks an SM on (four L5 meshes on 152 SMs) the force kernel's
+    blocks take their pieces in another order, the grid rounded up to whole
+    pieces: every droplet as alone, bit for bit."""
+    box = 64
+    meshes = [I.icosphere(5, 20.0 + 0.5 * k, (32.2, 31.7, 31.5 + 0.1 * k)) for k in range(n)]
+
+    def run(ms):
+        c = iblb.iblb_batch_create([iblb.lattice_desc(box, box, box, tau_out=0.9) for _ in ms],
+                                   [iblb.physics_desc(sigma=0.01, theta_eq_deg=80.0, xi=2.0) for _ in ms], stream())
+        try:
+            for k, m in enumerate(ms):
+                iblb.iblb_set_membrane(c, k, *m)
+            iblb.iblb_step(c, 2)
+            return [(iblb.iblb_get_nodes(c, k), iblb.iblb_get_node_forces(c, k)) for k in range(len(ms))]
+        finally:
+            iblb.iblb_destroy(c)
+
+    together = run(meshes)
+    for m, (xyz, phi) in zip(meshes, together):
+        alone = run([m])[0]
+        np.testing.assert_array_equal(xyz, alone[0])
+        np.testing.assert_array_equal(phi, alone[1])
