@@ -1147,8 +1147,8 @@ constexpr int NF_THREADS = 64;   // block size of the force kernel (16 nodes): s
 // 214 464 in 32 boxes 49.3 -> 43.9, 163 842 on one 35.7 -> 33.0, 40 962 on one
 // 12.2 -> 12.2; fewer make one wave, whose order does not matter.  The
 // interpolation, whose blocks share what they read, loses by it (53 -> 60), and
-so does a warp whose eight nodes lie apart (50 -> 66: their loads no longer
-coalesce).
+// so does a warp whose eight nodes lie apart (50 -> 66: their loads no longer
+// coalesce).
 constexpr int FORCE_SPREAD = 16;
 __device__ __forceinline__ int64_t force_piece(int sms)
 {
