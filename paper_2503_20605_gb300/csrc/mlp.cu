@@ -27,6 +27,7 @@
 
 #include "../../include/iblb.h"
 #include "iblb_internal.h"
+#include "mlp_exchange.h"
 
 using namespace iblb;
 
@@ -40,9 +41,10 @@ constexpr float BETA1 = 0.9f, BETA2 = 0.999f, ADAM_EPS = 1e-8f;
 constexpr int TC_M = 128;            // rows of one tcgen05.mma (samples, or units of a weight gradient)
 constexpr int THREADS = 256;         // update kernel: warp w reads TMEM lanes 32 (w mod 4) .., columns of half w / 4
 constexpr int NET_THREADS = 512;     // forward / backward kernel: columns of quarter w / 4
-constexpr int CLUSTER = 8;           // CTAs per 128 samples: CTA c owns units 32c .. 32c + 31 of a hidden layer
+constexpr int CLUSTER = EX_CTAS;     // CTAs per 128 samples
 constexpr int UNITS = NH / CLUSTER;
-constexpr int OUT_CTAS = 4, OUT_UNITS = NOUT / OUT_CTAS;   // the output layer: 16 units on each of four CTAs
+constexpr int OUT_CTAS = EX_OUT, OUT_UNITS = NOUT / OUT_CTAS;   // the output layer: 16 units on each of four CTAs
+static_assert(EX_H1.units == UNITS && EX_DY.units == OUT_UNITS, "pieces of a layer");
 constexpr long long TC_WAIT_CYCLES = 1000000000LL;   // ~0.5 s: bounded barrier wait
 
 __device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -291,8 +293,8 @@ static_assert(TRAIN_SMEM <= 226 * 1024, "shared memory of one CTA");
 // and sends that 8 KB piece to the seven others (bulk copies between shared
 // memories, counted on an mbarrier there): no launch, no pass through global
 // memory and no cluster barrier stands between the layers.  Two buffers
-// suffice: a CTA sends into a buffer only after every other one's next data
-// reached it, which they send after their last product from that buffer.
+// suffice with the senders and receivers of mlp_exchange.h, which shows that a
+// CTA sends into a buffer only after every receiver's last product from it.
 // What bounds it is the chain of copies, products and tanh epilogues (8 per
 // thread), not a throughput: eight CTAs of 512 threads per 128 samples keep
 // each link short, and everything a thread reads from global memory (weights'
@@ -358,22 +360,27 @@ __global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(NET_THREADS, 1
         if (TRAIN)
             load_floats(g.y + (int64_t)src * NOUT + o0, yl);
     }
+    constexpr Exchange h1 = EX_H1, h2 = EX_H2, h3 = EX_H3, dy = EX_DY, d3 = EX_D3, d2 = EX_D2;
     uint32_t parity = 0, fparity[2] = {0, 0};
     bool failed = false;
     uint32_t tmem = 0;
-    // The CTA's piece of buffer b (kn columns from k0) is written: make it and
-    // the staged weights visible to the tensor core and the copies, order the
-    // accumulator's readers before its next use, and send it to the others.
-    auto publish = [&](int b, int k0, int kn) {
+    // The CTA's piece of the exchange is written: make it and the staged
+    // weights visible to the tensor core and the copies, order the
+    // accumulator's readers before its next use, and send it to the receivers.
+    auto publish = [&](const Exchange &x) {
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncthreads();
-        if (kn && threadIdx.x < CLUSTER && (int)threadIdx.x != cta)
-            send(sa[b] + (k0 >> 3) * A_KGROUP, (uint32_t)(kn >> 3) * A_KGROUP, &full[b], threadIdx.x);
+        if (cta < x.senders && (int)threadIdx.x < x.receivers && (int)threadIdx.x != cta)
+            send(sa[x.buffer] + (x.units * cta >> 3) * A_KGROUP, (uint32_t)(x.units >> 3) * A_KGROUP, &full[x.buffer],
+                 threadIdx.x);
     };
-    // the product of buffer b (`bytes` of it come from other CTAs) with B
-    auto product = [&](int b, uint32_t bytes, Operand B, int N, int ksteps, bool b_mn) {
-        if (!failed) {
+    // a receiver's product of the exchange's buffer with B, once the other
+    // senders' pieces are in
+    auto product = [&](const Exchange &x, Operand B, int N, bool b_mn) {
+        if (!failed && cta < x.receivers) {
+            const int b = x.buffer, ksteps = x.senders * x.units / 16;
+            const uint32_t bytes = (uint32_t)(x.senders - (cta < x.senders)) * (uint32_t)(x.units >> 3) * A_KGROUP;
             bool ok = true;
             if (threadIdx.x == 0) {
                 asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(&full[b])),
@@ -395,7 +402,6 @@ __global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(NET_THREADS, 1
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         }
     };
-    constexpr uint32_t OTHERS = (CLUSTER - 1) * (UNITS / 8) * A_KGROUP;
     uint4 hk1, hk2, hk3, w;              // its activations, kept for the backward pass
     float v[8] = {};
     // the backward pass's dz = dh (1 - h^2)
@@ -436,12 +442,12 @@ __global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(NET_THREADS, 1
     *reinterpret_cast<uint4 *>(row_at(sa[0], c0)) = hk1;
     cp_wait<TRAIN ? 5 : 2>();
     cluster_wait();      // every CTA of the cluster runs: its shared memory and barriers may be written
-    publish(0, n0, UNITS);
+    publish(h1);
     tmem = tslot;
     if (TRAIN)
         store(g.h1, hk1);
     // hidden layers 2 and 3
-    product(0, OTHERS, k_major(smem + OFF_SW1, 4096), UNITS, NH / 16, false);
+    product(h1, k_major(smem + OFF_SW1, 4096), UNITS, false);
     if (!failed)
         read_acc(tmem, 8 * quarter, v);
 #pragma unroll
@@ -450,10 +456,10 @@ __global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(NET_THREADS, 1
     hk2 = pack8(v);
     *reinterpret_cast<uint4 *>(row_at(sa[1], c0)) = hk2;
     cp_wait<TRAIN ? 4 : 1>();
-    publish(1, n0, UNITS);
+    publish(h2);
     if (TRAIN)
         store(g.h2, hk2);
-    product(1, OTHERS, k_major(smem + OFF_SW2, 4096), UNITS, NH / 16, false);
+    product(h2, k_major(smem + OFF_SW2, 4096), UNITS, false);
     if (!failed)
         read_acc(tmem, 8 * quarter, v);
 #pragma unroll
@@ -462,13 +468,13 @@ __global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(NET_THREADS, 1
     hk3 = pack8(v);
     *reinterpret_cast<uint4 *>(row_at(sa[0], c0)) = hk3;
     cp_wait<TRAIN ? 3 : 0>();
-    publish(0, n0, UNITS);
+    publish(h3);
     if (TRAIN)
         store(g.h3, hk3);
     // output layer, loss gradient 2 (yhat - y) / (S 64) and squared errors
     const bool out_cta = cta < OUT_CTAS;
     float o[4] = {}, q[4] = {};
-    product(0, OTHERS, k_major(smem + OFF_SW3, 4096), OUT_UNITS, out_cta ? NH / 16 : 0, false);
+    product(h3, k_major(smem + OFF_SW3, 4096), OUT_UNITS, false);
     if (out_cta) {
         if (!failed)
             read_acc(tmem, 4 * quarter, o);
@@ -491,37 +497,36 @@ __global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(NET_THREADS, 1
             *reinterpret_cast<uint2 *>(row_at(sa[1], o0)) = t;
         }
         cp_wait<2>();
-        publish(1, cta * OUT_UNITS, out_cta ? OUT_UNITS : 0);
+        publish(dy);
         if (live && out_cta) {
             *reinterpret_cast<uint2 *>(g.dyb + (int64_t)s * NOUT + o0) = t;
             store_floats(g.dy + (int64_t)s * NOUT + o0, o);
             store_floats(g.sq + (int64_t)s * NOUT + o0, q);
         }
         // d3 = (dy W3) (1 - h3^2)
-        product(1, (OUT_CTAS - out_cta) * (OUT_UNITS / 8) * A_KGROUP, mn_major(smem + OFF_TW3, UNITS), UNITS, NOUT / 16,
-                true);
+        product(dy, mn_major(smem + OFF_TW3, UNITS), UNITS, true);
         if (!failed)
             read_acc(tmem, 8 * quarter, v);
         dtanh(hk3);
         w = pack8(v);
         *reinterpret_cast<uint4 *>(row_at(sa[0], c0)) = w;
         cp_wait<1>();
-        publish(0, n0, UNITS);
+        publish(d3);
         store_f(g.d3);
         store(g.d3b, w);
         // d2 = (d3 W2) (1 - h2^2)
-        product(0, OTHERS, mn_major(smem + OFF_TW2, UNITS), UNITS, NH / 16, true);
+        product(d3, mn_major(smem + OFF_TW2, UNITS), UNITS, true);
         if (!failed)
             read_acc(tmem, 8 * quarter, v);
         dtanh(hk2);
         w = pack8(v);
         *reinterpret_cast<uint4 *>(row_at(sa[1], c0)) = w;
         cp_wait<0>();
-        publish(1, n0, UNITS);
+        publish(d2);
         store_f(g.d2);
         store(g.d2b, w);
         // d1 = (d2 W1) (1 - h1^2)
-        product(1, OTHERS, mn_major(smem + OFF_TW1, UNITS), UNITS, NH / 16, true);
+        product(d2, mn_major(smem + OFF_TW1, UNITS), UNITS, true);
         if (!failed)
             read_acc(tmem, 8 * quarter, v);
         dtanh(hk1);
