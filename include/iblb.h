@@ -476,9 +476,17 @@ int iblb_mlp_grad(iblb_mlp *m, const double *x, const double *y, int S, double *
  * beta2 0.999, eps 1e-8, learning rate lr, bias-corrected; the step counter
  * continues across calls).  loss_per_epoch[epochs] (may be NULL) receives
  * the mean batch loss of each epoch.  IBLB_E_TIMEOUT if a bounded wait in
- * the tensor-core kernel gave up. */
+ * the tensor-core kernels gave up: no step follows the one it happened in,
+ * whose update is left out (or, if the wait was the update's own, may be
+ * incomplete), while the step counter goes to the epoch's end.  Create the
+ * network anew from parameters kept before. */
 int iblb_mlp_train(iblb_mlp *m, const double *x, const double *y, int S, int epochs, int batch,
                    double lr, uint64_t seed, double *loss_per_epoch);
+
+/* Record a wait that gave up, as the network's kernels would (they have none
+ * that can be made to): the next call on m returns IBLB_E_TIMEOUT and clears
+ * the record. */
+int iblb_selftest_mlp_give_up(iblb_mlp *m);
 
 #ifdef __cplusplus
 }

@@ -309,6 +309,7 @@ __global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(NET_THREADS, 1
     extern __shared__ __align__(1024) uint8_t smem[];
     __shared__ __align__(8) uint64_t bar, full[2];     // a product is done; an operand buffer's pieces have arrived
     __shared__ uint32_t tslot;
+    __shared__ int gave_up;                            // a wait of an earlier launch did
     uint8_t *sa[2] = {smem + OFF_SA, smem + OFF_SA + A_BYTES};
     const int cta = blockIdx.x & (CLUSTER - 1), m0 = (blockIdx.x / CLUSTER) * TC_M, n0 = cta * UNITS;
     const int warp = threadIdx.x >> 5, row = threadIdx.x & 127, quarter = threadIdx.x >> 7;
@@ -329,6 +330,7 @@ __global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(NET_THREADS, 1
     }
     cluster_arrive();    // waited for before the first write to another CTA
     griddep_wait();
+    const int err = threadIdx.x == 0 ? *g.err : 0;
     float w0[24], b0[8], b1[8], b2[8], b3[4], f[3] = {0.f, 0.f, 0.f}, yl[4] = {0.f, 0.f, 0.f, 0.f};
     int src = 0;
     if (live)
@@ -367,11 +369,15 @@ __global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(NET_THREADS, 1
     // The CTA's piece of the exchange is written: make it and the staged
     // weights visible to the tensor core and the copies, order the
     // accumulator's readers before its next use, and send it to the receivers.
-    auto publish = [&](const Exchange &x) {
+    // A CTA whose wait gave up sends no more: the others' waits for it give up
+    // in turn, long after what they sent it has landed.
+    auto publish = [&](const Exchange &x, bool first = false) {
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncthreads();
-        if (cta < x.senders && (int)threadIdx.x < x.receivers && (int)threadIdx.x != cta)
+        if (first)
+            failed = gave_up != 0;
+        if (!failed && cta < x.senders && (int)threadIdx.x < x.receivers && (int)threadIdx.x != cta)
             send(sa[x.buffer] + (x.units * cta >> 3) * A_KGROUP, (uint32_t)(x.units >> 3) * A_KGROUP, &full[x.buffer],
                  threadIdx.x);
     };
@@ -441,8 +447,10 @@ __global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(NET_THREADS, 1
     hk1 = pack8(v);
     *reinterpret_cast<uint4 *>(row_at(sa[0], c0)) = hk1;
     cp_wait<TRAIN ? 5 : 2>();
+    if (threadIdx.x == 0)
+        gave_up = err;
     cluster_wait();      // every CTA of the cluster runs: its shared memory and barriers may be written
-    publish(h1);
+    publish(h1, true);
     tmem = tslot;
     if (TRAIN)
         store(g.h1, hk1);
@@ -534,8 +542,12 @@ __global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(NET_THREADS, 1
     }
     cluster_arrive();    // no CTA leaves while its pieces are read or its buffers written
     cluster_wait();
-    if (failed)   // give MMAs still in flight a bounded chance to finish before TMEM is freed
+    if (failed) {   // give MMAs and copies still in flight a bounded chance to finish before TMEM and shared memory go
         mbar_wait_bounded(&bar, parity ^ 1u);
+        if (threadIdx.x == 0)
+            for (int b = 0; b < 2; ++b)
+                mbar_wait_bounded(&full[b], fparity[b] ^ 1u);
+    }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (warp == 0) {
@@ -576,7 +588,7 @@ constexpr int UP_BLOCKS = UP_GEMM + UP_RED + 1;      // and the loss
 // Weight gradient tile dW(o, i) = sum_s dz(s, o) h(s, i): both operands are
 // stored sample-major, so they are staged MN-major as they are; the samples
 // run along K in order, UP_K at a time through two buffers.
-__device__ __forceinline__ void weight_grad(const Update &g, uint8_t *smem, uint64_t *bar, uint32_t *tslot)
+__device__ __forceinline__ void weight_grad(const Update &g, uint8_t *smem, uint64_t *bar, uint32_t *tslot, int *gave_up)
 {
     const int t = blockIdx.x / TILES, n0 = (blockIdx.x % TILES) * UP_N;
     const __nv_bfloat16 *A = t < 2 ? g.d3b : (t < 4 ? g.d2b : g.dyb);
@@ -595,6 +607,7 @@ __device__ __forceinline__ void weight_grad(const Update &g, uint8_t *smem, uint
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     griddep_wait();
+    const int err = threadIdx.x == 0 ? *g.err : 0;
     const int chunks = (g.S + UP_K - 1) / UP_K;
     // the thread's 8 parameters and moments, in flight with the operands
     const int row = threadIdx.x & 127, c0 = 8 * (threadIdx.x >> 7);
@@ -614,6 +627,8 @@ __device__ __forceinline__ void weight_grad(const Update &g, uint8_t *smem, uint
         cp_commit();
     };
     stage(0);
+    if (threadIdx.x == 0)
+        *gave_up = err;
     uint32_t tmem = 0, parity = 0;
     bool failed = false;
     for (int c = 0; c < chunks; ++c) {
@@ -623,6 +638,10 @@ __device__ __forceinline__ void weight_grad(const Update &g, uint8_t *smem, uint
         __syncthreads();
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         tmem = *tslot;
+        if (*gave_up) {
+            failed = true;
+            break;
+        }
         const uint8_t *sa = smem + (c & 1) * (UP_A + UP_B), *sb = sa + UP_A;
         if (threadIdx.x == 0)
             issue_mma(tmem, mn_major(sa, TC_M), mn_major(sb, UP_N), (min(UP_K, g.S - c * UP_K) + 15) / 16,
@@ -672,9 +691,10 @@ __device__ __forceinline__ void weight_grad(const Update &g, uint8_t *smem, uint
 // gradient too.
 template <bool U>
 __device__ __forceinline__ void unit_sums(const Update &g, const float *dz, int ld, int64_t off_b, int unit0,
-                                          float (*sh)[32][33])
+                                          float (*sh)[32][33], int *gave_up)
 {
     constexpr int NV = U ? 1 + NIN : 1;
+    const int err = threadIdx.x == 0 ? *g.err : 0;
     const int o = threadIdx.x & 31, w = threadIdx.x >> 5;
     // the parameter that this thread updates: value w of unit o
     const bool mine = w < NV;
@@ -710,8 +730,10 @@ __device__ __forceinline__ void unit_sums(const Update &g, const float *dz, int 
     for (int q = 0; q < 4; ++q)
         for (int k = 0; k < NV; ++k)
             sh[k][4 * w + q][o] = acc[q][k];
+    if (threadIdx.x == 0)
+        *gave_up = err;
     __syncthreads();
-    if (!mine)
+    if (!mine || *gave_up)
         return;
     float t[32];
 #pragma unroll
@@ -736,30 +758,33 @@ __device__ __forceinline__ void unit_sums(const Update &g, const float *dz, int 
 // the loss: CTAs [0, UP_GEMM) one 128 x 16 tile of a weight matrix each on
 // the tensor cores, the next 32 units' biases each (with the input layer's
 // weights), the last the loss.  Small tiles because the time of a CTA is its
-// loads and its divisions: 107 CTAs share both.  Measured: an Adam step at
+// loads and its divisions: 107 CTAs share both.  Once a wait of the net kernel
+// (or of an earlier update) gave up, nothing is updated any more: what the
+// gradients would be formed from is not there.  Measured: an Adam step at
 // batch 128 766 -> 32 us (15 launches before), 10 of them here.
 __global__ void __launch_bounds__(THREADS, 1) update_kernel(Update g)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
     __shared__ __align__(8) uint64_t bar;
     __shared__ uint32_t tslot;
+    __shared__ int gave_up;
     if (blockIdx.x < UP_GEMM) {
-        weight_grad(g, smem, &bar, &tslot);
+        weight_grad(g, smem, &bar, &tslot, &gave_up);
         return;
     }
     griddep_wait();
     const int b = blockIdx.x - UP_GEMM;
     float(*sh)[32][33] = reinterpret_cast<float(*)[32][33]>(smem);
     if (b < NOUT / 32) {
-        unit_sums<false>(g, g.dy, NOUT, OFF_B3, 32 * b, sh);
+        unit_sums<false>(g, g.dy, NOUT, OFF_B3, 32 * b, sh, &gave_up);
     } else if (b < UP_RED) {
         const int k = b - NOUT / 32, layer = k / (NH / 32), u0 = 32 * (k % (NH / 32));
         if (layer == 0)
-            unit_sums<false>(g, g.d3, NH, OFF_B2, u0, sh);
+            unit_sums<false>(g, g.d3, NH, OFF_B2, u0, sh, &gave_up);
         else if (layer == 1)
-            unit_sums<false>(g, g.d2, NH, OFF_B1, u0, sh);
+            unit_sums<false>(g, g.d2, NH, OFF_B1, u0, sh, &gave_up);
         else
-            unit_sums<true>(g, g.d1, NH, OFF_B0, u0, sh);
+            unit_sums<true>(g, g.d1, NH, OFF_B0, u0, sh, &gave_up);
     } else {     // loss = mean of the squared errors, FP64, fixed order
         double *red = reinterpret_cast<double *>(smem);
         double a[4] = {0.0, 0.0, 0.0, 0.0};
@@ -1043,6 +1068,15 @@ int iblb_mlp_get_params(iblb_mlp *m, float *out, int64_t n)
     if (!m || !out || n != NPARAM)
         return mfail(m, IBLB_E_ARG, "iblb_mlp_get_params: bad arguments");
     MCK(cudaMemcpyAsync(out, m->p, sizeof(float) * NPARAM, cudaMemcpyDeviceToHost, m->stream));
+    MCK(cudaStreamSynchronize(m->stream));
+    return IBLB_OK;
+}
+
+int iblb_selftest_mlp_give_up(iblb_mlp *m)
+{
+    if (!m)
+        return mfail(m, IBLB_E_ARG, "iblb_selftest_mlp_give_up: null network");
+    MCK(cudaMemsetAsync(m->err, 1, 1, m->stream));
     MCK(cudaStreamSynchronize(m->stream));
     return IBLB_OK;
 }

@@ -120,6 +120,7 @@ _SIGS = {
     "iblb_mlp_predict": (C.c_int, [_P, _D, C.c_int, _D]),
     "iblb_mlp_grad": (C.c_int, [_P, _D, _D, C.c_int, _D, _D]),
     "iblb_mlp_train": (C.c_int, [_P, _D, _D, C.c_int, C.c_int, C.c_int, C.c_double, C.c_uint64, _D]),
+    "iblb_selftest_mlp_give_up": (C.c_int, [_P]),
 }
 
 _lib = None
@@ -468,3 +469,9 @@ def iblb_selftest_wait_timeout(cycles, stream=0):
     """Run the bounded mbarrier wait on a barrier that never completes;
     returns the status code (IBLB_E_TIMEOUT is the expected outcome)."""
     return lib().iblb_selftest_wait_timeout(int(cycles), _P(stream))
+
+
+def iblb_selftest_mlp_give_up(m):
+    """Record a wait of the network's kernels that gave up: the next call on
+    m raises IBLB_E_TIMEOUT and clears the record."""
+    _mcheck(m, lib().iblb_selftest_mlp_give_up(m))
