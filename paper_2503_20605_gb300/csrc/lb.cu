@@ -115,6 +115,11 @@ __device__ __forceinline__ uint32_t band_ballot(const Arrays &a, const int *list
     return __ballot_sync(0xffffffffu, band);
 }
 
+// First cell of population i's plane: beyond 32 bits from 119 M cells on (a
+// box may have 2^30, its padded rows up to twice that).
+__host__ __device__ constexpr int64_t plane_offset(int i, int plane_cells) { return (int64_t)i * plane_cells; }
+static_assert(plane_offset(Q - 1, 1 << 30) == 18LL << 30, "no 32-bit product");
+
 // Producer warp: fetch a group into a stage, in two parts.
 // The populations: the source rows of population i for rows y0 .. y0+nr-1 of
 // plane z are rows y0-c_iy .. of plane z-c_iz (or the group's own rows of the
@@ -149,7 +154,7 @@ __device__ __forceinline__ void produce_populations(const LbConst &c, const S *s
         y_a = ys; n_a = nr;
     }
     mbar_expect_tx(bar, rowb * (uint32_t)(n_a + n_b));
-    const S *plane = src + (int64_t)Q * c.pcell0 + (int64_t)src_pop * c.PC + (int64_t)P * ny * zs;
+    const S *plane = src + (int64_t)Q * c.pcell0 + plane_offset(src_pop, c.PC) + (int64_t)P * ny * zs;
     S *dst = reinterpret_cast<S *>(sbase) + (int64_t)i * c.R * P;
     const uint64_t pol = l2_evict_first();
     if (n_a > 0)
@@ -246,7 +251,7 @@ __device__ __forceinline__ void collide_group(const Arrays &a, const LbConst &c,
         S *o = outb + P * y + x;
         if (x >= nx) {      // the row's padding (see the file's head)
             for (int i = 0; i < Q; ++i)
-                st(o + i * PC, 0.0f);
+                st(o + plane_offset(i, PC), 0.0f);
             continue;
         }
         float Fx = 0.0f, Fy = 0.0f, Fz = 0.0f;
@@ -337,8 +342,8 @@ __device__ __forceinline__ void collide_group(const Arrays &a, const LbConst &c,
                 Mm = __fmul_rn(ec, cJ_);                                                                 \
                 Pp = fmaf(__fmul_rn(ea, cu_), cu_, b);                                                   \
             }                                                                                            \
-            st(o + (i) * PC, fmaf(om1, (si), Pp + Mm));                                                  \
-            st(o + (j) * PC, fmaf(om1, (sj), Pp - Mm));                                                  \
+            st(o + plane_offset(i, PC), fmaf(om1, (si), Pp + Mm));                                       \
+            st(o + plane_offset(j, PC), fmaf(om1, (sj), Pp - Mm));                                       \
         }
         PAIR(1, 2, b1, ea1, ec1, kf1, kd1, ux, Jx, Fx, s1, s2);
         PAIR(3, 4, b1, ea1, ec1, kf1, kd1, uy, Jy, Fy, s3, s4);
@@ -567,7 +572,7 @@ __device__ __forceinline__ void collide_pairs(const Arrays &a, const LbConst &c,
         // one store for cells and padding alike, so that sectors go out whole
 #pragma unroll
         for (int i = 0; i < Q; ++i)
-            __stcs(reinterpret_cast<PT *>(o + (int64_t)i * PC), PO::pack(oa[i], ob[i]));
+            __stcs(reinterpret_cast<PT *>(o + plane_offset(i, PC)), PO::pack(oa[i], ob[i]));
 #undef SC
     }
 }
