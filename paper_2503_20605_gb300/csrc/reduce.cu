@@ -336,24 +336,34 @@ int64_t observe_scratch_doubles(int n_nodes, int n_tri)
     return (int64_t)(NRED + 5) * mesh_chunks(n_nodes, n_tri, fpc, npc);
 }
 
+// meshes per launch: a grid has at most this many blocks in y
+constexpr int OBS_GRID_Y = 65535;
+
 // chained by programmatic dependent launch: each kernel waits for the
 // previous one before reading its results
 cudaError_t enqueue_observe(const ObsMesh *table, const ObsMesh *one, int n, int max_chunks, double zcut_frac,
                             double eps_flat, cudaStream_t s)
 {
     const ObsMesh m = one ? *one : ObsMesh{};
-    const dim3 g(max_chunks, n);
-    cudaError_t e;
-    if ((e = launch_k(pass1_kernel, g, dim3(RB), 0, s, true, table, m)) != cudaSuccess ||
-        (e = launch_k(pass2_kernel, g, dim3(RB), 0, s, true, table, m, zcut_frac, eps_flat)) != cudaSuccess)
-        return e;
-    return launch_k(pass3_kernel, g, dim3(RB), 0, s, true, table, m, zcut_frac);
+    cudaError_t e = cudaSuccess;
+    for (int i = 0; i < n && e == cudaSuccess; i += OBS_GRID_Y) {
+        const dim3 g(max_chunks, std::min(n - i, OBS_GRID_Y));
+        const ObsMesh *t = table ? table + i : nullptr;
+        if ((e = launch_k(pass1_kernel, g, dim3(RB), 0, s, true, t, m)) == cudaSuccess &&
+            (e = launch_k(pass2_kernel, g, dim3(RB), 0, s, true, t, m, zcut_frac, eps_flat)) == cudaSuccess)
+            e = launch_k(pass3_kernel, g, dim3(RB), 0, s, true, t, m, zcut_frac);
+    }
+    return e;
 }
 cudaError_t enqueue_observe_result(const ObsMesh *table, const ObsMesh *one, int n, const double *mass,
                                    const int *status, int d0, double *out, cudaStream_t s)
 {
-    return launch_k(obs_result_kernel, dim3(1, n), dim3(FIN_THREADS), 0, s, true, table, one ? *one : ObsMesh{}, mass,
-                    status, d0, out);
+    cudaError_t e = cudaSuccess;
+    for (int i = 0; i < n && e == cudaSuccess; i += OBS_GRID_Y)
+        e = launch_k(obs_result_kernel, dim3(1, std::min(n - i, OBS_GRID_Y)), dim3(FIN_THREADS), 0, s, true,
+                     table ? table + i : nullptr, one ? *one : ObsMesh{}, mass, status, d0 + i,
+                     out + (int64_t)OBS_RAW * i);
+    return e;
 }
 
 // h_out: V, A, cx, cy, cz, zmin, zmax, theta(R0), theta(R_V), rc_cut,
