@@ -439,6 +439,7 @@ void layout(iblb_ctx *c)
     const bool several = c->ndrops > 1;
     c->grp.clear();
     c->lbc.clear();
+    c->A.mask_unstaged = 0;
     c->grp_dirty = true;
     for (auto &D : c->drops) {
         D.cell0 = cell0;
@@ -480,7 +481,10 @@ void layout(iblb_ctx *c)
         k.PC = (int)D.pcells;
         k.nzf = D.nzf;
         k.walls = D.walls;
-        k.vartau = D.vartau;
+        // where two stages of one row fit without the inside bits only, they
+        // are read from global memory
+        k.mask_staged = D.mask_pitch &&
+                        2 * (size_t)lb_stage_bytes(D.lb_rows, D.pitch, sb, several, D.mask_pitch) <= LB_SMEM_LAUNCH;
         k.npr = lb_items_per_row(D.pitch, sb);
         k.step_r = lb_consumers(sb) / k.npr;
         k.step_x = lb_consumers(sb) - k.step_r * k.npr;
@@ -502,7 +506,9 @@ void layout(iblb_ctx *c)
         c->lbc.push_back(k);
         D.mass_block0 = mb0;
         D.mass_nblocks = (int)((D.cells + MASS_CELLS_PER_BLOCK - 1) / MASS_CELLS_PER_BLOCK);
-        stage = std::max(stage, lb_stage_bytes(D.lb_rows, D.pitch, sb, several, D.mask_pitch));
+        c->A.mask_unstaged |= D.mask_pitch && !k.mask_staged;
+        stage = std::max(stage,
+                         lb_stage_bytes(D.lb_rows, D.pitch, sb, several, k.mask_staged ? D.mask_pitch : 0));
         cell0 += D.cells;
         pcell0 += D.pcells;
         row0 += (int64_t)D.ny * D.nzf;

@@ -64,7 +64,7 @@ struct Drop {
 // so that a block that moves to another droplet waits for nothing.
 struct __align__(16) LbConst {
     int nx, ny, P, R;              // P: row pitch, R: rows per group
-    int PC, nzf, walls, vartau;    // PC: cells per population plane
+    int PC, nzf, walls, mask_staged;   // PC: cells per population plane; its inside bits travel with the rows
     int npr, step_r, step_x, tx;   // work items per row and pitch (cells, or pairs of 16-bit cells); the stride of
     int ty;                        // a thread's items in rows and items; tiles per row and column
     float inv_npr;                 // 1 / npr
@@ -103,6 +103,7 @@ struct Arrays {
     int lb_blocks_total;           // row groups of the stream-collide launch
     const int4 *grp;               // per group: droplet, first row y0, plane z, rows
     const LbConst *lbc;            // per droplet
+    int mask_unstaged;             // some droplet's inside bits do not travel in the stages (LbConst::mask_staged)
     int lb_stage_bytes;            // bytes of one shared-memory stage of the stream-collide kernel
     int64_t total_pcells;          // sum of Drop::pcells
     int64_t total_rows;            // sum of ny * nzf
@@ -255,7 +256,9 @@ struct LaunchCfg {
 int lb_rows_per_group(int nx);     // 256-thread groups: max(1, 256 / nx) rows
 // bytes of one stage of the stream-collide kernel: 19 population rows and 3
 // force rows per cell row, its inside bits with two viscosities, the group's
-// header and with several droplets its droplet's constants (128-byte multiple)
+// header and with several droplets its droplet's constants (a multiple of 128
+// bytes; of 16, where two stages of such multiples do not fit a block)
+constexpr size_t LB_SMEM_LAUNCH = 227 * 1024 - 128;   // dynamic shared memory of a block, beside its barriers
 int lb_stage_bytes(int rows, int pitch, int storage_bytes, bool several, int mask_pitch);
 // work items per row and consumer threads per block, for LbConst
 int lb_items_per_row(int pitch, int storage_bytes);

@@ -74,8 +74,9 @@ constexpr float W0 = 1.0f / 3.0f, W1 = 1.0f / 18.0f, W2 = 1.0f / 36.0f;
 constexpr float K2 = 1.0f / 12.0f, K1 = (1.0f - 8.0f * K2) * 0.5f;
 
 // stage layout: [19][R][P] populations | [3][R][P] force | with two
-// viscosities [R][mask_pitch] inside bits | header (int4: band flag, droplet, first row y0, rows << 16 | plane z) | with several droplets
-// the group's LbConst
+// viscosities [R][mask_pitch] inside bits (unless rows are too long for them:
+// LbConst::mask_staged) | header (int4: band flag, droplet, first row y0,
+// rows << 16 | plane z) | with several droplets the group's LbConst
 template <typename S>
 struct Stage {
     S *pop;
@@ -169,7 +170,7 @@ __device__ __forceinline__ void produce_populations(const LbConst &c, const S *s
 // two viscosities lane 23 the rows' inside bits.  Every lane announces the
 // bytes of its own copies with its arrival on the mbarrier (initialised for
 // 32) before issuing them.
-template <typename S, bool VARTAU>
+template <typename S, int VARTAU>
 __device__ __forceinline__ void produce_rest(const Arrays &a, const LbConst &c, int d, int y0, int z, int nr,
                                              unsigned char *sbase, uint64_t *bar, bool band)
 {
@@ -182,7 +183,7 @@ __device__ __forceinline__ void produce_rest(const Arrays &a, const LbConst &c, 
         mine = (uint32_t)(nr * P * sizeof(float));
     else if (lane == Q + 3 && a.ndrops > 1)
         mine = sizeof(LbConst);
-    else if (VARTAU && lane == Q + 4)
+    else if (VARTAU && lane == Q + 4 && c.mask_staged)
         mine = (uint32_t)(nr * c.mask_pitch);
     int4 *header = stage_header(sbase, a);
     if (lane == 0)
@@ -193,7 +194,7 @@ __device__ __forceinline__ void produce_rest(const Arrays &a, const LbConst &c, 
         bulk_g2s(stg.F + (int64_t)k * R * P, a.F + k * a.total_pcells + c.pcell0 + (int64_t)P * row0, mine, bar);
     } else if (lane == Q + 3 && a.ndrops > 1) {
         bulk_g2s(header + 1, a.lbc + d, sizeof(LbConst), bar);
-    } else if (VARTAU && lane == Q + 4 && c.mask_pitch) {
+    } else if (VARTAU && lane == Q + 4 && c.mask_staged) {
         bulk_g2s(stg.mask, a.mask + c.mask0 + c.mask_pitch * row0, mine, bar);
     }
 }
@@ -222,7 +223,24 @@ __device__ __forceinline__ bool in_band_tile(const Arrays &a, const LbConst &c, 
 // below the half added)
 __device__ __forceinline__ int item_row(int e, float inv_npr) { return (int)(((float)e + 0.5f) * inv_npr); }
 
-template <typename S, bool VARTAU, bool FORCE>
+// VARTAU of the kernel and its parts: 0 one viscosity in every droplet, 1 two,
+// 2 two and some droplet's inside bits are not in the stages (16-bit rows of
+// 2313 to 2320 cells; with FP32 storage every row that fits two stages fits
+// with its bits).  Asked at run time alone, that cost 0.4 % of a step with two
+// viscosities (256^2 x 128 BF16).
+
+// the inside bits of the 32 cells about cell (x, y) of plane z, row r of the group
+template <int VARTAU, typename S>
+__device__ __forceinline__ uint32_t inside_word(const Arrays &a, const LbConst &c, const Stage<S> &stg, int r, int x, int y,
+                                                int z)
+{
+    const int at = (x >> 5) * 4;
+    if (VARTAU == 1 || c.mask_staged)
+        return *reinterpret_cast<const uint32_t *>(stg.mask + r * c.mask_pitch + at);
+    return *reinterpret_cast<const uint32_t *>(a.mask + c.mask0 + c.mask_pitch * ((int64_t)c.ny * z + y) + at);
+}
+
+template <typename S, int VARTAU, bool FORCE>
 __device__ __forceinline__ void collide_group(const Arrays &a, const LbConst &c, const Stage<S> &stg, int y0, int z,
                                               int nr, bool band, S *__restrict__ dst, uint32_t gen)
 {
@@ -268,7 +286,7 @@ __device__ __forceinline__ void collide_group(const Arrays &a, const LbConst &c,
         }
         float omega = omega_out;
         if (VARTAU && c.mask_pitch) {
-            const uint32_t m = *reinterpret_cast<const uint32_t *>(stg.mask + r * c.mask_pitch + (x >> 5) * 4);
+            const uint32_t m = inside_word<VARTAU>(a, c, stg, r, x, y, z);
             if ((m >> (x & 31)) & 1u)
                 omega = omega_in;
         }
@@ -443,7 +461,7 @@ __device__ __forceinline__ void bgk_guo_cell(const float (&s)[Q], float Fx, floa
 // divide evenly among the consumer threads, the threads that take one pair
 // more change from group to group (a rotation by kk times the remainder),
 // so that no warp is always the last to release a stage.
-template <typename S, bool VARTAU, bool FORCE>
+template <typename S, int VARTAU, bool FORCE>
 __device__ __forceinline__ void collide_pairs(const Arrays &a, const LbConst &c, const Stage<S> &stg, int y0, int z,
                                               int nr, bool band, S *__restrict__ dst, int kk, uint32_t gen)
 {
@@ -504,7 +522,7 @@ __device__ __forceinline__ void collide_pairs(const Arrays &a, const LbConst &c,
         const bool ub = FORCE && band && hasA && in_band_tile(a, c, x, y, z, gen);   // both cells share the tile
         float omegaA = c.omega_out, omegaB = c.omega_out;
         if (VARTAU && c.mask_pitch) {      // x is even: both cells' bits in one word
-            const uint32_t m = *reinterpret_cast<const uint32_t *>(stg.mask + r * c.mask_pitch + (x >> 5) * 4) >> (x & 31);
+            const uint32_t m = inside_word<VARTAU>(a, c, stg, r, x, y, z) >> (x & 31);
             omegaA = (m & 1u) ? c.omega_in : omegaA;
             omegaB = (m & 2u) ? c.omega_in : omegaB;
         }
@@ -577,7 +595,7 @@ __device__ __forceinline__ void collide_pairs(const Arrays &a, const LbConst &c,
     }
 }
 
-template <typename S, bool VARTAU, bool TR>
+template <typename S, int VARTAU, bool TR>
 __global__ void __launch_bounds__(lb_block<S>(), 2)
     lb_kernel(Arrays a, const S *__restrict__ src, S *__restrict__ dst, int ns, const int *__restrict__ list,
               const int *__restrict__ count, int no_force, int early, unsigned long long *tr)
@@ -713,8 +731,12 @@ cudaError_t launch_t(const Arrays &a, const void *src, void *dst, bool vartau, c
     const int ns = cfg.lb_stages < 2 ? 2 : (cfg.lb_stages > LB_MAX_STAGES ? LB_MAX_STAGES : cfg.lb_stages);
     const size_t smem = (size_t)ns * a.lb_stage_bytes;
     const bool traced = g_trace_lb != nullptr;
-    const void *fn = vartau ? (traced ? (const void *)lb_kernel<S, true, true> : (const void *)lb_kernel<S, true, false>)
-                            : (traced ? (const void *)lb_kernel<S, false, true> : (const void *)lb_kernel<S, false, false>);
+    auto *fn = traced ? lb_kernel<S, 0, true> : lb_kernel<S, 0, false>;
+    if (vartau)
+        fn = traced ? lb_kernel<S, 1, true> : lb_kernel<S, 1, false>;
+    if constexpr (sizeof(S) == 2)
+        if (vartau && a.mask_unstaged)
+            fn = traced ? lb_kernel<S, 2, true> : lb_kernel<S, 2, false>;
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess)
         return e;
@@ -730,17 +752,8 @@ cudaError_t launch_t(const Arrays &a, const void *src, void *dst, bool vartau, c
     int grid = cfg.sm_count * per_sm;
     grid = grid < total ? grid : total;
     const int nf = no_force ? 1 : 0, ea = early && !list ? 1 : 0;
-    unsigned long long *tr = g_trace_lb;
-    const dim3 g(grid), b(lb_block<S>());
-    if (vartau)
-        return traced ? launch_k(lb_kernel<S, true, true>, g, b, smem, s, a.pdl != 0, a, (const S *)src, (S *)dst, ns,
-                                 list, count, nf, ea, tr)
-                      : launch_k(lb_kernel<S, true, false>, g, b, smem, s, a.pdl != 0, a, (const S *)src, (S *)dst, ns,
-                                 list, count, nf, ea, tr);
-    return traced ? launch_k(lb_kernel<S, false, true>, g, b, smem, s, a.pdl != 0, a, (const S *)src, (S *)dst, ns, list,
-                             count, nf, ea, tr)
-                  : launch_k(lb_kernel<S, false, false>, g, b, smem, s, a.pdl != 0, a, (const S *)src, (S *)dst, ns,
-                             list, count, nf, ea, tr);
+    return launch_k(fn, dim3(grid), dim3(lb_block<S>()), smem, s, a.pdl != 0, a, (const S *)src, (S *)dst, ns, list, count,
+                    nf, ea, g_trace_lb);
 }
 
 }  // namespace
@@ -755,7 +768,8 @@ int lb_stage_bytes(int rows, int pitch, int sb, bool several, int mask_pitch)
 {
     const size_t b = (size_t)rows * Q * pitch * sb + (size_t)rows * 3 * pitch * sizeof(float) +
                      (size_t)rows * mask_pitch + sizeof(int4) + (several ? sizeof(LbConst) : 0);
-    return (int)((b + 127) & ~(size_t)127);
+    const size_t r = (b + 127) & ~(size_t)127;
+    return (int)(2 * r > LB_SMEM_LAUNCH ? b : r);
 }
 
 cudaError_t launch_lb(const Arrays &a, int storage, const void *src, void *dst, bool vartau,
