@@ -186,7 +186,7 @@ typedef struct {
                                  (whole rows: max(1, round(cells / nx)) rows, at most ny),
                                  in place of IBLB_OPT_LB_ROW_MULT (1..16384; 0 = use the
                                  multiplier; until either is set, chosen from the boxes'
-                                 sizes and the storage)                                  */
+                                 sizes, the storage and the stages asked for)            */
 #define IBLB_OPT_GRAPH_CHUNK 11 /* steps per replayed CUDA graph (1..64; default 1): with
                                  K > 1, iblb_step runs whole chunks of K steps as one
                                  captured graph each and the rest one step per graph,

@@ -93,8 +93,8 @@ struct iblb_ctx {
     double step_ms = 0.0;
     int64_t prof_steps = 0;
     int64_t step_count = 0;
-    LaunchCfg cfg{0, 2, 148, 3, 1, 0};
-    bool auto_cells = true, auto_stages = true;   // group size / pipeline depth by pick_shape
+    LaunchCfg cfg{0, 148, 3, 1};
+    LbRequest lb_ask{-1, 2, 0};    // group size and pipeline depth that the options ask for
     int *h_status = nullptr;     // pinned, 4 per droplet
     double *obs_scr = nullptr;   // scratch of the mesh observation kernels, every droplet's
     ObsMesh *d_obs = nullptr;    // the droplets' meshes for them (with the membranes)
@@ -352,91 +352,22 @@ void fill_drop_params(Drop &D, const iblb_lattice_desc &l, const iblb_physics_de
     D.ka = (float)p.area_modulus;
 }
 
-// shared memory a block of the stream-collide kernel may give its stages: the
-// opt-in maximum of sm_100 and later (227 KB) less 1 KB for its static part
-constexpr int64_t kLbSmemOptin = 227 * 1024 - 1024;
-
-// as many of the asked pipeline stages as fit the block's shared memory
-void fit_stages(iblb_ctx *c)
-{
-    while (c->cfg.lb_stages > 2 && (int64_t)c->cfg.lb_stages * c->A.lb_stage_bytes > kLbSmemOptin)
-        --c->cfg.lb_stages;
-}
-
-// bytes per row of a droplet's inside bits
-int mask_pitch(const Drop &D) { return D.vartau ? (D.nx + 127) / 128 * 16 : 0; }
-
-// rows per stream-collide group for about `cells` cells, of ny rows of pitch P
-int rows_for(int cells, const Drop &D) { return std::min(D.ny, std::max(1, (cells + D.nx / 2) / D.nx)); }
-
-// Group size and pipeline depth of the stream-collide kernel, unless they were
-// set: the pair with the least estimated time over the persistent blocks.
-// A group costs its cells plus a fixed part worth kGroupCells cells (its
-// hand-over and the latency of one pass; 128^3 in FP16, one block's time per
-// group at 256 .. 1024 cells), and half of an uneven last round is idle (the
-// blocks that still run get the others' bandwidth).  Two blocks an SM, as
-// registers allow, need their stages to fit half its shared memory; two
-// stages instead of three make larger groups fit, which pays when a block
-// has only a group or two.  Measured in the step (stream-collide, us, against
-// 768 cells, three stages and a short last group a plane): 32^3 FP32 6.1 ->
-// 4.6, 80^2 x 60 FP32 13.6 -> 9.8, 61 x 53 x 47 FP32 9.2 -> 7.3, 64 boxes of
-// 48 to 96 in FP16 491 -> 416, 32 boxes with tau_in != tau_out 232 -> 171.
-constexpr int kGroupCells = 160;
-constexpr int64_t kLbSmemSm = 228 * 1024, kLbSmemBlock = 1024 + 128;   // an SM's; reserved and static per block
-void pick_shape(iblb_ctx *c)
-{
-    const int sb = (int)storage_bytes(c->storage);
-    double best = 1e300;
-    const int ns_set = c->cfg.lb_stages, cells_set = c->cfg.lb_group_cells;
-    for (int ns = c->auto_stages ? 2 : ns_set; ns <= (c->auto_stages ? 3 : ns_set); ++ns)
-        for (int cells = 32; cells <= 1024; cells += 32) {
-            int64_t stage = 0, groups = 0;
-            double work = 0.0, largest = 0.0;
-            for (const Drop &D : c->drops) {
-                const int P = (D.nx * sb + 15) / 16 * 16 / sb, gpp = (D.ny - 1) / rows_for(cells, D) + 1;
-                const int rows = (D.ny - 1) / gpp + 1;
-                stage = std::max(stage, (int64_t)lb_stage_bytes(rows, P, sb, c->ndrops > 1, mask_pitch(D)));
-                groups += (int64_t)gpp * D.nzf;
-                work += (double)D.nzf * ((double)gpp * kGroupCells + (double)D.ny * P);
-                largest = std::max(largest, (double)rows * P + kGroupCells);
-            }
-            const int64_t fit = (kLbSmemSm / 2 >= ns * stage + kLbSmemBlock) ? 2 : 1;
-            if (ns * stage > kLbSmemOptin)
-                continue;
-            const double blocks = (double)c->cfg.sm_count * fit, rounds = groups / blocks;
-            double cost = work / blocks + 0.5 * (std::ceil(rounds) - rounds) * largest;
-            if (groups <= blocks)
-                cost = largest;
-            // one block an SM has half the warps: slower, except where FP32's
-            // traffic leaves them idle and there are rounds enough to fill in
-            if (fit == 1)
-                cost *= sb == 4 && rounds > 3.0 ? 0.5 : 0.6;
-            if (ns == 2 && rounds > 2.0)
-                cost *= 1.1;
-            if (cost < best) {
-                best = cost;
-                if (c->auto_cells)
-                    c->cfg.lb_group_cells = cells;
-                if (c->auto_stages)
-                    c->cfg.lb_stages = ns;
-            }
-        }
-    if (!c->auto_cells)
-        c->cfg.lb_group_cells = cells_set;
-    else if (best == 1e300)
-        c->cfg.lb_group_cells = 32;   // rows too long for two full stages: layout shortens the groups
-}
-
 // Offsets of cells, tiles, columns, launch blocks for the current launch shape.
 void layout(iblb_ctx *c)
 {
-    if (c->auto_cells)
-        pick_shape(c);
-    int64_t cell0 = 0, tile0 = 0, col0 = 0, pcell0 = 0, row0 = 0, trow0 = 0, mask0 = 0;
-    int mask_cols = 0;
-    int mb0 = 0, stage = 0;
     const int sb = (int)storage_bytes(c->storage);
     const bool several = c->ndrops > 1;
+    std::vector<LbBox> boxes;
+    for (auto &D : c->drops) {
+        // bytes per row of its inside bits
+        D.mask_pitch = D.vartau ? (D.nx + 127) / 128 * 16 : 0;
+        boxes.push_back({D.nx, D.ny, D.nzf, D.mask_pitch});
+    }
+    const LbShape shape = lb_shape(boxes, sb, c->cfg.sm_count, c->lb_ask);
+    c->cfg.lb_stages = shape.stages;
+    int64_t cell0 = 0, tile0 = 0, col0 = 0, pcell0 = 0, row0 = 0, trow0 = 0, mask0 = 0;
+    int mask_cols = 0;
+    int mb0 = 0;
     c->grp.clear();
     c->lbc.clear();
     c->A.mask_unstaged = 0;
@@ -448,26 +379,17 @@ void layout(iblb_ctx *c)
         D.col0 = col0;
         // rows padded to 16 bytes of population storage (and of the float
         // force / velocity rows, whose pitch is the same)
-        const int align = 16 / sb;
-        D.pitch = (D.nx + align - 1) / align * align;
+        D.pitch = lb_pitch(D.nx, sb);
         D.pcells = (int64_t)D.pitch * D.ny * D.nzf;
-        D.mask_pitch = mask_pitch(D);
         D.mask0 = mask0;
         D.mask_col0 = mask_cols;
         mask0 += (int64_t)D.mask_pitch * D.ny * D.nzf;
         mask_cols += D.mask_pitch / 4 * D.ny;
         D.pcell0 = pcell0;
         D.row0 = row0;
-        D.lb_rows = c->cfg.lb_group_cells > 0 ? rows_for(c->cfg.lb_group_cells, D)
-                                              : std::min(D.ny, c->cfg.lb_row_mult * lb_rows_per_group(D.nx));
-        // two stages of the group must fit the opt-in shared memory of a block
-        while (D.lb_rows > 1 &&
-               2 * (int64_t)lb_stage_bytes(D.lb_rows, D.pitch, sb, several, D.mask_pitch) > kLbSmemOptin)
-            --D.lb_rows;
-        // as many groups a plane, their rows as even as they go: a short last
-        // group would fall to the same blocks in every round
-        const int d = (int)c->lbc.size(), gpp = (D.ny - 1) / D.lb_rows + 1;
-        D.lb_rows = (D.ny - 1) / gpp + 1;
+        const int d = (int)c->lbc.size();
+        D.lb_rows = lb_group_rows(shape.cells, shape.mult, boxes[d], sb, several);
+        const int gpp = (D.ny - 1) / D.lb_rows + 1;
         for (int z = 0; z < D.nzf; ++z)
             for (int g = 0; g < gpp; ++g) {
                 const int y = (int)((int64_t)D.ny * g / gpp);
@@ -481,10 +403,7 @@ void layout(iblb_ctx *c)
         k.PC = (int)D.pcells;
         k.nzf = D.nzf;
         k.walls = D.walls;
-        // where two stages of one row fit without the inside bits only, they
-        // are read from global memory
-        k.mask_staged = D.mask_pitch &&
-                        2 * (size_t)lb_stage_bytes(D.lb_rows, D.pitch, sb, several, D.mask_pitch) <= LB_SMEM_LAUNCH;
+        k.mask_staged = lb_mask_staged(D.lb_rows, boxes[d], sb, several);
         k.npr = lb_items_per_row(D.pitch, sb);
         k.step_r = lb_consumers(sb) / k.npr;
         k.step_x = lb_consumers(sb) - k.step_r * k.npr;
@@ -507,8 +426,6 @@ void layout(iblb_ctx *c)
         D.mass_block0 = mb0;
         D.mass_nblocks = (int)((D.cells + MASS_CELLS_PER_BLOCK - 1) / MASS_CELLS_PER_BLOCK);
         c->A.mask_unstaged |= D.mask_pitch && !k.mask_staged;
-        stage = std::max(stage,
-                         lb_stage_bytes(D.lb_rows, D.pitch, sb, several, k.mask_staged ? D.mask_pitch : 0));
         cell0 += D.cells;
         pcell0 += D.pcells;
         row0 += (int64_t)D.ny * D.nzf;
@@ -526,9 +443,8 @@ void layout(iblb_ctx *c)
     c->A.total_mask_cols = mask_cols;
     c->mask_bytes = mask0;
     c->A.lb_blocks_total = (int)c->grp.size();
-    c->A.lb_stage_bytes = stage;
+    c->A.lb_stage_bytes = shape.stage_bytes;
     c->mass_blocks = mb0;
-    fit_stages(c);
 }
 
 int upload_drops(iblb_ctx *c)
@@ -819,6 +735,18 @@ int rebuild_membranes(iblb_ctx *c)
 int ensure_ready(iblb_ctx *c)
 {
     return rebuild_membranes(c);
+}
+
+// Lay the groups of the stream-collide kernel out anew for another request.
+int reshape(iblb_ctx *c, const LbRequest &ask)
+{
+    int r = ensure_ready(c);
+    if (r)
+        return r;
+    c->lb_ask = ask;
+    layout(c);
+    invalidate_graphs(c);
+    return upload_drops(c);
 }
 
 // One time step on c->stream with population buffers (src = fbuf[par]).
@@ -1688,29 +1616,19 @@ int iblb_set_option(iblb_ctx *c, int option, int value)
     case IBLB_OPT_LB_GROUP_CELLS: {
         if (value < 0 || value > 16384)
             return fail(c, IBLB_E_ARG, "cells per group must be in [0, 16384]");
-        int r = ensure_ready(c);
-        if (r)
-            return r;
-        c->auto_cells = false;
-        c->cfg.lb_group_cells = value;
-        layout(c);
-        invalidate_graphs(c);
-        return upload_drops(c);
+        LbRequest ask = c->lb_ask;
+        ask.cells = value;
+        return reshape(c, ask);
     }
     case IBLB_OPT_LB_ROW_MULT: {
         if (value == 0)
             value = 1;
         if (value < 1 || value > 4)
             return fail(c, IBLB_E_ARG, "row multiplier must be in [1, 4]");
-        int r = ensure_ready(c);
-        if (r)
-            return r;
-        c->cfg.lb_row_mult = value;
-        c->auto_cells = false;
-        c->cfg.lb_group_cells = 0;             // the multiplier takes over
-        layout(c);
-        invalidate_graphs(c);
-        return upload_drops(c);
+        LbRequest ask = c->lb_ask;
+        ask.mult = value;
+        ask.cells = 0;                         // the multiplier takes over
+        return reshape(c, ask);
     }
     case IBLB_OPT_FUSED_IB:
         c->fused_ib = value != 0;
@@ -1743,14 +1661,13 @@ int iblb_set_option(iblb_ctx *c, int option, int value)
         c->cfg.ib_blocks_per_sm = value;
         invalidate_graphs(c);
         return IBLB_OK;
-    case IBLB_OPT_LB_STAGES:
+    case IBLB_OPT_LB_STAGES: {
         if (value < 2 || value > 8)
             return fail(c, IBLB_E_ARG, "pipeline stages must be in [2, 8]");
-        c->auto_stages = false;
-        c->cfg.lb_stages = value;
-        fit_stages(c);
-        invalidate_graphs(c);
-        return IBLB_OK;
+        LbRequest ask = c->lb_ask;
+        ask.stages = value;
+        return reshape(c, ask);
+    }
     }
     return fail(c, IBLB_E_ARG, "unknown option");
 }
@@ -1815,7 +1732,8 @@ int iblb_autotune(iblb_ctx *c, const char *cache_path)
     // spare one: the current state is left untouched
     const int bpsm[2] = {0, 1};
     float best = 1e30f;
-    int bb = c->cfg.lb_blocks_per_sm, bm = c->cfg.lb_row_mult, bcells = c->cfg.lb_group_cells;
+    int bb = c->cfg.lb_blocks_per_sm;
+    LbRequest ask = c->lb_ask;     // the best so far
     int dev = 0, smem_max = 0;
     CK(cudaGetDevice(&dev));
     CK(cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
@@ -1832,16 +1750,14 @@ int iblb_autotune(iblb_ctx *c, const char *cache_path)
     CK(cudaEventCreate(&ev.e[1]));
     cudaEvent_t e0 = ev.e[0], e1 = ev.e[1];
     Entered entered_(c);
-    int bs = c->cfg.lb_stages;
-    c->auto_cells = c->auto_stages = false;
     // group sizes of 256 .. 1024 cells in steps of 128 (whole rows), with
     // every pipeline depth and both residencies whose stages fit
     for (int cells = 256; cells <= 1024; cells += 128)
         for (int bi = 0; bi < 2; ++bi)
             for (int ns = 2; ns <= 8; ++ns) {
                 c->cfg.lb_blocks_per_sm = bpsm[bi];
-                c->cfg.lb_group_cells = cells;
-                c->cfg.lb_stages = ns;
+                c->lb_ask.cells = cells;
+                c->lb_ask.stages = ns;
                 layout(c);
                 if (ns * (int64_t)c->A.lb_stage_bytes + 1024 > smem_max)
                     continue;                  // these stages do not fit
@@ -1860,22 +1776,16 @@ int iblb_autotune(iblb_ctx *c, const char *cache_path)
                 if (ms < best) {
                     best = ms;
                     bb = bpsm[bi];
-                    bcells = cells;
-                    bs = ns;
+                    ask = c->lb_ask;
                 }
             }
     c->cfg.lb_blocks_per_sm = bb;
-    c->cfg.lb_row_mult = bm;
-    c->cfg.lb_group_cells = bcells;
-    c->cfg.lb_stages = bs;
-    layout(c);
-    invalidate_graphs(c);
-    if ((r = upload_drops(c)))
+    if ((r = reshape(c, ask)))
         return r;
-    if (cache_path) {
+    if (cache_path && best < 1e30f) {
         FILE *fp = fopen(cache_path, "a");
         if (fp) {
-            fprintf(fp, "%s|%d %d %d %d\n", key, bb, bm, bs, bcells);
+            fprintf(fp, "%s|%d %d %d %d\n", key, bb, ask.mult, ask.stages, ask.cells);
             fclose(fp);
         }
     }

@@ -9,6 +9,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "lb_shape.h"
+
 namespace iblb {
 
 constexpr int Q = 19;
@@ -74,7 +76,7 @@ struct __align__(16) LbConst {
     int64_t tile0, trow0;
     int has_bf, mask_pitch, spare[2];
 };
-static_assert(sizeof(LbConst) == 128, "copied in one piece");
+static_assert(sizeof(LbConst) == LB_CONST_BYTES, "copied in one piece");
 
 // Record written per node by the force kernel and read by the spread and
 // the interpolation: base cell of the 4^3 support (fluid coordinates, x and
@@ -247,19 +249,10 @@ __host__ __device__ inline int floordiv(int a, int b) { return a >= 0 ? a / b : 
 // Host-side launchers (lb.cu, ib.cu, inout.cu, reduce.cu, fields.cu).
 struct LaunchCfg {
     int lb_blocks_per_sm;          // resident stream-collide blocks per SM (0: as many as fit)
-    int lb_row_mult;               // cell rows per group = lb_row_mult * lb_rows_per_group(nx)
     int sm_count;
     int lb_stages;                 // shared-memory stages of the stream-collide pipeline (2..8)
     int ib_blocks_per_sm;          // blocks per SM of the cooperative membrane kernels (0: all that fit)
-    int lb_group_cells = 0;        // if > 0: about this many cells per group (whole rows), in place of the multiplier
 };
-int lb_rows_per_group(int nx);     // 256-thread groups: max(1, 256 / nx) rows
-// bytes of one stage of the stream-collide kernel: 19 population rows and 3
-// force rows per cell row, its inside bits with two viscosities, the group's
-// header and with several droplets its droplet's constants (a multiple of 128
-// bytes; of 16, where two stages of such multiples do not fit a block)
-constexpr size_t LB_SMEM_LAUNCH = 227 * 1024 - 128;   // dynamic shared memory of a block, beside its barriers
-int lb_stage_bytes(int rows, int pitch, int storage_bytes, bool several, int mask_pitch);
 // work items per row and consumer threads per block, for LbConst
 int lb_items_per_row(int pitch, int storage_bytes);
 int lb_consumers(int storage_bytes);

@@ -42,7 +42,6 @@ unsigned long long *g_trace_lb = nullptr;   // host: stamp buffer of a traced st
 // a register spill, and the traced step would not time the plain kernel.
 __device__ __noinline__ void lb_trace_start(unsigned long long *tr) { trace_start(tr, TR_LB); }
 
-constexpr int LB_THREADS = 256;                   // consumer threads per block (FP32 storage)
 // 16-bit storage takes two cells per work item and needs more registers per
 // thread: 7 consumer warps (+ the producer) keep two blocks of 8 warps on an
 // SM at up to 128 registers, where two blocks of 9 warps allow 96
@@ -758,19 +757,9 @@ cudaError_t launch_t(const Arrays &a, const void *src, void *dst, bool vartau, c
 
 }  // namespace
 
-int lb_rows_per_group(int nx) { return nx >= LB_THREADS ? 1 : LB_THREADS / nx; }
-
 int lb_items_per_row(int pitch, int sb) { return sb == 2 ? pitch / 2 : pitch; }
 
 int lb_consumers(int sb) { return sb == 2 ? cons_threads<__half>() : cons_threads<float>(); }
-
-int lb_stage_bytes(int rows, int pitch, int sb, bool several, int mask_pitch)
-{
-    const size_t b = (size_t)rows * Q * pitch * sb + (size_t)rows * 3 * pitch * sizeof(float) +
-                     (size_t)rows * mask_pitch + sizeof(int4) + (several ? sizeof(LbConst) : 0);
-    const size_t r = (b + 127) & ~(size_t)127;
-    return (int)(2 * r > LB_SMEM_LAUNCH ? b : r);
-}
 
 cudaError_t launch_lb(const Arrays &a, int storage, const void *src, void *dst, bool vartau,
                       const LaunchCfg &cfg, cudaStream_t s, const int *list, const int *count, bool no_force,
