@@ -111,8 +111,8 @@ __device__ __forceinline__ void moments_half(const float (&v)[Q], double &r, dou
 
 // One block per MACRO_X cells of a row (no division per cell).  Measured with
 // the copy into kept host arrays, where the buffer was allocated and freed
-// for each call before: 128^3 FP16 1.43 -> 0.48 ms (0.36 of it the copy),
-// 80^2 x 60 FP32 0.39 -> 0.17 ms.
+// for each call before: 128^3 FP16 1.43 -> 0.66 ms (0.36 of it the copy),
+// 80^2 x 60 FP32 0.39 -> 0.20 ms.
 constexpr int MACRO_X = 128;
 template <typename S>
 __global__ void __launch_bounds__(MACRO_X) macros_kernel(Arrays a, int d, const S *f, double *rho, double *u)
@@ -148,9 +148,12 @@ __global__ void __launch_bounds__(MACRO_X) macros_kernel(Arrays a, int d, const 
             F[e] += a.F[e * a.total_pcells + D.pcell0 + cell];
     rho[c] = r;
     // post-collision momentum = sum c_i f_i + F (BGK keeps rho U, Guo adds (1-1/2tau) F)
-    const double inv = 1.0 / r;
+    // Divided, so that U is rounded once: products with 1 / rho are off by up to
+    // one and a half units, and brought back to the rounded quotients by their
+    // remainders cost more than the divisions (the call at 128^3 FP16: 0.47 ms
+    // products, 0.66 divisions, 0.72 corrected products).
     for (int e = 0; e < 3; ++e)
-        u[e * D.cells + c] = (j[e] - 0.5 * F[e]) * inv;
+        u[e * D.cells + c] = (j[e] - 0.5 * F[e]) / r;
 }
 
 __global__ void force_kernel(Arrays a, int d, double *F)
