@@ -109,20 +109,24 @@ __device__ __forceinline__ void moments_half(const float (&v)[Q], double &r, dou
         j[e] *= 1.0 / 16777216.0;
 }
 
-// One block per MACRO_X cells of a row (no division per cell).  Measured with
-// the copy into kept host arrays, where the buffer was allocated and freed
-// for each call before: 128^3 FP16 1.43 -> 0.66 ms (0.36 of it the copy),
-// 80^2 x 60 FP32 0.39 -> 0.20 ms.
-constexpr int MACRO_X = 128;
+// A thread per cell, consecutive ones whatever the row's length: FP64 bounds the
+// kernel, and an FP64 instruction costs a warp the same with 8 cells as with 32;
+// the two integer divisions that find the row cost next to nothing.  Measured
+// (ms, with the copy into kept host arrays), as it was with a buffer allocated
+// for each call -> a block per 128 cells of a row -> this: 8 x 64 x 4000 FP32 1.38
+// -> 2.32 -> 0.86, 24 x 100 x 900 BF16 1.44 -> 1.08 -> 0.90, 80^2 x 60 FP32 0.38 ->
+// 0.20 -> 0.19, 128^3 FP16 1.40 -> 0.66 -> 0.66 (0.36 of it the copy).
+constexpr int MACRO_THREADS = 128;
 template <typename S>
-__global__ void __launch_bounds__(MACRO_X) macros_kernel(Arrays a, int d, const S *f, double *rho, double *u)
+__global__ void __launch_bounds__(MACRO_THREADS) macros_kernel(Arrays a, int d, const S *f, double *rho, double *u)
 {
     const Drop &D = a.drops[d];
-    const int chunks = (D.nx + MACRO_X - 1) / MACRO_X, row = blockIdx.x / chunks;
-    const int x = (blockIdx.x - row * chunks) * MACRO_X + threadIdx.x, z = row / D.ny, y = row - z * D.ny;
-    if (x >= D.nx)
+    const uint32_t c = blockIdx.x * MACRO_THREADS + threadIdx.x;      // (below 2^30 cells)
+    if (c >= D.cells)
         return;
-    const int64_t cell = x + (int64_t)D.pitch * row, c = x + (int64_t)D.nx * row;
+    const uint32_t r0 = c / (uint32_t)D.nx;
+    const int x = (int)(c - r0 * (uint32_t)D.nx), row = (int)r0, z = row / D.ny, y = row - z * D.ny;
+    const int64_t cell = x + (int64_t)D.pitch * row;
     const S *p = f + (int64_t)Q * D.pcell0 + cell;
     double r = D.rho0, j[3];
     float v[Q], most = 0.0f;
@@ -228,11 +232,11 @@ cudaError_t launch_init_populations(const Arrays &a, int storage, void *f, cudaS
 cudaError_t launch_export_macros(const Arrays &a, const Drop &D, int d, int storage, const void *f, double *rho,
                                  double *u, cudaStream_t s)
 {
-    const unsigned g = (unsigned)((D.nx + MACRO_X - 1) / MACRO_X * D.ny * D.nzf);
+    const unsigned g = blocks_for(D.cells, MACRO_THREADS);
     switch (storage) {
-    case 0: macros_kernel<float><<<g, MACRO_X, 0, s>>>(a, d, (const float *)f, rho, u); break;
-    case 1: macros_kernel<__half><<<g, MACRO_X, 0, s>>>(a, d, (const __half *)f, rho, u); break;
-    case 2: macros_kernel<__nv_bfloat16><<<g, MACRO_X, 0, s>>>(a, d, (const __nv_bfloat16 *)f, rho, u); break;
+    case 0: macros_kernel<float><<<g, MACRO_THREADS, 0, s>>>(a, d, (const float *)f, rho, u); break;
+    case 1: macros_kernel<__half><<<g, MACRO_THREADS, 0, s>>>(a, d, (const __half *)f, rho, u); break;
+    case 2: macros_kernel<__nv_bfloat16><<<g, MACRO_THREADS, 0, s>>>(a, d, (const __nv_bfloat16 *)f, rho, u); break;
     default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
