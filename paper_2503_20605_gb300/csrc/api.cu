@@ -174,6 +174,34 @@ struct Entered {
     Entered &operator=(const Entered &) = delete;
 };
 
+// Work on the side stream, forked from the context's and joined again on
+// every way out of the scope, early error returns included: what it reads and
+// writes is the next call's too.
+struct SideWork {
+    iblb_ctx *c;
+    bool open = false;
+    explicit SideWork(iblb_ctx *ctx) : c(ctx) {}
+    SideWork(const SideWork &) = delete;
+    SideWork &operator=(const SideWork &) = delete;
+    cudaError_t fork()
+    {
+        cudaError_t e = cudaEventRecord(c->ev_fork, c->stream);
+        if (e == cudaSuccess)
+            e = cudaStreamWaitEvent(c->side, c->ev_fork, 0);
+        open = e == cudaSuccess;
+        return e;
+    }
+    cudaError_t join()
+    {
+        if (!open)
+            return cudaSuccess;
+        open = false;
+        const cudaError_t e = cudaEventRecord(c->ev_join, c->side);
+        return e == cudaSuccess ? cudaStreamWaitEvent(c->stream, c->ev_join, 0) : e;
+    }
+    ~SideWork() { join(); }
+};
+
 void invalidate_graphs(iblb_ctx *c)
 {
     for (int p = 0; p < 2; ++p) {
@@ -775,17 +803,16 @@ int enqueue_step(iblb_ctx *c, int par, bool forces_only)
     // membrane kernels (the in/out test goes first: the far groups inside a
     // droplet need it, and the node positions are final)
     const bool split = nodes && c->split_lb && !forces_only;
+    SideWork side(c);
     if (split) {
         CK(launch_classify(a, s));
         if (c->any_vartau) {
             CK(launch_corrected_positions(a, s));     // the force kernel has not written them yet
             CK(launch_inout(a, s));
         }
-        CK(cudaEventRecord(c->ev_fork, s));
-        CK(cudaStreamWaitEvent(c->side, c->ev_fork, 0));
+        CK(side.fork());
         CK(launch_lb(a, c->storage, c->fbuf[par], c->fbuf[par ^ 1], c->any_vartau, c->cfg, c->side,
                      a.grp_list + a.total_rows, a.grp_cnt + 1, true, c->lb_far_blocks_per_sm));
-        CK(cudaEventRecord(c->ev_join, c->side));
     }
     // (one kernel per stage: the spread's blocks take the crossings too)
     const bool faces_in_spread = c->any_vartau && !split && !c->fused_ib;
@@ -822,8 +849,7 @@ int enqueue_step(iblb_ctx *c, int par, bool forces_only)
         if (nodes && c->any_volcorr)
             CK(launch_volume_correction(a, c->n_red_chunks, s));
     }
-    if (split)
-        CK(cudaStreamWaitEvent(s, c->ev_join, 0));
+    CK(side.join());
     CK(mark(6));
     return IBLB_OK;
 }
@@ -1518,23 +1544,15 @@ int observe_range(iblb_ctx *c, int k, int n, double zcut_frac, double eps_flat, 
         blocks += c->drops[d].mass_nblocks;
         chunks = std::max(chunks, c->A.total_nodes ? c->obs[d].nc : 0);
     }
-    CK(cudaEventRecord(c->ev_fork, c->stream));
-    CK(cudaStreamWaitEvent(c->side, c->ev_fork, 0));
+    SideWork side(c);
+    CK(side.fork());
     CK(launch_mass(c->A, c->storage, c->fbuf[c->cur], c->d_mass, c->drops[k].mass_block0, blocks, k, n, c->side));
-    CK(cudaEventRecord(c->ev_join, c->side));
-    int r = IBLB_OK;
     const ObsMesh none{}, *table = c->A.total_nodes ? c->d_obs + k : nullptr;
-    auto enqueue = [&]() -> int {
-        if (chunks) {
-            CK(launch_corrected_positions(c->A, c->stream));
-            CK(enqueue_observe(table, nullptr, n, chunks, zcut_frac, eps_flat, c->stream));
-        }
-        return IBLB_OK;
-    };
-    r = enqueue();
-    CK(cudaStreamWaitEvent(c->stream, c->ev_join, 0));   // on every way out: the side stream's work is joined
-    if (r)
-        return r;
+    if (chunks) {
+        CK(launch_corrected_positions(c->A, c->stream));
+        CK(enqueue_observe(table, nullptr, n, chunks, zcut_frac, eps_flat, c->stream));
+    }
+    CK(side.join());
     CK(enqueue_observe_result(table, table ? nullptr : &none, n, c->d_mass, c->A.status, k, c->h_obs, c->stream));
     CK(cudaStreamSynchronize(c->stream));
     for (int i = 0; i < n; ++i) {
