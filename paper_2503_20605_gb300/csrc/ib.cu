@@ -1176,7 +1176,11 @@ __global__ void __launch_bounds__(SP_THREADS, SP_PER_SM) spread_kernel(Arrays a,
     // (the stream-collide kernel then requests its first populations while the
     // last tiles are summed).  Every block of this launch is resident when the
     // last one says so.  Measured (step, us): 32^3 17.3 -> 16.5, 128^3 FP16 53.6
-    // -> 52.1, 163 842 nodes 289 -> 286; but 64 boxes 647 -> 666, so not there.
+    // -> 52.1, 163 842 nodes 289 -> 286.  With several it goes both ways: 2, 8 and
+    // 32 equal boxes of 72 x 72 x 56 in FP16 gain (47.8 -> 45.1, 117.2 -> 114.1,
+    // 408 -> 406), 64 of sides 48 to 96 lose 2.6 %, and with two viscosities
+    // nothing changes (the inside bits' kernel comes next: 32 boxes 443 -> 442).  So
+    // not there; what tells the two apart is not known, the number is not it.
     if (a.ndrops == 1)
         launch_dependents();
     __shared__ SpreadSmem sm;

@@ -44,7 +44,7 @@ struct Drop {
     int64_t col0;                  // first column (nx*ny per droplet)
     int64_t mask0;                 // inside bits: first byte; row (y, z) at mask0 + mask_pitch (y + ny z)
     int mask_pitch, mask_col0;     // bytes per row (a multiple of 16; 0: one viscosity), first word column
-    int pitch;                     // population row pitch: nx rounded up to 16 elements
+    int pitch;                     // population row pitch: nx rounded up to 16 bytes of storage (lb_pitch)
     int64_t pcell0, pcells;        // population planes: first padded cell, pitch*ny*nzf
     int64_t row0;                  // first row (y + ny z) in the pooled row arrays
     int node0, nnodes, tri0, ntri;

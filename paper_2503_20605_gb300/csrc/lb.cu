@@ -4,8 +4,10 @@
 // offsets s_i = f_i - w_i rho0 in FP32, FP16 or BF16, arithmetic in FP32.
 //
 // Data movement.  Populations and the force / velocity fields live in rows
-// (y, z) of pitch P (nx rounded up to 16 elements), so every row starts on a
-// 32-byte boundary.  A group is R consecutive cell rows of one droplet.  In
+// (y, z) of pitch P (nx rounded up so that a row of populations is a multiple
+// of 16 bytes, which the bulk copies need; a 32-byte sector at a row's end may
+// be shared with the next row).  A group is R consecutive cell rows of one
+// droplet.  In
 // the pull scheme population i of row (y, z) comes entirely from row
 // (y - c_iy, z - c_iz) (or, at a wall, from row (y, z) of the opposite
 // population), so one producer warp per block fetches the 19 R source rows of
@@ -20,10 +22,10 @@
 // The producer refills a stage as soon as it is empty, so up to ns groups
 // are in flight, and no consumer warp waits for the others.
 //
-// Rows are written whole, padding included (as zeros): a 32-byte sector that
-// stays partly written costs a read of the rest when it leaves L2.  Twenty
-// 85^3 boxes in FP16 (pitch 88) ran at 3.4 TB/s without the padding's stores,
-// as against 5.3 TB/s for 88^3.
+// Rows are written whole, padding included (as zeros), so that a group's rows
+// leave no gap in a plane: a 32-byte sector that stays partly written costs a
+// read of the rest when it leaves L2.  Twenty 85^3 boxes in FP16 (pitch 88) ran
+// at 3.4 TB/s without the padding's stores, as against 5.3 TB/s for 88^3.
 //
 // Memory traffic per fluid cell: 19 reads + 19 writes of the storage type
 // (152 B for FP32, 76 B for 16-bit storage); the force density is read and
@@ -254,7 +256,7 @@ __device__ __forceinline__ void collide_group(const Arrays &a, const LbConst &c,
     const int RP = R * P;
     S *outb = dst + (int64_t)Q * pcell0 + (int64_t)P * ny * z;
     float4 *U = a.U;
-    // cell e = r * nx + x of the group, walked without divisions
+    // cell e = r * P + x of the group (padding included), walked without divisions
     const int step_r = c.step_r, step_x = c.step_x;
     int r = item_row(threadIdx.x, c.inv_npr), x = threadIdx.x - r * P;
     for (; r < nr; r += step_r, x += step_x) {

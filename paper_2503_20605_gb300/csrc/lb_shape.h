@@ -89,6 +89,17 @@ inline bool lb_mask_staged(int rows, const LbBox &b, int sb, bool several)
 // 768 cells, three stages and a short last group a plane): 32^3 FP32 6.1 ->
 // 4.6, 80^2 x 60 FP32 13.6 -> 9.8, 61 x 53 x 47 FP32 9.2 -> 7.3, 64 boxes of
 // 48 to 96 in FP16 491 -> 416, 32 boxes with tau_in != tau_out 232 -> 171.
+// The factors below are fitted, not derived.  The chosen shape against the best
+// of 64 .. 1024 cells with two and three stages (a step without membranes, us):
+// 32^3 FP32 3.88 / 3.88, 61 x 53 x 47 FP32 5.78 / 5.78, 80^2 x 60 FP32 7.95 /
+// 7.95, 128^3 FP16 28.0 / 27.5, 256^2 x 128 BF16 101.1 / 101.0, 64 boxes FP16
+// 301.7 / 301.7; but 8 boxes FP32 58.3 / 54.9, 128^3 FP32 54.8 / 50.0, 256^2 x
+// 128 FP32 210 / 188: there two blocks an SM with groups of 256 cells, or one
+// with twice that, are better than the larger groups that the 0.5 favours.
+// One block an SM against two of the same group (us): 128^3 FP16 896 cells 32.4
+// (three stages, one) / 29.5 (two stages, two), 80^2 x 60 FP32 512 cells 11.9 /
+// 9.3; three stages against two, two blocks each: 128^3 FP16 640 cells 28.0 /
+// 32.3, 64 boxes 640 cells 301.9 / 336.0, below two rounds no difference.
 constexpr int LB_GROUP_CELLS = 160;
 inline LbShape lb_shape(const std::vector<LbBox> &boxes, int sb, int sms, const LbRequest &ask)
 {
